@@ -245,7 +245,8 @@ typedef enum {
   FAS_K_RESTRICT = 2,    /* restriction of u and r                                              */
   FAS_K_TAU = 3,         /* coarse source term f_c = R(r) + A_c R(u)                             */
   FAS_K_PROLONG = 4,     /* prolongation of the correction (+ post-smoothing when fused)         */
-  FAS_K_COARSE = 5,      /* single-CTA V-cycle over the small levels                             */
+  FAS_K_COARSE = 5,      /* the small levels: the single-block V-cycle, and tile-kernel launches on
+                          * levels of at most 128 x 128 cells below the finest                  */
   FAS_K_IR = 6,          /* mixed precision: float64 residual r = b - A u, rounded to float32    */
   FAS_K_NORM = 7,        /* norms and means                                                     */
   FAS_K_OTHER = 8,       /* right-hand sides, fills, conversions                                */

@@ -10,6 +10,7 @@
 
 #include "bits64.cuh"
 #include "common.cuh"
+#include "solve_state.cuh"
 
 namespace fasmg {
 
@@ -363,21 +364,12 @@ __global__ void k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
     smooth_colour4_body<T, DIM, false>(u, f, L, colour);
 }
 
-// r (nullable) = f - A u; per-block partial of sum (s r)^2 into partials[blockIdx.x], s = *nsp (or 1).
+// r (nullable) = f - A u, and the norm of the residual (scaled by s = *E.nsp before squaring).
 template <typename T, int DIM>
-__global__ void k_residual(T* r, const T* u, const T* f, LevelDesc<T> L, const float* nsp, double* partials) {
-  const float acc = L.per ? residual_range<T, DIM, true>(r, u, f, L, nsp ? *nsp : 1.f, gtid(), gstride())
-                          : residual_range<T, DIM, false>(r, u, f, L, nsp ? *nsp : 1.f, gtid(), gstride());
-  const double s = block_sum((double)acc);
-  if (threadIdx.x == 0 && partials) partials[blockIdx.x] = s;
-}
-
-// out[0] = sqrt(sum of partials) / s (s = *nsp, or 1), summed in a fixed order by one block.
-static __global__ void k_finish_norm(const double* partials, int nblocks, double* out, const float* nsp) {
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[b];
-  v = block_sum(v);
-  if (threadIdx.x == 0) out[0] = sqrt(v) / (nsp ? (double)*nsp : 1.0);
+__global__ void k_residual(T* r, const T* u, const T* f, LevelDesc<T> L, const __grid_constant__ NormEnd E) {
+  const float acc = L.per ? residual_range<T, DIM, true>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride())
+                          : residual_range<T, DIM, false>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride());
+  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
 // out[0] = sum of partials (no square root), used for means.
@@ -432,9 +424,9 @@ __global__ void k_sub_mean(T* x, const T* y, int64_t n, const double* sum) {
   for (int64_t i = gtid(); i < n; i += gstride()) x[i] = y[i] - m;
 }
 
-// heat step right-hand side: b = u + dt * fsrc (fsrc may be null: b = u), with the per-block partial
-// sums of b^2 (float squares) for ||b||
-static __global__ void k_heat_rhs(double* b, const double* u, const double* fsrc, double dt, int64_t n, double* partials) {
+// heat step right-hand side: b = u + dt * fsrc (fsrc may be null: b = u), and ||b|| (float squares)
+static __global__ void k_heat_rhs(double* b, const double* u, const double* fsrc, double dt, int64_t n,
+                                  const __grid_constant__ NormEnd E) {
   float acc = 0.f;
   for (int64_t i = gtid(); i < n; i += gstride()) {
     const double v = fsrc ? fma(dt, fsrc[i], u[i]) : u[i];
@@ -442,8 +434,7 @@ static __global__ void k_heat_rhs(double* b, const double* u, const double* fsrc
     const float vf = f64_to_f32_rn_bits(v);
     acc = fmaf(vf, vf, acc);
   }
-  const double s = block_sum((double)acc);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
 // ---- mixed precision (iterative refinement): u += e, and r32 = (float)(b - A u) with its norm
@@ -489,14 +480,14 @@ __device__ __forceinline__ unsigned nb_bits(const double* __restrict__ u, int64_
   return mask;
 }
 
-// r32 = (float)(b - A u) and the per-block partial of sum (nscale r32)^2. With constant kappa the
+// r32 = (float)(b - A u) and its norm. With constant kappa the
 // point equation is evaluated as fma(c, S, fma(-alpha, u, b)) with S = sum_nb u_nb - M u exact
 // (bits64.cuh); cells where that does not apply take the float64 point equation.
 template <int DIM>
-__global__ void k_ir_residual(float* r32, const double* u, const double* b, LevelDesc<double> L, const float* nsp,
-                              double* partials) {
+__global__ void k_ir_residual(float* r32, const double* u, const double* b, LevelDesc<double> L,
+                              const __grid_constant__ NormEnd E) {
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
-  const float nscale = nsp ? *nsp : 1.f;
+  const float nscale = E.nsp ? *E.nsp : 1.f;
   float acc = 0.f;
   for (int64_t idx = gtid(); idx < n; idx += gstride()) {
     const int i = (int)(idx & (L.nx - 1));
@@ -525,22 +516,20 @@ __global__ void k_ir_residual(float* r32, const double* u, const double* b, Leve
     const float rs = rv * nscale;
     acc = fmaf(rs, rs, acc);
   }
-  const double s = block_sum((double)acc);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
-// per-block partial of sum (nscale x)^2, squares of the float-rounded values (norms for stopping
+// ||x||, squares of the float-rounded values (norms for stopping
 // tests need a few digits only, and the conversion keeps the work off the FP64 pipe)
 template <typename T>
-__global__ void k_norm2(const T* x, int64_t n, const float* nsp, double* partials) {
-  const float nscale = nsp ? *nsp : 1.f;
+__global__ void k_norm2(const T* x, int64_t n, const __grid_constant__ NormEnd E) {
+  const float nscale = E.nsp ? *E.nsp : 1.f;
   float acc = 0.f;
   for (int64_t i = gtid(); i < n; i += gstride()) {
     const float v = (float)x[i] * nscale;
     acc = fmaf(v, v, acc);
   }
-  const double s = block_sum((double)acc);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
 template <typename T>
@@ -955,67 +944,6 @@ __global__ void k_kappa_grad(double* g, const double* u, const double* mu, int n
 // y += a x
 static __global__ void k_axpy(double* y, double a, const double* x, int64_t n) {
   for (int64_t i = gtid(); i < n; i += gstride()) y[i] = fma(a, x[i], y[i]);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Device-side state of one solve (Algorithm 1's outer loop): the stopping decision is taken on the
-// device, so that the same kernels serve a host-driven loop and a graph with a conditional node.
-// ------------------------------------------------------------------------------------------------
-struct SolveState {
-  double fn;      // ||f||_2
-  double res0;    // ||f - A u||_2 before the first cycle
-  double res;     // after the last cycle
-  double ref;     // reference of the relative test (||f||, or res0 when f = 0), 1 in absolute mode
-  double w;       // 1 (relative test) or h^{d/2} (the paper's absolute h-weighted norm)
-  double tol;
-  float nscale;   // power of two applied to values before squaring them in float
-  int kmax;
-  int cycles;
-  int converged;
-  int nonfinite;
-  int cond;       // 1: run another cycle
-};
-
-// After ||f|| is known: the norm scale (a power of two bringing the rms of f near 1).
-static __global__ void k_solve_begin(SolveState* S, double tol, int kmax, double w, double ncells) {
-  const double fn = S->fn;
-  float s = 1.f;
-  if (fn > 0.0 && isfinite(fn)) {
-    const int e = (int)lrint(log2(fn / sqrt(ncells)));
-    s = (float)ldexp(1.0, -max(-120, min(120, e)));
-  }
-  S->nscale = s;
-  S->tol = tol;
-  S->kmax = kmax;
-  S->w = w;
-  S->cycles = 0;
-  S->converged = 0;
-  S->nonfinite = 0;
-  S->cond = 1;  // Algorithm 1 runs at least one cycle
-}
-
-// After the initial residual: the reference of the relative test.
-static __global__ void k_solve_ref(SolveState* S, int relative) {
-  S->ref = relative ? (S->fn > 0.0 ? S->fn : S->res0) : 1.0;
-}
-
-// After each cycle's residual norm (in S->res): count it and decide whether to continue. When
-// set_cond, also set the graph's conditional (the kernel then runs inside the while node's body).
-static __global__ void k_solve_step(SolveState* S, cudaGraphConditionalHandle h, int set_cond) {
-  S->cycles += 1;
-  const double res = S->w * S->res;
-  int cond = 1;
-  if (!isfinite(res)) {
-    S->nonfinite = 1;
-    cond = 0;
-  } else if (res <= S->tol * S->ref) {
-    S->converged = 1;
-    cond = 0;
-  } else if (S->cycles >= S->kmax) {
-    cond = 0;
-  }
-  S->cond = cond;
-  if (set_cond) cudaGraphSetConditional(h, (unsigned)cond);
 }
 
 }  // namespace fasmg

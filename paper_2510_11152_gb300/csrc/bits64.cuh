@@ -137,6 +137,24 @@ __device__ __forceinline__ bool f32_normal_range(double x) {
   return a - (897u << 20) < (254u << 20);
 }
 
+__device__ __forceinline__ int exp_field(double x) {
+  return (int)(((uint64_t)__double_as_longlong(x) >> 52) & 0x7FF);
+}
+
+// X in units of 2^(base - 1086), rounded to the nearest float64 (ties to even); the caller's base keeps the
+// result normal (base - 63 .. base are the exponent fields it may get, less one).
+__device__ __forceinline__ double f64_of_units(int64_t X, int base) {
+  const uint64_t sign = (uint64_t)X & (1ull << 63);
+  const uint64_t A = X < 0 ? (uint64_t)(-X) : (uint64_t)X;
+  const int z = __clzll((long long)A);
+  const uint64_t n = A << z;  // leading one at bit 63
+  const uint64_t q = (n >> 11) + ((((uint32_t)n & 0x7FFu) + 0x3FFu + ((uint32_t)(n >> 11) & 1u)) >> 11);
+  // q has its leading one at bit 52, which adds one to the exponent field; a carry out of the rounding
+  // lands there as well
+  const uint64_t r = ((uint64_t)(base - z) << 52) + q;
+  return __longlong_as_double((long long)(A == 0 ? 0ull : (sign | r)));
+}
+
 // Largest exponent spread handled exactly: significands < 2^58, at most 6 neighbours plus M <= 9
 // times the centre keep |S| < 2^62.
 constexpr int kMaxExpSpread = 5;

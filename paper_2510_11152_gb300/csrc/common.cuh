@@ -44,6 +44,7 @@ struct LevelDesc {
   const T* Dh;     // D / h^2
   T alpha;         // alpha of A u = alpha u - beta div(kappa grad u)
   T a[kClasses], b[kClasses], d[kClasses];
+  short alo[kClasses];         // a 2^64 beyond float64's a (block fixed point, tile2d.cu)
   unsigned char mt[kClasses];  // M of d = alpha + c M: neighbours plus boundary multiplicities
 };
 

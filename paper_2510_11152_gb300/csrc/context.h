@@ -7,6 +7,7 @@
 
 #include "../../include/fas.h"
 #include "common.cuh"
+#include "tile2d.h"
 
 namespace fasmg {
 
@@ -23,6 +24,11 @@ struct Hier {
   std::vector<T*> u, f, u0;
   std::vector<T*> u2, rc;  // fused path: second u buffer (ping-pong) and R(r) from the finer level
   int nfast = 0;           // levels 0..nfast-1 use the fused kernels
+  int ntile = 0;           // > 0: levels nfast..ntile-1 run the register-tile kernels and levels
+                           // ntile.. the single-block tile kernel; 0 with tiled: all run in that block
+  bool tiled = false;
+  std::vector<int> tile_bits;  // fixed-point bits of each tiled level (float64; 0: float64 arithmetic)
+  TileCoarse<T> tile_coarse;   // arguments of the single-block tile kernel
   SmemLayout smem;         // shared-memory layout of the single-CTA kernel (levels >= switch_level)
   size_t smem_bytes = 0;
   T** d_u = nullptr;

@@ -21,6 +21,7 @@
 #include "ir_strip.h"
 #include "stream2d.h"
 #include "stream3d.h"
+#include "tile2d.h"
 #include "tma.cuh"
 
 using namespace fasmg;
@@ -164,6 +165,18 @@ LevelDesc<T> make_desc(const fas_params& p, const LevelShape& s) {
     }
     const double D = p.alpha * h2 + bk * m;
     L.mt[cls] = (unsigned char)m;
+    {
+      // the rest of a = bk / D beyond its float64 value, with D = alpha h^2 + bk m carried to twice the
+      // precision: in fixed point alpha b + M a = 1 then holds to 2^-64, where a float64 a (or d) that is off
+      // by 2^-54 acts like a source of d 2^-54 u (4096 x 2048 heat run: solution error 3e-13)
+      const double p1 = p.alpha * h2, e1 = std::fma(p.alpha, h2, -p1), p2 = bk * m;  // m <= 9: bk m has an error too
+      const double e2 = std::fma(bk, m, -p2), Ds = p1 + p2, t = Ds - p1;
+      const double Dl = ((p1 - (Ds - t)) + (p2 - t)) + (e1 + e2);
+      const double q = Ds != 0.0 ? bk / Ds : 0.0;
+      const double rest = Ds != 0.0 ? (std::fma(-q, Ds, bk) - q * Dl) / Ds : 0.0;
+      const double lo = std::ldexp(rest + (q - (Ds != 0.0 ? bk / D : 0.0)), 64);
+      L.alo[cls] = std::fabs(lo) < 30000.0 ? (short)std::lrint(lo) : (short)0;
+    }
     L.a[cls] = (T)(D != 0.0 ? bk / D : 0.0);
     L.b[cls] = (T)(D != 0.0 ? h2 / D : 0.0);
     L.d[cls] = (T)(D / h2);
@@ -191,6 +204,8 @@ void free_hier(Hier<T>& H) {
   H.u2.clear();
   H.rc.clear();
   H.nfast = 0;
+  H.ntile = 0;
+  H.tiled = false;
   H.d_desc = nullptr;
   H.cinv = nullptr;
   H.allocated = false;
@@ -398,17 +413,29 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       }
       if (l > 0) STATUS_TRY(dev_alloc(H, &H.u0[l], n));
     }
+    // register-tile path: 2D cell levels of either precision whose coarsest levels fit the single-block
+    // tile kernel (at most 64 x 64 cells)
+    H.tiled = false;
+    H.ntile = 0;
+    if (p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL && p.nu1 >= 1 && p.nu1 <= kTileMaxNu &&
+        p.nu2 >= 1 && p.nu2 <= kTileMaxNu) {
+      int lc = 0;
+      while (lc < c->nlev && (c->shape[lc].nx > kTileCoarseCells || c->shape[lc].ny > kTileCoarseCells)) ++lc;
+      H.tiled = lc < c->nlev;
+      H.ntile = H.tiled ? lc : 0;
+    }
     // sweep-fused 2D path (float32 only): consecutive levels from the finest that the fused kernels
     // handle and that are larger than the single-CTA switch level
     H.nfast = 0;
     if (sizeof(T) == 4 && p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL &&
         p.ordering == FAS_ORDER_FORWARD && p.nu1 >= 1 && p.nu2 >= 1 && periodic_mask(p) == 0) {
       // below 2^20 cells a level's fused kernels are latency-bound (one warp streams a long segment of
-      // rows) and the per-operation kernels measured faster (8192^2 run: 127.8 -> 125.8 ms); the finest
-      // level stays fused for its float64 update
+      // rows) and the register-tile kernels take it; where those do not apply (narrow hierarchies) the
+      // finest level stays fused for its float64 update and the others run per operation
       while (H.nfast < H.switch_level &&
              stream2d_supported(c->shape[H.nfast].nx, c->shape[H.nfast].ny, std::max(p.nu1, p.nu2)) &&
-             (H.nfast == 0 || c->shape[H.nfast].cells() >= kFusedMinCells2D || p.path == 2))
+             ((H.nfast == 0 && !H.tiled) || c->shape[H.nfast].cells() >= kFusedMinCells2D || p.path == 2) &&
+             (!H.tiled || H.nfast < H.ntile))
         H.nfast++;
     }
     H.u2.assign(c->nlev, nullptr);
@@ -416,6 +443,40 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
     for (int l = 0; l < H.nfast; ++l) {
       STATUS_TRY(dev_alloc(H, &H.u2[l], c->shape[l].cells()));
       if (l + 1 < H.nfast) STATUS_TRY(dev_alloc(H, &H.rc[l + 1], c->shape[l + 1].cells()));
+    }
+    for (int l = H.nfast; l < H.ntile && H.tiled; ++l) {
+      // without room for the second buffers the levels run the per-operation kernels
+      if (dev_alloc(H, &H.u2[l], c->shape[l].cells()) != FAS_OK ||
+          (l > 0 && dev_alloc(H, &H.rc[l], c->shape[l].cells()) != FAS_OK)) {
+        cudaGetLastError();
+        H.tiled = false;
+        H.ntile = 0;
+      }
+    }
+    if (H.tiled) {
+      TileCoarse<T>& A = H.tile_coarse;
+      std::memset(&A, 0, sizeof(A));
+      H.tile_bits.assign(c->nlev, 0);
+      const int nuc = p.nu_coarse > 0 ? p.nu_coarse : p.nu1;
+      A.bits = 63;
+      for (int l = 0; l < c->nlev; ++l) {
+        if constexpr (std::is_same<T, double>::value) {
+          H.tile_bits[l] = tile_fixed_bits(H.desc[l], std::max(p.nu1, p.nu2));
+          const int bl = l == c->nlev - 1 && !p.coarse_exact ? tile_fixed_bits(H.desc[l], nuc) : H.tile_bits[l];
+          if (l >= H.ntile) A.bits = std::min(A.bits, std::min(H.tile_bits[l], bl));
+        }
+        if (l >= H.ntile) {
+          A.off[l] = A.total;
+          A.total += 2 * (int)((c->shape[l].cells() + 3) / 4 * 4);
+        }
+      }
+      A.l0 = H.ntile;
+      A.nlev = c->nlev;
+      A.nu1 = p.nu1;
+      A.nu2 = p.nu2;
+      A.nuc = nuc;
+      A.ordering = p.ordering;
+      A.tau = H.ntile > 0;
     }
     // sweep-fused 3D smoothing (float32): a second buffer on every level that the fused sweep handles
     // (its sweeps ping-pong between the two) and that is large enough for it to pay: measured at
@@ -445,6 +506,8 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
   }
   STATUS_TRY(dev_alloc(H, &H.d_desc, c->nlev));
   CUDA_TRY(cudaMemcpy(H.d_desc, H.desc.data(), c->nlev * sizeof(LevelDesc<T>), cudaMemcpyHostToDevice));
+  H.tile_coarse.desc = H.d_desc;
+  H.tile_coarse.cinv = H.cinv;
   return FAS_OK;
 }
 
@@ -531,18 +594,44 @@ void launch_smooth(fas_ctx* c, const LevelDesc<T>& L, int level, T* u, const T* 
   }
 }
 
-// ||f - A u||_2 into *out (device); r (nullable) receives the residual; nsp: device norm scale or null.
+// The end of a kernel that forms a norm on this context's stream (partials and counter are the
+// context's; norms of one context never overlap).
+NormEnd norm_to(fas_ctx* c, int use, const float* nsp, double* out = nullptr) {
+  NormEnd E{};
+  E.partials = c->partials;
+  E.ticket = c->ir_ticket + 1;
+  E.nsp = nsp;
+  E.out = out;
+  E.S = c->S;
+  E.use = use;
+  E.relative = c->p.tol_relative;
+  return E;
+}
+
+// ||f||: starts a solve of at most max_cycles cycles
+NormEnd norm_rhs(fas_ctx* c, int max_cycles) {
+  NormEnd E = norm_to(c, kNormRhs, nullptr);
+  E.tol = c->p.tol;
+  E.kmax = max_cycles;
+  E.w = c->p.tol_relative ? 1.0 : std::pow(c->shape[0].h, c->p.dim / 2.0);  // Eq. residual weight
+  E.ncells = (double)c->shape[0].cells();
+  return E;
+}
+
+// the residual after a cycle; h: the graph's conditional (set_cond)
+NormEnd norm_cycle(fas_ctx* c, cudaGraphConditionalHandle h, int set_cond) {
+  NormEnd E = norm_to(c, kNormCycle, &c->S->nscale);
+  E.cond = h;
+  E.set_cond = set_cond;
+  return E;
+}
+
+// r = f - A u (r nullable) and its norm
 template <typename T, int DIM>
-void launch_residual(fas_ctx* c, const LevelDesc<T>& L, int level, T* r, const T* u, const T* f, const float* nsp,
-                     double* out) {
+void launch_residual(fas_ctx* c, const LevelDesc<T>& L, int level, T* r, const T* u, const T* f, const NormEnd& E) {
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
-  const int g = grid_for(c, n);
-  {
-    Prof pr(c, FAS_K_RESIDUAL, level, (double)n);
-    k_residual<T, DIM><<<g, kBlock, 0, c->stream>>>(r, u, f, L, nsp, c->partials);
-  }
-  Prof pr(c, FAS_K_NORM, level, 0.0);
-  k_finish_norm<<<1, kBlock, 0, c->stream>>>(c->partials, g, out, nsp);
+  Prof pr(c, FAS_K_RESIDUAL, level, (double)n);
+  k_residual<T, DIM><<<grid_for(c, n), kBlock, 0, c->stream>>>(r, u, f, L, E);
 }
 
 template <typename T, int DIM>
@@ -566,6 +655,22 @@ fas_status launch_coarse(fas_ctx* c, Hier<T>& H, int l0, T* utop, const T* ftop)
     k_coarse_smem<T, DIM, decltype(tag)::value><<<1, kCoarseThreads, H.smem_bytes, c->stream>>>(A, H.smem, utop, ftop);
   });
   return FAS_OK;
+}
+
+// f += A u on level l (the tau correction; H.f[l] holds R(r), H.u[l] the restricted start).
+template <typename T, int DIM>
+void launch_tau(fas_ctx* c, Hier<T>& H, int l) {
+  const LevelDesc<T>& L = H.desc[l];
+  const int64_t n = (int64_t)L.nx * L.ny * L.nz;
+  Prof pr(c, FAS_K_TAU, l, (double)n);
+  if constexpr (std::is_same<T, float>::value && DIM == 3) {
+    // 3D float32 cell levels: 4 cells per thread (path 1: one per cell)
+    if (c->p.path != 1 && L.fax < 0 && !L.per && !L.varkappa && (L.nx & 3) == 0) {
+      k_tau4_3d<<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(H.f[l], H.u[l], L);
+      return;
+    }
+  }
+  k_tau<T, DIM><<<grid_for(c, n), kBlock, 0, c->stream>>>(H.f[l], H.u[l], L);
 }
 
 // Levels lfrom..switch-1 through the per-operation kernels around the single-CTA kernel (any value
@@ -598,18 +703,7 @@ fas_status vcycle_basic_from(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T
                                                                                  H.f[l + 1], u, f, L);
       });
     }
-    {
-      Prof pr(c, FAS_K_TAU, l + 1, (double)nc);
-      const LevelDesc<T>& Lc = H.desc[l + 1];
-      bool groups = false;  // 3D float32 cell levels: 4 cells per thread (path 1: one per cell)
-      if constexpr (std::is_same<T, float>::value && DIM == 3) {
-        if (c->p.path != 1 && Lc.fax < 0 && !Lc.per && !Lc.varkappa && (Lc.nx & 3) == 0) {
-          k_tau4_3d<<<grid_for(c, nc / 4), kBlock, 0, c->stream>>>(H.f[l + 1], H.u[l + 1], Lc);
-          groups = true;
-        }
-      }
-      if (!groups) k_tau<T, DIM><<<grid_for(c, nc), kBlock, 0, c->stream>>>(H.f[l + 1], H.u[l + 1], Lc);
-    }
+    launch_tau<T, DIM>(c, H, l + 1);
   }
   STATUS_TRY((launch_coarse<T, DIM>(c, H, sw, sw == lfrom ? utop : H.u[sw], sw == lfrom ? ftop : H.f[sw])));
   for (int l = sw - 1; l >= lfrom; --l) {
@@ -637,30 +731,80 @@ int seg_for_level(const fas_ctx* c, int nx, int ny) {
   return (int)std::max<int64_t>(8, std::min<int64_t>(128, (seg + 7) / 8 * 8));
 }
 
+// Levels lfrom..ntile-1 through the register-tile kernels around the single-block tile kernel. Level
+// lfrom works on (utop, ftop); tau: ftop holds R(r) of a finer level, and f is formed from it (into
+// H.f[lfrom]). zero_init: the initial guess of level lfrom is 0 (utop is not read). u64 (nullable, float32
+// level 0): add the result to this float64 field instead of storing it in utop. norm (nullable, float64,
+// lfrom < ntile): what becomes of the norm of the residual after the cycle.
+template <typename T>
+fas_status vcycle_tile(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T* ftop, bool tau, bool zero_init,
+                       double* u64, const NormEnd* norm = nullptr) {
+  const fas_params& p = c->p;
+  const int lc = H.ntile;
+  auto tried = [](cudaError_t e, const char* what) {
+    return e == cudaSuccess ? FAS_OK : fail(FAS_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
+  };
+  // the small levels (from the switch level on) are timed as the coarse family, whichever kernels run them
+  auto family = [&](int l, int fam) { return l >= H.switch_level && l > lfrom ? (int)FAS_K_COARSE : fam; };
+  for (int l = lfrom; l < lc; ++l) {
+    const bool top = l == lfrom, t = !top || tau;
+    Prof pr(c, family(l, FAS_K_SMOOTH), l, (double)c->shape[l].cells());
+    STATUS_TRY(tried(launch_tile_pre<T>(top ? (zero_init ? nullptr : utop) : H.u[l], top ? ftop : H.rc[l],
+                                        t ? H.f[l] : nullptr, H.u2[l], H.u[l + 1], l + 1 < lc ? H.rc[l + 1] : H.f[l + 1],
+                                        H.desc[l], p.nu1, p.ordering, t, H.tile_bits[l], c->sm_count, c->stream),
+                     "tile pre"));
+  }
+  {
+    Prof pr(c, FAS_K_COARSE, lc, (double)c->shape[lc].cells());
+    TileCoarse<T> A = H.tile_coarse;
+    A.tau = lc > lfrom || tau;
+    STATUS_TRY(tried(launch_tile_coarse<T>(A, lc == lfrom ? utop : H.u[lc], lc == lfrom ? ftop : H.f[lc], c->stream),
+                     "tile coarse"));
+  }
+  for (int l = lc - 1; l >= lfrom; --l) {
+    const bool top = l == lfrom, t = !top || tau;
+    Prof pr(c, family(l, (l == 0 && u64) ? FAS_K_UPDATE : FAS_K_PROLONG), l, (double)c->shape[l].cells());
+    if constexpr (std::is_same<T, double>::value) {
+      if (top && norm) {
+        STATUS_TRY(tried(launch_tile_post_norm(H.u2[l], ftop, H.u[l + 1], utop, H.desc[l], p.nu2, p.ordering,
+                                               H.tile_bits[l], *norm, c->sm_count, c->stream),
+                         "tile post"));
+        continue;
+      }
+    }
+    STATUS_TRY(tried(launch_tile_post<T>(H.u2[l], t ? H.f[l] : ftop, H.u[l + 1], top ? utop : H.u[l],
+                                         l == 0 ? u64 : nullptr, H.desc[l], p.nu2, p.ordering,
+                                         t && sizeof(T) == 8, H.tile_bits[l], c->sm_count, c->stream),
+                     "tile post"));
+  }
+  return FAS_OK;
+}
+
 // One float32 V-cycle through the sweep-fused 2D kernels on levels 0..nfast-1 (ping-pong buffers u/u2,
-// R(r) in rc), the per-operation tau kernel and the single-CTA kernel below. Result in H.u[0].
-// zero_init: the level-0 initial guess is 0 (H.u[0] is not read).
+// R(r) in rc) and the register-tile kernels (or the per-operation ones around the single-CTA kernel)
+// below. Result in H.u[0]. zero_init: the level-0 initial guess is 0 (H.u[0] is not read).
 // u64 (nullable): add the result to this float64 field instead of storing it in H.u[0].
 fas_status vcycle_fast(fas_ctx* c, Hier<float>& H, bool zero_init, double* u64) {
   const fas_params& p = c->p;
   const int nf = H.nfast;
+  if (nf == 0) return vcycle_tile<float>(c, H, 0, H.u[0], H.f[0], false, zero_init, u64);
   for (int l = 0; l < nf; ++l) {
     const LevelDesc<float>& L = H.desc[l];
     const int seg = seg_for_level(c, L.nx, L.ny);
     const bool tau = l > 0;
-    float* rc_next = (l + 1 == nf) ? H.f[l + 1] : H.rc[l + 1];
+    float* rc_next = (l + 1 < nf || (H.tiled && nf < H.ntile)) ? H.rc[l + 1] : H.f[l + 1];
     Prof pr(c, FAS_K_SMOOTH, l, (double)c->shape[l].cells());
     cudaError_t e = launch_stream2d_pre(H.u[l], tau ? H.rc[l] : H.f[l], tau ? H.f[l] : nullptr, H.u2[l], H.u[l + 1],
                                         rc_next, L, p.nu1, l == 0 && zero_init, tau, seg, c->stream);
     if (e != cudaSuccess) return fail(FAS_ECUDA, std::string("stream2d pre: ") + cudaGetErrorString(e));
   }
-  {
-    const int64_t nc = c->shape[nf].cells();
-    Prof pr(c, FAS_K_TAU, nf, (double)nc);
-    k_tau<float, 2><<<grid_for(c, nc), kBlock, 0, c->stream>>>(H.f[nf], H.u[nf], H.desc[nf]);
+  if (H.tiled) {
+    STATUS_TRY((vcycle_tile<float>(c, H, nf, H.u[nf], nf < H.ntile ? H.rc[nf] : H.f[nf], true, false, nullptr)));
+  } else {
+    launch_tau<float, 2>(c, H, nf);
+    // levels between the fused ones and the single-CTA level (narrow grids), then the small levels
+    STATUS_TRY((vcycle_basic_from<float, 2>(c, H, nf, H.u[nf], H.f[nf])));
   }
-  // levels between the fused ones and the single-CTA level (narrow grids), then the small levels
-  STATUS_TRY((vcycle_basic_from<float, 2>(c, H, nf, H.u[nf], H.f[nf])));
   for (int l = nf - 1; l >= 0; --l) {
     const LevelDesc<float>& L = H.desc[l];
     const int seg = seg_for_level(c, L.nx, L.ny);
@@ -675,6 +819,7 @@ fas_status vcycle_fast(fas_ctx* c, Hier<float>& H, bool zero_init, double* u64) 
 
 template <typename T>
 fas_status vcycle(fas_ctx* c, Hier<T>& H, T* u, const T* f) {
+  if (H.tiled) return vcycle_tile<T>(c, H, 0, u, f, false, false, nullptr);
   if (c->p.dim == 2) return vcycle_basic_from<T, 2>(c, H, 0, u, f);
   return vcycle_basic_from<T, 3>(c, H, 0, u, f);
 }
@@ -693,47 +838,41 @@ fas_status sync_read(fas_ctx* c, double* out) {
 // through its conditional handle.
 // ---------------------------------------------------------------------------------------------
 
-// ||x||_2 of a float64 level-0 field into *out (device), squares of the float-rounded values
-void enqueue_norm(fas_ctx* c, const double* x, const float* nsp, double* out) {
+// ||x||_2 of a float64 level-0 field, squares of the float-rounded values
+void enqueue_norm(fas_ctx* c, const double* x, const NormEnd& E) {
   const int64_t n = c->shape[0].cells();
-  const int g = grid_for(c, n);
-  {
-    Prof pr(c, FAS_K_NORM, 0, (double)n);
-    k_norm2<double><<<g, kBlock, 0, c->stream>>>(x, n, nsp, c->partials);
-  }
-  Prof pr(c, FAS_K_NORM, 0, 0.0);
-  k_finish_norm<<<1, kBlock, 0, c->stream>>>(c->partials, g, out, nsp);
+  Prof pr(c, FAS_K_NORM, 0, (double)n);
+  k_norm2<double><<<grid_for(c, n), kBlock, 0, c->stream>>>(x, n, E);
 }
 
-// ||b - A u||_2 into *out; mixed precision also leaves r32 = (float)(b - A u) in h32.f[0]
-// r32 = (float)(b - A u) on level 0 with per-block partials of its (nsp-scaled) squares; returns the
-// number of partials.
-int launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b, const float* nsp) {
+// r32 = (float)(b - A u) on level 0 and its norm
+void launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b, const NormEnd& E) {
   const LevelDesc<double>& L = c->h64.desc[0];
   const int64_t n = c->shape[0].cells();
-  int g = grid_for(c, n);
   Prof pr(c, FAS_K_IR, 0, (double)n);
   if (ir_strip_supported(L) &&
-      launch_ir_strip(r32, u, b, L, nsp, c->partials, c->ir_ticket, c->sm_count, c->max_blocks, &g, c->stream,
+      launch_ir_strip(r32, u, b, L, E, c->ir_ticket, c->sm_count, c->max_blocks, c->stream,
                       Ir3Wait{g_wait_limit_ns.load(), take_withhold(1)}) == cudaSuccess)
     ;  // the strip kernels took the level
   else if (c->p.dim == 2)
-    k_ir_residual<2><<<g, kBlock, 0, c->stream>>>(r32, u, b, L, nsp, c->partials);
+    k_ir_residual<2><<<grid_for(c, n), kBlock, 0, c->stream>>>(r32, u, b, L, E);
   else
-    k_ir_residual<3><<<g, kBlock, 0, c->stream>>>(r32, u, b, L, nsp, c->partials);
-  return g;
+    k_ir_residual<3><<<grid_for(c, n), kBlock, 0, c->stream>>>(r32, u, b, L, E);
 }
 
-void enqueue_residual_norm(fas_ctx* c, const double* u, const double* b, const float* nsp, double* out) {
+// The norm of b - A u; mixed precision also leaves r32 = (float)(b - A u) in h32.f[0]
+void enqueue_residual_norm(fas_ctx* c, const double* u, const double* b, const NormEnd& E) {
+  const Hier<double>& H = c->h64;
   if (c->p.precision == FAS_MIXED) {
-    const int g = launch_ir_residual(c, c->h32.f[0], u, b, nsp);
-    Prof pr(c, FAS_K_NORM, 0, 0.0);
-    k_finish_norm<<<1, kBlock, 0, c->stream>>>(c->partials, g, out, nsp);
-  } else if (c->p.dim == 2) {
-    launch_residual<double, 2>(c, c->h64.desc[0], 0, nullptr, u, b, nsp, out);
-  } else {
-    launch_residual<double, 3>(c, c->h64.desc[0], 0, nullptr, u, b, nsp, out);
-  }
+    launch_ir_residual(c, c->h32.f[0], u, b, E);
+  } else if (H.tiled && H.ntile > 0) {
+    Prof pr(c, FAS_K_RESIDUAL, 0, (double)c->shape[0].cells());
+    launch_tile_post_norm(u, b, nullptr, nullptr, H.desc[0], 0, c->p.ordering, H.tile_bits[0], E, c->sm_count,
+                          c->stream);
+  } else if (c->p.dim == 2)
+    launch_residual<double, 2>(c, c->h64.desc[0], 0, nullptr, u, b, E);
+  else
+    launch_residual<double, 3>(c, c->h64.desc[0], 0, nullptr, u, b, E);
 }
 
 void enqueue_remove_mean(fas_ctx* c, double* x, const double* y) {
@@ -757,7 +896,7 @@ fas_status mixed_step(fas_ctx* c, double* u) {
   const int64_t n = c->shape[0].cells();
   const int inner = c->p.inner_cycles > 0 ? c->p.inner_cycles : 1;
   Hier<float>& H = c->h32;
-  if (H.nfast > 0) {
+  if (H.nfast > 0 || (H.tiled && H.ntile > 0)) {
     // the last cycle's post-smoothing kernel adds its result to u in float64
     for (int k = 0; k < inner; ++k) STATUS_TRY(vcycle_fast(c, H, k == 0, k == inner - 1 ? u : nullptr));
   } else {
@@ -772,24 +911,16 @@ fas_status mixed_step(fas_ctx* c, double* u) {
 // The right-hand side the solve works with (the mean-free copy for singular problems).
 const double* solve_rhs(fas_ctx* c, const double* f) { return c->singular ? c->fproj : f; }
 
-// Enqueue everything before the first cycle. fn_ready: S->fn already holds ||f|| (heat steps).
+// Enqueue everything before the first cycle. fn_ready: S->fn and the state it starts are already set
+// (heat steps).
 fas_status enqueue_prologue(fas_ctx* c, double* u, const double* f_in, bool fn_ready, int max_cycles) {
-  const fas_params& p = c->p;
-  SolveState* S = c->S;
   const double* f = solve_rhs(c, f_in);
   if (c->singular) {
     enqueue_remove_mean(c, c->fproj, f_in);
     fn_ready = false;
   }
-  if (!fn_ready) enqueue_norm(c, f, nullptr, &S->fn);
-  const double w = p.tol_relative ? 1.0 : std::pow(c->shape[0].h, p.dim / 2.0);  // Eq. residual weight
-  {
-    Prof pr(c, FAS_K_OTHER, 0, 0.0);
-    k_solve_begin<<<1, 1, 0, c->stream>>>(S, p.tol, max_cycles, w, (double)c->shape[0].cells());
-  }
-  enqueue_residual_norm(c, u, f, &S->nscale, &S->res0);
-  Prof pr(c, FAS_K_OTHER, 0, 0.0);
-  k_solve_ref<<<1, 1, 0, c->stream>>>(S, p.tol_relative);
+  if (!fn_ready) enqueue_norm(c, f, norm_rhs(c, max_cycles));
+  enqueue_residual_norm(c, u, f, norm_to(c, kNormFirst, &c->S->nscale));
   return FAS_OK;
 }
 
@@ -798,14 +929,22 @@ fas_status enqueue_body(fas_ctx* c, double* u, const double* f_in, cudaGraphCond
   const double* f = solve_rhs(c, f_in);
   if (c->p.precision == FAS_MIXED) {
     STATUS_TRY(mixed_step(c, u));
+  } else if (c->h64.tiled && c->h64.ntile > 0 && !c->singular) {  // the last launch forms the norm as well
+    const NormEnd E = norm_cycle(c, h, set_cond);
+    return vcycle_tile<double>(c, c->h64, 0, u, f, false, false, nullptr, &E);
   } else {
     STATUS_TRY(vcycle<double>(c, c->h64, u, f));
   }
   if (c->singular) enqueue_remove_mean(c, u, u);
-  enqueue_residual_norm(c, u, f, &c->S->nscale, &c->S->res);
-  Prof pr(c, FAS_K_OTHER, 0, 0.0);
-  k_solve_step<<<1, 1, 0, c->stream>>>(c->S, h, set_cond);
+  enqueue_residual_norm(c, u, f, norm_cycle(c, h, set_cond));
   return FAS_OK;
+}
+
+// Heat step: b = u + dt fsrc and ||b||.
+void enqueue_heat_rhs(fas_ctx* c, const double* u, const double* fsrc, double dt, int max_cycles) {
+  const int64_t n = c->shape[0].cells();
+  Prof pr(c, FAS_K_OTHER, 0, (double)n);
+  k_heat_rhs<<<grid_for(c, n), kBlock, 0, c->stream>>>(c->b, u, fsrc, dt, n, norm_rhs(c, max_cycles));
 }
 
 // Enqueue the read-back of the refinement residual's timeout word (the host copy is valid after the
@@ -896,16 +1035,7 @@ fas_status solve_graph(fas_ctx* c, double* u, const double* f, const double* fsr
       cudaGraphDestroy(g.graph);
       return fail(FAS_ECUDA, std::string("graph capture: ") + cudaGetErrorString(eb));
     }
-    const int64_t n = c->shape[0].cells();
-    if (kind == 1) {
-      const int gb = grid_for(c, n);
-      {
-        Prof pr(c, FAS_K_OTHER, 0, (double)n);
-        k_heat_rhs<<<gb, kBlock, 0, main>>>(c->b, u, fsrc, dt, n, c->partials);
-      }
-      Prof pr(c, FAS_K_NORM, 0, 0.0);
-      k_finish_norm<<<1, kBlock, 0, main>>>(c->partials, gb, &c->S->fn, nullptr);
-    }
+    if (kind == 1) enqueue_heat_rhs(c, u, fsrc, dt, c->p.kmax);
     st = enqueue_prologue(c, u, f, kind == 1, c->p.kmax);
     cudaStreamCaptureStatus cs;
     cudaGraph_t cg = nullptr;
@@ -1404,7 +1534,10 @@ fas_status fas_create(const fas_params* pin, void* stream, fas_ctx** out) {
     fas_destroy(c);
     return s2;
   };
-  if (cudaMalloc(&c->partials, c->max_blocks * sizeof(double)) != cudaSuccess) return bail(fail(FAS_ENOMEM, "partials"));
+  int64_t nparts = c->max_blocks;
+  if (p.dim == 2 && p.nu2 >= 1 && p.nu2 <= kTileMaxNu)
+    nparts = std::max<int64_t>(nparts, tile_norm_blocks(c->shape[0].nx, c->shape[0].ny, p.nu2, c->sm_count));
+  if (cudaMalloc(&c->partials, nparts * sizeof(double)) != cudaSuccess) return bail(fail(FAS_ENOMEM, "partials"));
   if (cudaMalloc(&c->d_scalar, 8 * sizeof(double)) != cudaSuccess) return bail(fail(FAS_ENOMEM, "scalars"));
   if (cudaMalloc(&c->ir_ticket, 4 * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(c->ir_ticket, 0, 4 * sizeof(unsigned)) != cudaSuccess)
@@ -1428,6 +1561,7 @@ fas_status fas_create(const fas_params* pin, void* stream, fas_ctx** out) {
     return bail(fail(FAS_ENOMEM, "fproj"));
   // kernel attributes, set before any launch or stream capture
   cudaError_t e = stream2d_prepare();
+  if (e == cudaSuccess) e = tile2d_prepare();
   if (e == cudaSuccess) e = ir_strip_prepare();
   if (e == cudaSuccess) e = sweep3d_prepare();
   for (cudaError_t ek : {coarse_attr<double, 2>(), coarse_attr<double, 3>(), coarse_attr<float, 2>(),
@@ -1504,15 +1638,7 @@ fas_status fas_heat_run(fas_ctx* c, double* u, const double* fsrc, double dt, in
       c->launches += g->n_pro + (long long)c->Sh->cycles * g->n_body;
       st = finish_info(c, &inf, c->p.kmax);
     } else {
-      const int gb = grid_for(c, n);
-      {
-        Prof pr(c, FAS_K_OTHER, 0, (double)n);
-        k_heat_rhs<<<gb, kBlock, 0, c->stream>>>(c->b, u, fsrc, dt, n, c->partials);
-      }
-      {
-        Prof pr(c, FAS_K_NORM, 0, 0.0);
-        k_finish_norm<<<1, kBlock, 0, c->stream>>>(c->partials, gb, &c->S->fn, nullptr);
-      }
+      enqueue_heat_rhs(c, u, fsrc, dt, c->p.kmax);
       st = solve_impl(c, u, c->b, &inf, c->p.kmax, true);
     }
     if (infos) infos[s] = inf;
@@ -1788,9 +1914,9 @@ fas_status fas_residual(fas_ctx* c, int level, const double* u, const double* f,
   STATUS_TRY(check_field(out, false, "fas_residual"));
   const LevelDesc<double>& L = c->h64.desc[level];
   if (c->p.dim == 2)
-    launch_residual<double, 2>(c, L, level, out, u, f, nullptr, c->d_scalar);
+    launch_residual<double, 2>(c, L, level, out, u, f, norm_to(c, kNormOnly, nullptr, c->d_scalar));
   else
-    launch_residual<double, 3>(c, L, level, out, u, f, nullptr, c->d_scalar);
+    launch_residual<double, 3>(c, L, level, out, u, f, norm_to(c, kNormOnly, nullptr, c->d_scalar));
   double v = 0.0;
   STATUS_TRY(sync_read(c, &v));
   if (norm2) *norm2 = v;
@@ -1801,11 +1927,7 @@ fas_status fas_residual_ir(fas_ctx* c, const double* u, const double* f, float* 
   STATUS_TRY(check_ctx(c));
   for (const void* q : {(const void*)u, (const void*)f, (const void*)r32})
     STATUS_TRY(check_field(q, true, "fas_residual_ir"));
-  const int g = launch_ir_residual(c, r32, u, f, nullptr);
-  {
-    Prof pr(c, FAS_K_NORM, 0, 0.0);
-    k_finish_norm<<<1, kBlock, 0, c->stream>>>(c->partials, g, c->d_scalar, nullptr);
-  }
+  launch_ir_residual(c, r32, u, f, norm_to(c, kNormOnly, nullptr, c->d_scalar));
   CUDA_TRY(enqueue_timeout_read(c, c->stream));
   double v = 0.0;
   STATUS_TRY(sync_read(c, &v));

@@ -299,7 +299,7 @@ __device__ __forceinline__ void ir_row(const IrRowM<CPL>& P, const IrRowM<CPL>& 
 template <int CPL, int MINB>
 __global__ void __launch_bounds__(kIrThreads, MINB)
     k_ir_strip(float* __restrict__ r32, const double* __restrict__ u, const double* __restrict__ b, LevelDesc<double> L,
-               const float* nsp, double* partials, unsigned* ticket, int seg) {
+               const __grid_constant__ NormEnd E, unsigned* ticket, int seg) {
   constexpr int COLS = 32 * CPL;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kIrThreads, MINB)
   const int nstrips = nx / COLS;
   const int nseg = (ny + seg - 1) / seg;
   const int ntasks = nstrips * nseg;
-  const float nscale = nsp ? *nsp : 1.f;
+  const float nscale = E.nsp ? *E.nsp : 1.f;
   float acc = 0.f;
   (void)warp;
   for (;;) {
@@ -335,15 +335,8 @@ __global__ void __launch_bounds__(kIrThreads, MINB)
       R1 = R2;
     }
   }
-  const double s = block_sum((double)acc);  // every warp of the block has left the task loop
-  if (threadIdx.x == 0) {
-    partials[blockIdx.x] = s;
-    __threadfence();
-    if (atomicAdd(ticket + 1, 1u) == gridDim.x - 1) {  // the last block: no warp takes tasks any more
-      ticket[0] = 0u;
-      ticket[1] = 0u;
-    }
-  }
+  // every warp of the block has left the task loop; in the last block, no warp takes tasks any more
+  if (norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x)) ticket[0] = 0u;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -454,8 +447,8 @@ __device__ __forceinline__ void align_row(ARow& R, const uint64_t (&v)[4], const
 
 __global__ void __launch_bounds__(kIrThreads, 2)
     k_ir_strip3(float* __restrict__ r32, const double* __restrict__ u, const __grid_constant__ CUtensorMap tu,
-                const __grid_constant__ CUtensorMap tb, LevelDesc<double> L, const float* nsp, double* partials,
-                unsigned* ticket, int zseg, Ir3Wait wt) {
+                const __grid_constant__ CUtensorMap tb, LevelDesc<double> L,
+                const __grid_constant__ NormEnd E, unsigned* ticket, int zseg, Ir3Wait wt) {
   extern __shared__ __align__(128) unsigned char smem3[];
   // the rings start on a 128-byte boundary (tile copies land on 128-byte aligned slots)
   double* su = reinterpret_cast<double*>(smem3 + ((128u - (smem_u32(smem3) & 127u)) & 127u));
@@ -474,7 +467,7 @@ __global__ void __launch_bounds__(kIrThreads, 2)
   const int nyg = ny / kIr3Rows;
   const int nzs = (nz + zseg - 1) / zseg;
   const int ntasks = nstrips * nyg * nzs;
-  const float nscale = nsp ? *nsp : 1.f;
+  const float nscale = E.nsp ? *E.nsp : 1.f;
   if (tid == 0) {
     for (int k = 0; k < kNBar; ++k) mbar_init(bar + k, 1);
     mbar_init_fence();
@@ -710,15 +703,8 @@ __global__ void __launch_bounds__(kIrThreads, 2)
     for (int k = 0; k < kNBar; ++k)
       if ((pend >> k) & 1u) mbar_wait_bounded(bar + k, (par >> k) & 1u, wt.limit_ns);
   }
-  const double s = block_sum((double)acc);  // every warp of the block has left the task loop
-  if (tid == 0) {
-    partials[blockIdx.x] = s;
-    __threadfence();
-    if (atomicAdd(ticket + 1, 1u) == gridDim.x - 1) {  // the last block: no block takes tasks any more
-      ticket[0] = 0u;
-      ticket[1] = 0u;
-    }
-  }
+  // every warp of the block has left the task loop; in the last block, no block takes tasks any more
+  if (norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x)) ticket[0] = 0u;
 }
 
 }  // namespace
@@ -734,8 +720,8 @@ bool ir_strip_supported(const LevelDesc<double>& L) {
 }
 
 cudaError_t launch_ir_strip(float* r32, const double* u, const double* b, const LevelDesc<double>& L,
-                            const float* nsp, double* partials, unsigned* ticket, int sm_count, int max_blocks,
-                            int* nblocks, cudaStream_t stream, Ir3Wait wt) {
+                            const NormEnd& E, unsigned* ticket, int sm_count, int max_blocks, cudaStream_t stream,
+                            Ir3Wait wt) {
   const int nstrips = L.nx / kIrCols;
   if (L.nz > 1) {
     // one wave of two blocks of eight rows y per SM taking (strip, row group, plane segment) tasks;
@@ -750,8 +736,7 @@ cudaError_t launch_ir_strip(float* r32, const double* u, const double* b, const 
     cudaError_t e = tensor_map_3d(&tu, u, sizeof(double), L.nx, L.ny, L.nz, kU3W, kU3H, 1);
     if (e == cudaSuccess) e = tensor_map_3d(&tb, b, sizeof(double), L.nx, L.ny, L.nz, kIrCols, kIr3Rows, 1);
     if (e != cudaSuccess) return e;
-    *nblocks = blocks;
-    k_ir_strip3<<<blocks, kIrThreads, kIr3Smem, stream>>>(r32, u, tu, tb, L, nsp, partials, ticket, zseg, wt);
+    k_ir_strip3<<<blocks, kIrThreads, kIr3Smem, stream>>>(r32, u, tu, tb, L, E, ticket, zseg, wt);
     return cudaGetLastError();
   }
   // one wave of kIrMinBlocks2D blocks of eight warps per SM; segments of 16..256 rows (two halo rows
@@ -764,8 +749,7 @@ cudaError_t launch_ir_strip(float* r32, const double* u, const double* b, const 
   const int64_t want = (ntasks + kIrWarps - 1) / kIrWarps;
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(max_blocks, want),
                                                                    (int64_t)sm_count * kIrMinBlocks2D));
-  *nblocks = blocks;
-  k_ir_strip<kIrCpl2D, kIrMinBlocks2D><<<blocks, kIrThreads, 0, stream>>>(r32, u, b, L, nsp, partials, ticket, seg);
+  k_ir_strip<kIrCpl2D, kIrMinBlocks2D><<<blocks, kIrThreads, 0, stream>>>(r32, u, b, L, E, ticket, seg);
   return cudaGetLastError();
 }
 

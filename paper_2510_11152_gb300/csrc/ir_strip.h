@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "solve_state.cuh"
 
 namespace fasmg {
 
@@ -21,13 +22,12 @@ struct Ir3Wait {
 // Kernel attributes (dynamic shared memory of the 3D kernel); call once before any launch or capture.
 cudaError_t ir_strip_prepare();
 
-// r32 = (float)(b - A u) and per-block partials of sum (s r32)^2 (s = *nsp, or 1) into
-// partials[0 .. *nblocks). At most max_blocks blocks are launched. ticket: three zeroed counters; the
-// kernels hand out their work with the first two (and leave them zero again); the 3D kernel sets the
-// third when a bounded wait ran out (the caller reports FAS_ETIMEOUT and clears it). Launches sharing
-// them must not overlap.
+// r32 = (float)(b - A u) and its norm (solve_state.cuh; squares scaled by *E.nsp). At most max_blocks
+// blocks are launched. ticket: three zeroed counters; the kernels hand out their work with the first
+// and leave it zero again; E.ticket is the second; the 3D kernel sets the third when a bounded wait ran out
+// (the caller reports FAS_ETIMEOUT and clears it). Launches sharing them must not overlap.
 cudaError_t launch_ir_strip(float* r32, const double* u, const double* b, const LevelDesc<double>& L,
-                            const float* nsp, double* partials, unsigned* ticket, int sm_count, int max_blocks,
-                            int* nblocks, cudaStream_t stream, Ir3Wait wt);
+                            const NormEnd& E, unsigned* ticket, int sm_count, int max_blocks, cudaStream_t stream,
+                            Ir3Wait wt);
 
 }  // namespace fasmg
