@@ -1687,11 +1687,14 @@ fas_status fas_heat_adjoint(fas_ctx* c, const double* u0, const double* fsrc, do
     }
     return s2;
   };
-  // forward sweep, keeping every K-th state
+  // forward sweep, keeping every K-th state, and every state of the last segment: the backward sweep
+  // starts there, so that segment needs no recomputation (with nsteps <= K, none does)
+  const int last0 = (nseg - 1) * K;
   CUDA_TRY(cudaMemcpyAsync(work, u0, bytes, cudaMemcpyDeviceToDevice, st));
   for (int k = 0; k < nsteps; ++k) {
-    if (k % K == 0) CUDA_TRY(cudaMemcpyAsync(ckpt[k / K], work, bytes, cudaMemcpyDeviceToDevice, st));
+    if (k % K == 0 && k < last0) CUDA_TRY(cudaMemcpyAsync(ckpt[k / K], work, bytes, cudaMemcpyDeviceToDevice, st));
     STATUS_TRY(step(work));
+    if (k >= last0) CUDA_TRY(cudaMemcpyAsync(seg[k + 1 - last0], work, bytes, cudaMemcpyDeviceToDevice, st));
   }
   if (uT) CUDA_TRY(cudaMemcpyAsync(uT, work, bytes, cudaMemcpyDeviceToDevice, st));
   // backward sweep
@@ -1705,10 +1708,9 @@ fas_status fas_heat_adjoint(fas_ctx* c, const double* u0, const double* fsrc, do
   const int lx = c->h64.desc[0].lx, ly = c->h64.desc[0].ly;
   for (int sgi = nseg - 1; sgi >= 0; --sgi) {
     const int n0 = sgi * K, n1 = std::min(n0 + K, nsteps);
-    // recompute the segment's states u^{n0}..u^{n1}
-    CUDA_TRY(cudaMemcpyAsync(work, ckpt[sgi], bytes, cudaMemcpyDeviceToDevice, st));
-    CUDA_TRY(cudaMemcpyAsync(seg[0], work, bytes, cudaMemcpyDeviceToDevice, st));
-    for (int j = 1; j <= n1 - n0; ++j) {
+    // recompute the segment's states u^{n0 + 1}..u^{n1} (the last segment's are there)
+    if (sgi < nseg - 1) CUDA_TRY(cudaMemcpyAsync(work, ckpt[sgi], bytes, cudaMemcpyDeviceToDevice, st));
+    for (int j = 1; j <= n1 - n0 && sgi < nseg - 1; ++j) {
       STATUS_TRY(step(work));
       CUDA_TRY(cudaMemcpyAsync(seg[j], work, bytes, cudaMemcpyDeviceToDevice, st));
     }
