@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "basic_kernels.cuh"
+#include "col3d.h"
 #include "context.h"
 #include "ir_strip.h"
 #include "stream2d.h"
@@ -71,6 +72,7 @@ constexpr int64_t kSwitchCells3D = 4096;
 constexpr size_t kCoarseSmemMax = 200 * 1024;    // field arrays of the single-CTA kernel
 constexpr size_t kCoarseSmemLimit = 227 * 1024;  // with its level descriptors (per-CTA maximum)
 constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smoothed by the fused sweep
+constexpr int64_t kCol3dMinCells = (int64_t)1 << 21;  // smallest 3D level of the column-streaming kernels
 constexpr int64_t kFusedMinCells2D = (int64_t)1 << 20;  // smallest 2D level below the finest run fused
 
 int grid_for(const fas_ctx* c, int64_t work) {
@@ -206,6 +208,7 @@ void free_hier(Hier<T>& H) {
   H.nfast = 0;
   H.ntile = 0;
   H.tiled = false;
+  H.ncol = 0;
   H.d_desc = nullptr;
   H.cinv = nullptr;
   H.allocated = false;
@@ -482,7 +485,21 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
     // (its sweeps ping-pong between the two) and that is large enough for it to pay: measured at
     // 512^3 it beats two colour launches (0.58 against 0.67 ms), at 256^3 it does not
     if constexpr (std::is_same<T, float>::value) {
-      if (p.dim == 3 && p.path != 1 && p.ordering == FAS_ORDER_FORWARD && p.nu1 + p.nu2 >= 2)
+      // column-streaming 3D path: consecutive levels from the finest, where there is room for their second
+      // buffers
+      if (p.dim == 3 && p.path == 0 && p.ordering == FAS_ORDER_FORWARD) {
+        while (H.ncol < H.switch_level && col3d_supported(H.desc[H.ncol], p.nu1) &&
+               col3d_supported(H.desc[H.ncol], p.nu2) && c->shape[H.ncol].cells() >= kCol3dMinCells)
+          H.ncol++;
+        for (int l = 0; l < H.ncol; ++l)
+          if (dev_alloc(H, &H.u2[l], c->shape[l].cells()) != FAS_OK ||
+              (l > 0 && dev_alloc(H, &H.rc[l], c->shape[l].cells()) != FAS_OK)) {
+            cudaGetLastError();
+            H.ncol = 0;
+            std::fill(H.u2.begin(), H.u2.end(), nullptr);
+          }
+      }
+      if (p.dim == 3 && p.path != 1 && H.ncol == 0 && p.ordering == FAS_ORDER_FORWARD && p.nu1 + p.nu2 >= 2)
         for (int l = 0; l < H.switch_level; ++l)
           if (sweep3d_supported(H.desc[l]) && (c->shape[l].cells() >= kSweep3dMinCells || p.path == 2))
             STATUS_TRY(dev_alloc(H, &H.u2[l], c->shape[l].cells()));
@@ -817,6 +834,30 @@ fas_status vcycle_fast(fas_ctx* c, Hier<float>& H, bool zero_init, double* u64) 
   return FAS_OK;
 }
 
+// One float32 V-cycle of a 3D hierarchy on H.u[0], H.f[0]: levels 0..ncol-1 through the column-streaming
+// kernels, the others per operation. zero_init: the initial guess is 0 (H.u[0] is not read).
+fas_status vcycle_col(fas_ctx* c, Hier<float>& H, bool zero_init) {
+  const fas_params& p = c->p;
+  const int nc = H.ncol;
+  for (int l = 0; l < nc; ++l) {
+    Prof pr(c, FAS_K_SMOOTH, l, (double)c->shape[l].cells());
+    const cudaError_t e = launch_col3d_pre(l == 0 && zero_init ? nullptr : H.u[l], l == 0 ? H.f[0] : H.rc[l],
+                                           l == 0 ? nullptr : H.f[l], H.u2[l], H.u[l + 1],
+                                           l + 1 < nc ? H.rc[l + 1] : H.f[l + 1], H.desc[l], p.nu1, l > 0, c->sm_count,
+                                           c->stream);
+    if (e != cudaSuccess) return fail(FAS_ECUDA, std::string("col3d pre: ") + cudaGetErrorString(e));
+  }
+  launch_tau<float, 3>(c, H, nc);
+  STATUS_TRY((vcycle_basic_from<float, 3>(c, H, nc, H.u[nc], H.f[nc])));
+  for (int l = nc - 1; l >= 0; --l) {
+    Prof pr(c, FAS_K_PROLONG, l, (double)c->shape[l].cells());
+    const cudaError_t e =
+        launch_col3d_post(H.u2[l], H.f[l], H.u[l + 1], H.u[l], H.desc[l], p.nu2, c->sm_count, c->stream);
+    if (e != cudaSuccess) return fail(FAS_ECUDA, std::string("col3d post: ") + cudaGetErrorString(e));
+  }
+  return FAS_OK;
+}
+
 template <typename T>
 fas_status vcycle(fas_ctx* c, Hier<T>& H, T* u, const T* f) {
   if (H.tiled) return vcycle_tile<T>(c, H, 0, u, f, false, false, nullptr);
@@ -900,8 +941,9 @@ fas_status mixed_step(fas_ctx* c, double* u) {
     // the last cycle's post-smoothing kernel adds its result to u in float64
     for (int k = 0; k < inner; ++k) STATUS_TRY(vcycle_fast(c, H, k == 0, k == inner - 1 ? u : nullptr));
   } else {
-    CUDA_TRY(cudaMemsetAsync(H.u[0], 0, n * sizeof(float), c->stream));
-    for (int k = 0; k < inner; ++k) STATUS_TRY(vcycle<float>(c, H, H.u[0], H.f[0]));
+    if (H.ncol == 0) CUDA_TRY(cudaMemsetAsync(H.u[0], 0, n * sizeof(float), c->stream));
+    for (int k = 0; k < inner; ++k)
+      STATUS_TRY(H.ncol > 0 ? vcycle_col(c, H, k == 0) : vcycle<float>(c, H, H.u[0], H.f[0]));
     Prof pr(c, FAS_K_UPDATE, 0, (double)n);
     k_ir_update<<<grid_for(c, (n + 3) / 4), kBlock, 0, c->stream>>>(u, H.u[0], n);
   }
@@ -1562,6 +1604,7 @@ fas_status fas_create(const fas_params* pin, void* stream, fas_ctx** out) {
   // kernel attributes, set before any launch or stream capture
   cudaError_t e = stream2d_prepare();
   if (e == cudaSuccess) e = tile2d_prepare();
+  if (e == cudaSuccess) e = col3d_prepare();
   if (e == cudaSuccess) e = ir_strip_prepare();
   if (e == cudaSuccess) e = sweep3d_prepare();
   for (cudaError_t ek : {coarse_attr<double, 2>(), coarse_attr<double, 3>(), coarse_attr<float, 2>(),
