@@ -327,31 +327,57 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
       if (l > 0 || pz) b4.ld(u + (l > 0 ? idx - sz : idx + (nz - 1) * sz));
       if (l < nz - 1 || pz) t4.ld(u + (l < nz - 1 ? idx + sz : idx - (nz - 1) * sz));
     }
-    // cell x has the colour when (x + j + l + DIM + colour) is even; the same along a row
-    auto upd = [&](auto kc) {
-      constexpr int k = decltype(kc)::value;
-      const int i = x0 + k;
-      if (L.fax >= 0 && frozen(L, i, j, l)) return;
-      const T w = (i > 0 || px) ? (k > 0 ? c.v[k > 0 ? k - 1 : 0] : wedge) : T(0);
-      const T e = (i < nx - 1 || px) ? (k < 3 ? c.v[k < 3 ? k + 1 : 3] : eedge) : T(0);
-      const T sv = (j > 0 || py) ? s4.v[k] : T(0);
-      const T nv = (j < ny - 1 || py) ? n4.v[k] : T(0);
-      T acc = (w + e) + (sv + nv);
-      if (DIM == 3) {
-        const T bo = (l > 0 || pz) ? b4.v[k] : T(0);
-        const T to = (l < nz - 1 || pz) ? t4.v[k] : T(0);
-        acc = acc + (bo + to);
+    // cell x has the colour when (x + j + l + DIM + colour) is even; the same along a row: cells K and K + 2
+    auto upd2 = [&](auto kc) {
+      constexpr int K = decltype(kc)::value;
+      // row neighbours of the two cells (the middle one is common), and the others
+      const T x0v = K ? c.v[0] : (x0 > 0 || px ? wedge : T(0));
+      const T x1v = c.v[K + 1];
+      const T x2v = K ? (x0 + 4 < nx || px ? eedge : T(0)) : c.v[3];
+      T sv[2], nv[2], bo[2], to[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        sv[q] = (j > 0 || py) ? s4.v[K + 2 * q] : T(0);
+        nv[q] = (j < ny - 1 || py) ? n4.v[K + 2 * q] : T(0);
+        bo[q] = DIM == 3 && (l > 0 || pz) ? b4.v[K + 2 * q] : T(0);
+        to[q] = DIM == 3 && (l < nz - 1 || pz) ? t4.v[K + 2 * q] : T(0);
       }
-      const int cls = bclass<DIM>(i, j, l, nx, ny, nz);
-      c.v[k] = fma(L.a[cls], acc, L.b[cls] * f4.v[k]);
+      T acc[2];
+      bool done = false;
+      if constexpr (std::is_same<T, double>::value && DIM == 3) {
+        // both sums by integers at one scale (bits64.cuh), the common value converted once
+        int top = max(max(exp_field(x0v), exp_field(x1v)), exp_field(x2v));
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          top = max(top, max(max(exp_field(sv[q]), exp_field(nv[q])), max(exp_field(bo[q]), exp_field(to[q]))));
+        if (sum_range_ok(top)) {
+          const int64_t m = sum_units(x1v, top);
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            acc[q] = sum_value((m + sum_units(q ? x2v : x0v, top)) + (sum_units(sv[q], top) + sum_units(nv[q], top)) +
+                                   (sum_units(bo[q], top) + sum_units(to[q], top)),
+                               top);
+          done = true;
+        }
+      }
+      if (!done) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          acc[q] = (q ? x1v + x2v : x0v + x1v) + (sv[q] + nv[q]);
+          if (DIM == 3) acc[q] = acc[q] + (bo[q] + to[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = x0 + K + 2 * q;
+        const int cls = bclass<DIM>(i, j, l, nx, ny, nz);
+        if (!(L.fax >= 0 && frozen(L, i, j, l))) c.v[K + 2 * q] = fma(L.a[cls], acc[q], L.b[cls] * f4.v[K + 2 * q]);
+      }
     };
-    if (((x0 + j + l + DIM + colour) & 1) == 0) {
-      upd(std::integral_constant<int, 0>());
-      upd(std::integral_constant<int, 2>());
-    } else {
-      upd(std::integral_constant<int, 1>());
-      upd(std::integral_constant<int, 3>());
-    }
+    if (((x0 + j + l + DIM + colour) & 1) == 0)
+      upd2(std::integral_constant<int, 0>());
+    else
+      upd2(std::integral_constant<int, 1>());
     c.st(u + idx);
   }
 }
@@ -403,9 +429,67 @@ __global__ void k_restrict_face(T* uc, T* uc0, T* fc, const T* u, const T* r, in
   restrict_face_range<T, DIM, FAX>(uc, uc0, fc, u, r, nxf, nyf, nzf, gtid(), gstride());
 }
 
+// The same prolongation with a thread per coarse cell, that is per 2^DIM fine slots: the correction's tangential
+// interpolation (weights 3/4, 1/4; here 3 and 1 with the scale left to the end) is formed once for each of
+// the two coarse slots S - 1 and S along the face axis and used by all fine slots between them, instead of up
+// to 2^DIM weighted coarse values for every fine slot (128^3, float64: 149 us for about 32 float64
+// operations per fine cell; here about 6).
 template <typename T, int DIM, int FAX>
 __global__ void k_prolong_face(T* u, const T* uc, const T* uc0, int nxf, int nyf, int nzf) {
-  prolong_face_range<T, DIM, FAX>(u, uc, uc0, nxf, nyf, nzf, gtid(), gstride());
+  const int nc3[3] = {nxf >> 1, nyf >> 1, DIM == 3 ? nzf >> 1 : 1};
+  const int lxc = __ffs(nc3[0]) - 1, lyc = __ffs(nc3[1]) - 1;
+  const int64_t nc = (int64_t)nc3[0] * nc3[1] * nc3[2];
+  const int64_t cst[3] = {1, nc3[0], (int64_t)nc3[0] * nc3[1]};
+  const int64_t fst[3] = {1, nxf, (int64_t)nxf * nyf};
+  constexpr int T1 = FAX == 0 ? 1 : 0;                         // first tangential axis
+  constexpr int T2 = DIM == 3 ? (FAX == 2 ? 1 : 2) : T1;       // second (3D)
+  constexpr int N2 = DIM == 3 ? 3 : 1;
+  for (int64_t I = gtid(); I < nc; I += gstride()) {
+    const int c3[3] = {(int)(I & (nc3[0] - 1)), (int)((I >> lxc) & (nc3[1] - 1)), (int)(I >> (lxc + lyc))};
+    const int S = c3[FAX];
+    // w[s][a][b]: interpolated correction times 4^(DIM-1) at coarse slot S - 1 + s for tangential fine cells a, b
+    T w[2][2][DIM == 3 ? 2 : 1];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      // slot S - 1 is the near wall for S = 0, slot S the far wall for the last S: both 0
+      const bool wall = s == 0 ? S == 0 : S == nc3[FAX] - 1;
+      T v[3][N2];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < N2; ++b) {
+          const int pa = c3[T1] + a - 1, pb = DIM == 3 ? c3[T2] + b - 1 : 0;
+          const bool ga = pa < 0 || pa >= nc3[T1], gb = DIM == 3 && (pb < 0 || pb >= nc3[T2]);
+          int64_t q = I + (s - 1) * cst[FAX] + (ga ? 0 : (a - 1) * cst[T1]);
+          if (DIM == 3) q += gb ? 0 : (b - 1) * cst[T2];
+          T cv = T(0);
+          if (!wall) cv = uc0 ? uc[q] - uc0[q] : uc[q];
+          v[a][b] = ga != gb ? -cv : cv;  // the ghost beyond a wall is minus the value inside
+        }
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        T t[N2];
+#pragma unroll
+        for (int b = 0; b < N2; ++b) t[b] = fma(T(3), v[1][b], v[2 * a][b]);
+        if constexpr (DIM == 3) {
+          w[s][a][0] = fma(T(3), t[1], t[0]);
+          w[s][a][1] = fma(T(3), t[1], t[2]);
+        } else {
+          w[s][a][0] = t[0];
+        }
+      }
+    }
+    const int64_t base = (int64_t)(2 * c3[0]) + (int64_t)(2 * c3[1]) * fst[1] + (DIM == 3 ? 2 * c3[2] * fst[2] : 0);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < (DIM == 3 ? 2 : 1); ++b) {
+        const int64_t q = base + a * fst[T1] + (DIM == 3 ? b * fst[T2] : 0);
+        const T scale = DIM == 3 ? T(0.0625) : T(0.25);
+        u[q] = fma(T(0.5) * scale, w[0][a][b] + w[1][a][b], u[q]);  // halfway between coarse slots S - 1 and S
+        if (S < nc3[FAX] - 1) u[q + fst[FAX]] = fma(scale, w[1][a][b], u[q + fst[FAX]]);  // coincides with slot S
+      }
+  }
 }
 
 // per-block partial sums of x (for means of singular problems)

@@ -155,6 +155,21 @@ __device__ __forceinline__ double f64_of_units(int64_t X, int base) {
   return __longlong_as_double((long long)(A == 0 ? 0ull : (sign | r)));
 }
 
+// ---- sums of a few float64 values in block fixed point: each value v becomes the integer
+// v 2^(kSumBits + 1022 - top), top the largest biased exponent among them, cut below one unit (exact for
+// values within 2^7 of the largest; the unit is 2^-60 of it, where a float64 addition rounds at 2^-53 of its
+// result's magnitude). Up to six such values add up without overflow; the sum is rounded once.
+constexpr int kSumBits = 60;
+__device__ __forceinline__ bool sum_range_ok(int top) { return (unsigned)(top - 70) <= 1970u; }
+__device__ __forceinline__ int64_t sum_units(double v, int top) {
+  const uint32_t hi = (uint32_t)((uint64_t)__double_as_longlong(v) >> 32);
+  const uint64_t m = (((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | (uint32_t)__double_as_longlong(v)) << 7;
+  // a zero or subnormal has exponent field 0, at least 70 below top: shifted out
+  const int64_t X = (int64_t)(m >> min(top - (int)((hi >> 20) & 0x7FFu), 63));
+  return (int)hi < 0 ? -X : X;
+}
+__device__ __forceinline__ double sum_value(int64_t S, int top) { return f64_of_units(S, top - kSumBits + 63); }
+
 // Largest exponent spread handled exactly: significands < 2^58, at most 6 neighbours plus M <= 9
 // times the centre keep |S| < 2^62.
 constexpr int kMaxExpSpread = 5;

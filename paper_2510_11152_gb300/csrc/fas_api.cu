@@ -564,7 +564,7 @@ void launch_prolong(fas_ctx* c, int64_t n, T* u, const T* uc, const T* uc0, int 
     if constexpr (FAX < 0)
       k_prolong<T, DIM><<<grid_for(c, n >> DIM), kBlock, 0, c->stream>>>(u, uc, uc0, nx, ny, nz);
     else
-      k_prolong_face<T, DIM, FAX><<<grid_for(c, n), kBlock, 0, c->stream>>>(u, uc, uc0, nx, ny, nz);
+      k_prolong_face<T, DIM, FAX><<<grid_for(c, n >> DIM), kBlock, 0, c->stream>>>(u, uc, uc0, nx, ny, nz);
   });
 }
 
