@@ -603,6 +603,128 @@ __global__ void k_ir_residual(float* r32, const double* u, const double* b, Leve
   norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
+// The four cells of a group (x0 .. x0 + 3) and their neighbours, 0 where there is none.
+template <int DIM>
+struct Group4 {
+  Quad<double> c, s, n, b, t;
+  double w, e;
+  __device__ __forceinline__ void load(const double* __restrict__ u, int64_t idx, int x0, int j, int l,
+                                       const LevelDesc<double>& L) {
+    const int nx = L.nx, ny = L.ny, nz = L.nz;
+    const int64_t sy = nx, sz = (int64_t)nx * ny;
+    const bool px = L.per & 1, py = (L.per >> 1) & 1, pz = (L.per >> 2) & 1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s.v[k] = n.v[k] = b.v[k] = t.v[k] = 0.0;
+    c.ld(u + idx);
+    w = x0 > 0 || px ? u[x0 > 0 ? idx - 1 : idx + nx - 1] : 0.0;
+    e = x0 + 4 < nx || px ? u[x0 + 4 < nx ? idx + 4 : idx + 4 - nx] : 0.0;
+    if (j > 0 || py) s.ld(u + (j > 0 ? idx - sy : idx + (ny - 1) * sy));
+    if (j < ny - 1 || py) n.ld(u + (j < ny - 1 ? idx + sy : idx - (ny - 1) * sy));
+    if (DIM == 3) {
+      if (l > 0 || pz) b.ld(u + (l > 0 ? idx - sz : idx + (nz - 1) * sz));
+      if (l < nz - 1 || pz) t.ld(u + (l < nz - 1 ? idx + sz : idx - (nz - 1) * sz));
+    }
+  }
+  __device__ __forceinline__ int top() const {
+    int m = max(exp_field(w), exp_field(e));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      m = max(m, max(exp_field(c.v[k]), max(exp_field(s.v[k]), exp_field(n.v[k]))));
+      if (DIM == 3) m = max(m, max(exp_field(b.v[k]), exp_field(t.v[k])));
+    }
+    return m;
+  }
+  // the neighbours' float64 sum, in the order of nbsum_t
+  __device__ __forceinline__ double sum_f64(int k) const {
+    const double acc = ((k ? c.v[k > 0 ? k - 1 : 0] : w) + (k < 3 ? c.v[k < 3 ? k + 1 : 3] : e)) + (s.v[k] + n.v[k]);
+    return DIM == 3 ? acc + (b.v[k] + t.v[k]) : acc;
+  }
+};
+
+// The residual of a float64 level with constant kappa and a multiple of 4 cells per row, one thread per group of
+// 4 cells, with the neighbour sums in block fixed point at the group's scale (bits64.cuh): the group's 14
+// (2D) or 22 (3D) values are converted once and each cell's sum is integer additions.
+//   IR:  r32 = (float)(f - A u), the point equation as fma(c, S, fma(-alpha, u, f)) with S = sum_nb u_nb - M u
+//        (exact, rounded once, when the group's values lie within 2^6 (2D) or 2^5 (3D) of one another; cut below
+//        2^-59 (2^-58) of the largest otherwise);
+//   not IR: r (nullable) = fma(c, N, fma(-d, u, f)), N the neighbour sum.
+// About 90 (2D) and 110 (3D) instructions per cell; a thread per cell with its own conversions took 250, the 3D
+// plane-streaming kernel (ir_strip.cu) 247.
+template <int DIM, bool IR>
+__global__ void __launch_bounds__(256) k_residual4(typename std::conditional<IR, float, double>::type* r, const double* u,
+                                                   const double* f, const __grid_constant__ LevelDesc<double> L,
+                                                   const __grid_constant__ NormEnd E) {
+  constexpr int BITS = DIM == 2 ? 59 : 58;  // |S| <= (2 DIM + M) 2^BITS < 2^63, M <= 4 DIM
+  const int nx = L.nx, ny = L.ny, nz = L.nz;
+  const int lg = L.lx - 2;
+  const int64_t ngroups = (int64_t)1 << (lg + L.ly + L.lz);
+  const float nscale = E.nsp ? *E.nsp : 1.f;
+  float acc = 0.f;
+  for (int64_t g = gtid(); g < ngroups; g += gstride()) {
+    const int x0 = (int)(g & ((1 << lg) - 1)) << 2;
+    const int64_t rest = g >> lg;
+    const int j = (int)(rest & (ny - 1));
+    const int l = (int)(rest >> L.ly);
+    const int64_t idx = ((int64_t)l * ny + j) * nx + x0;
+    Group4<DIM> q;
+    q.load(u, idx, x0, j, l, L);
+    Quad<double> fq;
+    fq.ld(f + idx);
+    const int top = q.top();
+    double rv[4];
+    if (sum_range_ok(top)) {
+      int64_t C[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) C[k] = sum_units<BITS>(q.c.v[k], top);
+      const int64_t W = sum_units<BITS>(q.w, top), Ea = sum_units<BITS>(q.e, top);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        int64_t S = ((k ? C[k > 0 ? k - 1 : 0] : W) + (k < 3 ? C[k < 3 ? k + 1 : 3] : Ea)) +
+                    (sum_units<BITS>(q.s.v[k], top) + sum_units<BITS>(q.n.v[k], top));
+        if (DIM == 3) S += sum_units<BITS>(q.b.v[k], top) + sum_units<BITS>(q.t.v[k], top);
+        const int cls = bclass<DIM>(x0 + k, j, l, nx, ny, nz);
+        if (IR) {
+          S -= (int64_t)L.mt[cls] * C[k];
+          rv[k] = fma(L.c, sum_value<BITS>(S, top), fma(-L.alpha, q.c.v[k], fq.v[k]));
+        } else {
+          rv[k] = fma(L.c, sum_value<BITS>(S, top), fma(-L.d[cls], q.c.v[k], fq.v[k]));
+        }
+      }
+    } else {  // all zero, non-finite values, or values near the ends of the float64 range
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        rv[k] = fma(L.c, q.sum_f64(k), fma(-L.d[bclass<DIM>(x0 + k, j, l, nx, ny, nz)], q.c.v[k], fq.v[k]));
+    }
+    if (L.fax >= 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (frozen(L, x0 + k, j, l)) rv[k] = 0.0;
+    }
+    float o[4];
+    if (f32_normal_range(rv[0]) && f32_normal_range(rv[1]) && f32_normal_range(rv[2]) && f32_normal_range(rv[3])) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) o[k] = f64_to_f32_rn_normal(rv[k]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) o[k] = f64_to_f32_rn_bits(rv[k]);
+    }
+    if constexpr (IR) {
+      *reinterpret_cast<float4*>(r + idx) = make_float4(o[0], o[1], o[2], o[3]);
+    } else if (r) {
+      Quad<double> oq;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) oq.v[k] = rv[k];
+      oq.st(r + idx);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float v = o[k] * nscale;
+      acc = fmaf(v, v, acc);
+    }
+  }
+  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
+}
+
 // ||x||, squares of the float-rounded values (norms for stopping
 // tests need a few digits only, and the conversion keeps the work off the FP64 pipe)
 template <typename T>

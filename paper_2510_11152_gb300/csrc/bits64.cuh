@@ -161,14 +161,19 @@ __device__ __forceinline__ double f64_of_units(int64_t X, int base) {
 // result's magnitude). Up to six such values add up without overflow; the sum is rounded once.
 constexpr int kSumBits = 60;
 __device__ __forceinline__ bool sum_range_ok(int top) { return (unsigned)(top - 70) <= 1970u; }
+template <int BITS = kSumBits>
 __device__ __forceinline__ int64_t sum_units(double v, int top) {
   const uint32_t hi = (uint32_t)((uint64_t)__double_as_longlong(v) >> 32);
-  const uint64_t m = (((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | (uint32_t)__double_as_longlong(v)) << 7;
+  const uint64_t m = (((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | (uint32_t)__double_as_longlong(v))
+                     << (BITS - 53);
   // a zero or subnormal has exponent field 0, at least 70 below top: shifted out
   const int64_t X = (int64_t)(m >> min(top - (int)((hi >> 20) & 0x7FFu), 63));
   return (int)hi < 0 ? -X : X;
 }
-__device__ __forceinline__ double sum_value(int64_t S, int top) { return f64_of_units(S, top - kSumBits + 63); }
+template <int BITS = kSumBits>
+__device__ __forceinline__ double sum_value(int64_t S, int top) {
+  return f64_of_units(S, top - BITS + 63);
+}
 
 // Largest exponent spread handled exactly: significands < 2^58, at most 6 neighbours plus M <= 9
 // times the centre keep |S| < 2^62.

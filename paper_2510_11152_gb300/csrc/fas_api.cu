@@ -72,6 +72,7 @@ constexpr int64_t kSwitchCells3D = 4096;
 constexpr size_t kCoarseSmemMax = 200 * 1024;    // field arrays of the single-CTA kernel
 constexpr size_t kCoarseSmemLimit = 227 * 1024;  // with its level descriptors (per-CTA maximum)
 constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smoothed by the fused sweep
+constexpr int64_t kIr4MinCells3D = (int64_t)1 << 21;
 constexpr int64_t kCol3dMinCells = (int64_t)1 << 21;  // smallest 3D level of the column-streaming kernels
 constexpr int64_t kFusedMinCells2D = (int64_t)1 << 20;  // smallest 2D level below the finest run fused
 
@@ -648,6 +649,12 @@ template <typename T, int DIM>
 void launch_residual(fas_ctx* c, const LevelDesc<T>& L, int level, T* r, const T* u, const T* f, const NormEnd& E) {
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
   Prof pr(c, FAS_K_RESIDUAL, level, (double)n);
+  if constexpr (std::is_same<T, double>::value) {
+    if (c->p.path != 1 && !L.varkappa && L.nx % 4 == 0) {
+      k_residual4<DIM, false><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r, u, f, L, E);
+      return;
+    }
+  }
   k_residual<T, DIM><<<grid_for(c, n), kBlock, 0, c->stream>>>(r, u, f, L, E);
 }
 
@@ -891,10 +898,17 @@ void launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b
   const LevelDesc<double>& L = c->h64.desc[0];
   const int64_t n = c->shape[0].cells();
   Prof pr(c, FAS_K_IR, 0, (double)n);
-  if (ir_strip_supported(L) &&
+  const bool group = c->p.path != 1 && !L.varkappa && L.nx % 4 == 0;
+  if (group && c->p.dim == 3 && n >= kIr4MinCells3D)
+    k_residual4<3, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
+  else if (ir_strip_supported(L) &&
       launch_ir_strip(r32, u, b, L, E, c->ir_ticket, c->sm_count, c->max_blocks, c->stream,
                       Ir3Wait{g_wait_limit_ns.load(), take_withhold(1)}) == cudaSuccess)
     ;  // the strip kernels took the level
+  else if (group && c->p.dim == 2)
+    k_residual4<2, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
+  else if (group)
+    k_residual4<3, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
   else if (c->p.dim == 2)
     k_ir_residual<2><<<grid_for(c, n), kBlock, 0, c->stream>>>(r32, u, b, L, E);
   else
