@@ -69,6 +69,8 @@ constexpr int64_t kSwitchCells2D = 16384;  // levels at or below this size run i
 constexpr int64_t kSwitchCells2DLarge = 4096;  // the same on 2D grids of at least kLargeGrid2D cells
 constexpr int64_t kLargeGrid2D = (int64_t)1 << 24;
 constexpr int64_t kSwitchCells3D = 4096;
+constexpr int64_t kSwitchCells2DF64 = 1024;
+constexpr int64_t kSwitchCells3DF64 = 512;
 constexpr size_t kCoarseSmemMax = 200 * 1024;    // field arrays of the single-CTA kernel
 constexpr size_t kCoarseSmemLimit = 227 * 1024;  // with its level descriptors (per-CTA maximum)
 constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smoothed by the fused sweep
@@ -300,8 +302,13 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
   // per-operation launches across the GPU (8192^2: 118.1 -> 116.1 ms per 20-step run with the switch
   // at 64^2); smaller grids, often solved side by side in a batch, keep the switch at 128^2 (the
   // 96-problem batch was 2 % slower with 64^2).
-  const int64_t sw_cells =
-      p.dim == 2 ? (c->shape[0].cells() >= kLargeGrid2D ? kSwitchCells2DLarge : kSwitchCells2D) : kSwitchCells3D;
+  // In float64 one SM's FP64 pipe bounds the kernel and the switch is lower (levels that the register-tile
+  // kernels do not take): 512^2 adjoint 42.4 ms with 64^2, 38.5 with 32^2, 40.8 with 16^2; 128^3 cavity step
+  // 10.46 ms with 16^3, 10.15 with 8^3, 10.40 with 4^3.
+  const int64_t sw_cells = sizeof(T) == 8   ? (p.dim == 2 ? kSwitchCells2DF64 : kSwitchCells3DF64)
+                           : p.dim != 2     ? kSwitchCells3D
+                           : c->shape[0].cells() >= kLargeGrid2D ? kSwitchCells2DLarge
+                                                                 : kSwitchCells2D;
   H.switch_level = c->nlev - 1;
   for (int l = 0; l < c->nlev; ++l) {
     if (c->shape[l].cells() > sw_cells) continue;
@@ -418,13 +425,14 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       if (l > 0) STATUS_TRY(dev_alloc(H, &H.u0[l], n));
     }
     // register-tile path: 2D cell levels of either precision whose coarsest levels fit the single-block
-    // tile kernel (at most 64 x 64 cells)
+    // tile kernel
     H.tiled = false;
     H.ntile = 0;
     if (p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL && p.nu1 >= 1 && p.nu1 <= kTileMaxNu &&
         p.nu2 >= 1 && p.nu2 <= kTileMaxNu) {
       int lc = 0;
-      while (lc < c->nlev && (c->shape[lc].nx > kTileCoarseCells || c->shape[lc].ny > kTileCoarseCells)) ++lc;
+      const int most = tile_coarse_cells<T>();
+      while (lc < c->nlev && (c->shape[lc].nx > most || c->shape[lc].ny > most)) ++lc;
       H.tiled = lc < c->nlev;
       H.ntile = H.tiled ? lc : 0;
     }

@@ -80,8 +80,8 @@ __device__ __forceinline__ int64_t mul_frac(int64_t N, Frac a) {
   const int nh = (int)(N >> 32);
   const uint32_t nl = (uint32_t)N;
   // |nh lo| <= 2^62 and nl hi < 2^62 (a <= 1/4): the sum of the middle products does not overflow
-  const int64_t half = (int64_t)(a.lo >> 1) + (1ll << 31);
-  const int64_t mid = (int64_t)nh * a.lo + (int64_t)((uint64_t)nl * (uint32_t)a.hi + (uint64_t)half);
+  const uint32_t half = (uint32_t)(a.lo >> 1) + 0x80000000u;  // |lo >> 1| <= 2^30: positive
+  const int64_t mid = (int64_t)nh * a.lo + (int64_t)((uint64_t)nl * (uint32_t)a.hi + half);
   return (int64_t)nh * a.hi + (mid >> 32);
 }
 
@@ -144,7 +144,7 @@ struct RawF {
   const LevelDesc<float>& L;
   __device__ __forceinline__ A coef(int cls) const { return A{L.a[cls], L.b[cls]}; }
   __device__ __forceinline__ V in(float x) const { return x; }
-  __device__ __forceinline__ V in_f(float x, int, bool) const { return x; }
+  __device__ __forceinline__ V in_f(float x, int, bool, bool) const { return x; }
   __device__ __forceinline__ float out(V x) const { return x; }
   __device__ __forceinline__ V update(V nb, V f, A c) const { return fmaf(c.a, nb, c.b * f); }
   __device__ __forceinline__ V tau(V f, V u, V nb, A, int cls) const { return f + fmaf(L.d[cls], u, -L.c * nb); }
@@ -164,7 +164,7 @@ struct ScaledD {
   const LevelDesc<double>& L;
   __device__ __forceinline__ A coef(int cls) const { return A{L.a[cls]}; }
   __device__ __forceinline__ V in(double x) const { return x; }
-  __device__ __forceinline__ V in_f(double x, int cls, bool scaled) const { return scaled ? x : L.b[cls] * x; }
+  __device__ __forceinline__ V in_f(double x, int cls, bool, bool scaled) const { return scaled ? x : L.b[cls] * x; }
   __device__ __forceinline__ double out(V x) const { return x; }
   __device__ __forceinline__ V update(V nb, V f, A c) const { return fma(c.a, nb, f); }
   __device__ __forceinline__ V tau(V f, V u, V nb, A c, int) const { return f + fma(-c.a, nb, u); }
@@ -188,13 +188,13 @@ struct ScaledX {
   using A = Frac;
   const LevelDesc<double>& L;
   Scale s;
-  Mant b0;  // interior b
+  Mant be, bo;  // b of the thread's even and odd column away from the y boundaries
   __device__ __forceinline__ A coef(int cls) const { return INNER ? frac_of(L.a[cls], L.alo[cls]) : frac_of(0.5 * L.a[cls], L.alo[cls] >> 1); }
   __device__ __forceinline__ V times(V nb, A c) const { return mul_frac(INNER ? nb : nb + nb, c); }
   __device__ __forceinline__ V in(double x) const { return to_fixed(x, s); }
-  __device__ __forceinline__ V in_f(double x, int cls, bool scaled) const {
+  __device__ __forceinline__ V in_f(double x, int cls, bool odd, bool scaled) const {
     if (scaled) return to_fixed(x, s);
-    return to_fixed_mul(x, cls ? mant_of(L.b[cls]) : b0, s);
+    return to_fixed_mul(x, !INNER && (cls & 12) ? mant_of(L.b[cls]) : (!INNER && odd ? bo : be), s);
   }
   __device__ __forceinline__ double out(V x) const { return from_fixed(x, s); }
   __device__ __forceinline__ V update(V nb, V f, A c) const { return times(nb, c) + f; }
@@ -203,9 +203,12 @@ struct ScaledX {
   __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return (((a + b) + (c + d)) + 2) >> 2; }
   __device__ __forceinline__ double out_avg(V a, V b, V c, V d) const { return from_fixed((a + b) + (c + d), s, 2); }
   __device__ __forceinline__ double out_avg_r(V a, V b, V c, V d, int ca, int cb, int cc, int cd) const {
-    if ((ca | cb | cc | cd) == 0) return L.d[0] * from_fixed((a + b) + (c + d), s, 2);
-    return ((L.d[ca] * from_fixed(a, s) + L.d[cb] * from_fixed(b, s)) +
-            (L.d[cc] * from_fixed(c, s) + L.d[cd] * from_fixed(d, s))) * 0.25;
+    // d = alpha + c M: the interior's d times the sum, and c times the sum weighted by how far M is off there
+    const double r = L.d[0] * from_fixed((a + b) + (c + d), s, 2);
+    if (INNER || (ca | cb | cc | cd) == 0) return r;
+    const int m0 = L.mt[0];
+    const V wsum = (a * (L.mt[ca] - m0) + b * (L.mt[cb] - m0)) + (c * (L.mt[cc] - m0) + d * (L.mt[cd] - m0));
+    return fma(L.c, from_fixed(wsum, s, 2), r);
   }
   __device__ __forceinline__ float norm_factor(int cls, float ns) const {
     return (float)(L.d[cls] * from_fixed(1, s) * (double)ns);
@@ -235,7 +238,7 @@ struct Place {
   int srcW, srcE; // lanes of the west / east neighbour pair
   bool noW, noE;  // no such lane (the region's edge is the domain's, or nothing is needed there)
   bool active;    // the warp has rows of the domain (always true where regions have halos)
-  int wu, wd;     // warps whose edge rows lie above / below this one's rows (-1: none)
+  int wu, wd;     // warps whose edge rows lie above / below this one's rows (one past the last warp: zeros)
   int bar;        // threads that meet at a phase's barrier (0: the whole block)
   __device__ __forceinline__ bool row_in(int r) const { return (unsigned)(y + r) < (unsigned)ny; }
   __device__ __forceinline__ int yf(int r) const { return ((y + r == 0) << 2) | ((y + r == ny - 1) << 3); }
@@ -267,15 +270,17 @@ struct Region {
     if (INNER) {
       co[0][0] = p.coef(0);
     } else {
-      const A e0 = p.coef(pl.xfe), o0 = p.coef(pl.xfo);
+      // cells outside the domain get coefficients 0: with f = 0 their value then stays 0
+      const A none{}, e0 = pl.col_in ? p.coef(pl.xfe) : none, o0 = pl.col_in ? p.coef(pl.xfo) : none;
 #pragma unroll
       for (int r = 0; r < (INNER ? 1 : R); ++r) {
         A e = e0, o = o0;
         const int yf = pl.yf(r);
-        if (yf) {  // the same for the whole warp
+        if (yf && pl.col_in) {  // yf: the same for the whole warp
           e = p.coef(pl.xfe | yf);
           o = p.coef(pl.xfo | yf);
         }
+        if (!pl.row_in(r)) e = o = none;
         co[r][0] = odd(r) ? o : e;
         co[r][1] = odd(r) ? e : o;
       }
@@ -295,7 +300,7 @@ struct Region {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       u[r][k] = pol.in(uw[odd_col(r, k)]);
-      f[r][k] = pol.in_f(fw[odd_col(r, k)], cls(r, k), scaled);
+      f[r][k] = pol.in_f(fw[odd_col(r, k)], cls(r, k), odd_col(r, k), scaled);
     }
   }
   // the (even, odd) column of row r of x
@@ -308,11 +313,11 @@ struct Region {
   }
   __device__ __forceinline__ V above(int r, int k) const {  // row r - 1
     if (r > 0) return u[r > 0 ? r - 1 : 0][k];
-    return g.wu >= 0 ? edge[g.wu].v[1][k][lane] : V(0);
+    return edge[g.wu].v[1][k][lane];
   }
   __device__ __forceinline__ V below(int r, int k) const {  // row r + 1
     if (r < R - 1) return u[r < R - 1 ? r + 1 : 0][k];
-    return g.wd >= 0 ? edge[g.wd].v[0][k][lane] : V(0);
+    return edge[g.wd].v[0][k][lane];
   }
   // sum of the existing neighbours of cell (r, k): (west + east) + (row - 1 + row + 1)
   __device__ __forceinline__ V nbsum(int r, int k) const {
@@ -336,8 +341,7 @@ struct Region {
   __device__ __forceinline__ void phase() {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const V val = pol.update(nbsum(r, K), f[r][K], coef(r, K));
-      if (INNER || (g.col_in && g.row_in(r))) u[r][K] = val;
+      u[r][K] = pol.update(nbsum(r, K), f[r][K], coef(r, K));
     }
     publish(K);
     meet();
@@ -419,7 +423,7 @@ struct TileArgs {
 
 template <typename T, int NW>
 struct TileSmem {
-  typename std::conditional<sizeof(T) == 4, Edge<float>, Edge<int64_t>>::type edge[NW];
+  typename std::conditional<sizeof(T) == 4, Edge<float>, Edge<int64_t>>::type edge[NW + 1];
   int wmax[NW];
 };
 
@@ -447,8 +451,8 @@ __device__ __forceinline__ Place tile_place(int nx, int ny, int per, int halo, b
   g.noE = lane == 31;
   g.active = true;
   g.bar = 0;
-  g.wu = warp - 1;
-  g.wd = warp + 1 < NW ? warp + 1 : -1;
+  g.wu = warp > 0 ? warp - 1 : NW;
+  g.wd = warp + 1;
   *inner = (px || (rx0 >= 2 && rx0 + kTileCols <= nx - 2)) && (py || (ry0 >= 2 && ry0 + R * NW <= ny - 2));
   return g;
 }
@@ -612,6 +616,7 @@ __global__ void __launch_bounds__(32 * NW) k_tile_pre(const __grid_constant__ Ti
                                                       const __grid_constant__ LevelDesc<T> L) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
   auto& sm = *reinterpret_cast<TileSmem<T, NW>*>(tile_smem);
+  if (threadIdx.x < 128) reinterpret_cast<T*>(&sm.edge[NW])[threadIdx.x] = T(0);
   bool inner;
   const Place g = tile_place<R, NW>(L.nx, L.ny, L.per, a.halo, &inner);
   const RowMap rm{L.ny, (L.per & 2) != 0};
@@ -629,9 +634,9 @@ __global__ void __launch_bounds__(32 * NW) k_tile_pre(const __grid_constant__ Ti
     const Mant b0 = mant_of(L.b[0]);
     if (choose_scale(raw_exp<false>(w, b0.E + 1, false), a.bits, sm.wmax, NW, &s)) {
       if (inner)
-        pre_run<TAU, true>(ScaledX<true>{L, s, b0}, a, g, rm, sm, w, rows);
+        pre_run<TAU, true>(ScaledX<true>{L, s, b0, b0}, a, g, rm, sm, w, rows);
       else
-        pre_run<TAU, false>(ScaledX<false>{L, s, b0}, a, g, rm, sm, w, rows);
+        pre_run<TAU, false>(ScaledX<false>{L, s, mant_of(L.b[g.xfe]), mant_of(L.b[g.xfo])}, a, g, rm, sm, w, rows);
     } else {
       pre_run<TAU, false>(ScaledD{L}, a, g, rm, sm, w, rows);
     }
@@ -643,6 +648,7 @@ __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ T
                                                        const __grid_constant__ LevelDesc<T> L) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
   auto& sm = *reinterpret_cast<TileSmem<T, NW>*>(tile_smem);
+  if (threadIdx.x < 128) reinterpret_cast<T*>(&sm.edge[NW])[threadIdx.x] = T(0);
   bool inner;
   const Place g = tile_place<R, NW>(L.nx, L.ny, L.per, a.halo, &inner);
   const RowMap rm{L.ny, (L.per & 2) != 0};
@@ -661,9 +667,9 @@ __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ T
     const Mant b0 = mant_of(L.b[0]);
     if (choose_scale(raw_exp<true>(w, b0.E + 1, a.scaled), a.bits, sm.wmax, NW, &s)) {
       if (inner)
-        acc = post_run<RES, true>(ScaledX<true>{L, s, b0}, a, g, rm, sm, w, rows);
+        acc = post_run<RES, true>(ScaledX<true>{L, s, b0, b0}, a, g, rm, sm, w, rows);
       else
-        acc = post_run<RES, false>(ScaledX<false>{L, s, b0}, a, g, rm, sm, w, rows);
+        acc = post_run<RES, false>(ScaledX<false>{L, s, mant_of(L.b[g.xfe]), mant_of(L.b[g.xfo])}, a, g, rm, sm, w, rows);
     } else {
       acc = post_run<RES, false>(ScaledD{L}, a, g, rm, sm, w, rows);
     }
@@ -673,18 +679,20 @@ __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ T
 }
 
 // ------------------------------------------------------------------------------------------------
-// levels of at most 64 x 64 cells: a V-cycle in one block
+// levels of at most 64 x 64 (float64: 32 x 32) cells: a V-cycle in one block
 // ------------------------------------------------------------------------------------------------
 
 constexpr int kCoarseR = 2;  // rows per warp: the pass over a level is one warp's chain of instructions
-constexpr int kCoarseWarps = kTileCoarseCells / kCoarseR;
+template <typename T>
+constexpr int kCoarseWarps = tile_coarse_cells<T>() / kCoarseR;
 
 template <typename T>
 struct CoarseSmem {
-  typename std::conditional<sizeof(T) == 4, Edge<float>, Edge<int64_t>>::type edge[kCoarseWarps];
-  int wmax[kCoarseWarps];
+  typename std::conditional<sizeof(T) == 4, Edge<float>, Edge<int64_t>>::type edge[kCoarseWarps<T> + 1];
+  int wmax[kCoarseWarps<T>];
 };
 
+template <typename T>
 __device__ __forceinline__ Place coarse_place(int nx, int ny, int per) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool px = per & 1, py = per & 2;
@@ -703,8 +711,8 @@ __device__ __forceinline__ Place coarse_place(int nx, int ny, int per) {
   g.srcE = (lane + 1) & (np - 1);
   g.noW = !px && lane == 0;
   g.noE = !px && lane == np - 1;
-  g.wu = warp > 0 ? warp - 1 : (py ? nwa - 1 : -1);
-  g.wd = warp + 1 < nwa ? warp + 1 : (py ? 0 : -1);
+  g.wu = warp > 0 ? warp - 1 : (py ? nwa - 1 : kCoarseWarps<T>);
+  g.wd = warp + 1 < nwa ? warp + 1 : (py ? 0 : kCoarseWarps<T>);
   return g;
 }
 
@@ -785,17 +793,17 @@ template <Pass PASS, typename T, typename SM>
 __device__ __forceinline__ void coarse_step(const LevelDesc<T>& L, SM& sm, const TileCoarse<T>& A, const T* u,
                                             const T* f, const T* c, bool tau, bool scaled, int nu, T* su, T* sf, T* cu,
                                             T* cf) {
-  const Place g = coarse_place(L.nx, L.ny, L.per);
+  const Place g = coarse_place<T>(L.nx, L.ny, L.per);
   Raw<T, kCoarseR> w;
   coarse_load(w, g, u, f, c);
   if constexpr (sizeof(T) == 4) {
     if (g.active) coarse_level<PASS>(RawF{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
   } else {
     Scale s;
-    const Mant b0 = mant_of(L.b[0]);
-    if (choose_scale(raw_exp<PASS == Pass::kUp>(w, b0.E + 1, scaled), A.bits, sm.wmax, kCoarseWarps, &s)) {
+    const Mant be = mant_of(L.b[g.xfe]), bo = mant_of(L.b[g.xfo]);
+    if (choose_scale(raw_exp<PASS == Pass::kUp>(w, max(be.E, bo.E) + 1, scaled), A.bits, sm.wmax, kCoarseWarps<T>, &s)) {
       if (g.active)
-        coarse_level<PASS>(ScaledX<false>{L, s, b0}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+        coarse_level<PASS>(ScaledX<false>{L, s, be, bo}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
     } else if (g.active) {
       coarse_level<PASS>(ScaledD{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
     }
@@ -804,10 +812,11 @@ __device__ __forceinline__ void coarse_step(const LevelDesc<T>& L, SM& sm, const
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kCoarseWarps) k_tile_coarse(const __grid_constant__ TileCoarse<T> A, T* utop,
-                                                                   const T* ftop) {
+__global__ void __launch_bounds__(32 * kCoarseWarps<T>) k_tile_coarse(const __grid_constant__ TileCoarse<T> A, T* utop,
+                                                                      const T* ftop) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
   auto& sm = *reinterpret_cast<CoarseSmem<T>*>(tile_smem);
+  if (threadIdx.x < 128) reinterpret_cast<T*>(&sm.edge[kCoarseWarps<T>])[threadIdx.x] = T(0);
   T* fields = reinterpret_cast<T*>(tile_smem + (sizeof(CoarseSmem<T>) + 15) / 16 * 16);
   LevelDesc<T>* desc = reinterpret_cast<LevelDesc<T>*>(fields + A.total) - A.l0;
   {
@@ -818,6 +827,7 @@ __global__ void __launch_bounds__(32 * kCoarseWarps) k_tile_coarse(const __grid_
   }
   __syncthreads();
   const int last = A.nlev - 1;
+  // U(l), F(l): levels l0 .. last only (F reads the level's descriptor)
   auto U = [&](int l) { return fields + A.off[l]; };
   auto F = [&](int l) { return fields + A.off[l] + (desc[l].nx * desc[l].ny + 3) / 4 * 4; };
   for (int l = A.l0; l < last; ++l) {
@@ -982,7 +992,7 @@ size_t coarse_bytes(const TileCoarse<T>& A) {
 
 template <typename T>
 cudaError_t launch_tile_coarse(const TileCoarse<T>& A, T* utop, const T* ftop, cudaStream_t stream) {
-  k_tile_coarse<T><<<1, 32 * kCoarseWarps, coarse_bytes(A), stream>>>(A, utop, ftop);
+  k_tile_coarse<T><<<1, 32 * kCoarseWarps<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
   return cudaGetLastError();
 }
 
