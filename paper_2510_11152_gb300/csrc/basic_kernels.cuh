@@ -350,7 +350,7 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
 #pragma unroll
         for (int q = 0; q < 2; ++q)
           top = max(top, max(max(exp_field(sv[q]), exp_field(nv[q])), max(exp_field(bo[q]), exp_field(to[q]))));
-        if (sum_range_ok(top)) {
+        if (sum_range(top)) {
           const int64_t m = sum_units(x1v, top);
 #pragma unroll
           for (int q = 0; q < 2; ++q)
@@ -382,8 +382,10 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
   }
 }
 
+// At least three blocks per SM: the float64 3D phase waits for its rows from L2, and with two blocks (94 registers) too
+// few are in flight (256 x 128 x 64 heat run: 8.03 -> 7.44 ms; four blocks spill: 7.95).
 template <typename T, int DIM>
-__global__ void k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
+__global__ void __launch_bounds__(256, 3) k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
   if (L.per)
     smooth_colour4_body<T, DIM, true>(u, f, L, colour);
   else
@@ -651,7 +653,7 @@ struct Group4 {
 // About 90 (2D) and 110 (3D) instructions per cell; a thread per cell with its own conversions took 250, the 3D
 // plane-streaming kernel (ir_strip.cu) 247.
 template <int DIM, bool IR>
-__global__ void __launch_bounds__(256) k_residual4(typename std::conditional<IR, float, double>::type* r, const double* u,
+__global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<IR, float, double>::type* r, const double* u,
                                                    const double* f, const __grid_constant__ LevelDesc<double> L,
                                                    const __grid_constant__ NormEnd E) {
   constexpr int BITS = DIM == 2 ? 59 : 58;  // |S| <= (2 DIM + M) 2^BITS < 2^63, M <= 4 DIM
@@ -670,9 +672,9 @@ __global__ void __launch_bounds__(256) k_residual4(typename std::conditional<IR,
     q.load(u, idx, x0, j, l, L);
     Quad<double> fq;
     fq.ld(f + idx);
-    const int top = q.top();
+    int top = q.top();
     double rv[4];
-    if (sum_range_ok(top)) {
+    if (sum_range(top)) {
       int64_t C[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) C[k] = sum_units<BITS>(q.c.v[k], top);

@@ -160,7 +160,12 @@ __device__ __forceinline__ double f64_of_units(int64_t X, int base) {
 // values within 2^7 of the largest; the unit is 2^-60 of it, where a float64 addition rounds at 2^-53 of its
 // result's magnitude). Up to six such values add up without overflow; the sum is rounded once.
 constexpr int kSumBits = 60;
-__device__ __forceinline__ bool sum_range_ok(int top) { return (unsigned)(top - 70) <= 1970u; }
+// Scale of a sum from the values' largest biased exponent: all zeros take any; false (float64 additions instead) near
+// the ends of the float64 range and for infinities and NaN.
+__device__ __forceinline__ bool sum_range(int& top) {
+  if (top == 0) top = 70;
+  return (unsigned)(top - 70) <= 1970u;
+}
 template <int BITS = kSumBits>
 __device__ __forceinline__ int64_t sum_units(double v, int top) {
   const uint32_t hi = (uint32_t)((uint64_t)__double_as_longlong(v) >> 32);

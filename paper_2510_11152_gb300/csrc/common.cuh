@@ -71,9 +71,9 @@ __device__ __forceinline__ bool frozen(const LevelDesc<T>& L, int i, int j, int 
 template <typename T>
 __device__ __forceinline__ T sum6(T w, T e, T s, T n, T bo, T to) {
   if constexpr (std::is_same<T, double>::value) {
-    const int top = max(max(max(exp_field(w), exp_field(e)), max(exp_field(s), exp_field(n))),
+    int top = max(max(max(exp_field(w), exp_field(e)), max(exp_field(s), exp_field(n))),
                         max(exp_field(bo), exp_field(to)));
-    if (sum_range_ok(top))
+    if (sum_range(top))
       return sum_value((sum_units(w, top) + sum_units(e, top)) + (sum_units(s, top) + sum_units(n, top)) +
                            (sum_units(bo, top) + sum_units(to, top)),
                        top);

@@ -74,9 +74,18 @@ constexpr int64_t kSwitchCells3DF64 = 512;
 constexpr size_t kCoarseSmemMax = 200 * 1024;    // field arrays of the single-CTA kernel
 constexpr size_t kCoarseSmemLimit = 227 * 1024;  // with its level descriptors (per-CTA maximum)
 constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smoothed by the fused sweep
+// Refinement residual by groups of four cells (k_residual4) or by the strip kernels (ir_strip.cu). 2D: a strip
+// kernel's warp walks rows one after the other, and small grids leave it few warps (1024^2: 31 us against 18;
+// 2048^2: 45 against 42; 4096^2: 106 against 123; 8192^2: 351 against 428). 3D: the plane-streaming kernel takes 247
+// instructions per cell (512^3: 1.64 ms against 1.22) and keeps the small grids, where both are bound by latency.
+constexpr int64_t kIr4MaxCells2D = (int64_t)1 << 22;
 constexpr int64_t kIr4MinCells3D = (int64_t)1 << 21;
 constexpr int64_t kCol3dMinCells = (int64_t)1 << 21;  // smallest 3D level of the column-streaming kernels
-constexpr int64_t kFusedMinCells2D = (int64_t)1 << 20;  // smallest 2D level below the finest run fused
+// Smallest 2D level of the sweep-fused kernels: above the register-tile kernels (whose blocks recompute half again as
+// many cells; 4096^2 level of an 8192^2 run, pre-smoothing: 68 us against 89, 2048^2: 29 against 28, 1024^2: 18
+// against 8), and in hierarchies that those do not take.
+constexpr int64_t kFusedMinCells2D = (int64_t)1 << 22;
+constexpr int64_t kFusedMinCells2DUntiled = (int64_t)1 << 20;
 
 int grid_for(const fas_ctx* c, int64_t work) {
   int64_t g = (work + kBlock - 1) / kBlock;
@@ -441,12 +450,13 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
     H.nfast = 0;
     if (sizeof(T) == 4 && p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL &&
         p.ordering == FAS_ORDER_FORWARD && p.nu1 >= 1 && p.nu2 >= 1 && periodic_mask(p) == 0) {
-      // below 2^20 cells a level's fused kernels are latency-bound (one warp streams a long segment of
-      // rows) and the register-tile kernels take it; where those do not apply (narrow hierarchies) the
-      // finest level stays fused for its float64 update and the others run per operation
+      // below that a level's fused kernels are latency-bound (one warp streams a long segment of rows) and
+      // the register-tile kernels take it; where those do not apply (narrow hierarchies) the finest level
+      // stays fused for its float64 update and the others run per operation
+      const int64_t fused_min = H.tiled ? kFusedMinCells2D : kFusedMinCells2DUntiled;
       while (H.nfast < H.switch_level &&
              stream2d_supported(c->shape[H.nfast].nx, c->shape[H.nfast].ny, std::max(p.nu1, p.nu2)) &&
-             ((H.nfast == 0 && !H.tiled) || c->shape[H.nfast].cells() >= kFusedMinCells2D || p.path == 2) &&
+             ((H.nfast == 0 && !H.tiled) || c->shape[H.nfast].cells() >= fused_min || p.path == 2) &&
              (!H.tiled || H.nfast < H.ntile))
         H.nfast++;
     }
@@ -907,7 +917,9 @@ void launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b
   const int64_t n = c->shape[0].cells();
   Prof pr(c, FAS_K_IR, 0, (double)n);
   const bool group = c->p.path != 1 && !L.varkappa && L.nx % 4 == 0;
-  if (group && c->p.dim == 3 && n >= kIr4MinCells3D)
+  if (group && c->p.dim == 2 && n <= kIr4MaxCells2D)
+    k_residual4<2, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
+  else if (group && c->p.dim == 3 && n >= kIr4MinCells3D)
     k_residual4<3, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
   else if (ir_strip_supported(L) &&
       launch_ir_strip(r32, u, b, L, E, c->ir_ticket, c->sm_count, c->max_blocks, c->stream,
