@@ -910,6 +910,63 @@ __global__ void k_restrict_resid(T* uc, T* uc0, T* fc, const T* u, const T* f, L
     restrict_resid_face_range<T, DIM, FAX>(uc, uc0, fc, u, f, L, gtid(), gstride());
 }
 
+// The same for 3D float64 levels with constant kappa, with the fine residuals of a coarse cell spread over the lanes of
+// a warp: 8 lanes on cells (one child each), 4 on faces (one tangential cell each, the three normal slots one
+// after the other). For small levels: one thread per coarse cell evaluates 8 or 12 residuals in a row, a chain that
+// took 12 to 15 us there (now 7).
+template <int FAX>
+__global__ void __launch_bounds__(256) k_restrict_resid_lanes(double* uc, double* uc0, double* fc, const double* u,
+                                                              const double* f, const __grid_constant__ LevelDesc<double> L) {
+  constexpr int LOG = FAX < 0 ? 3 : 2;
+  const int lxc = L.lx - 1, lyc = L.ly - 1, lzc = L.lz - 1;
+  const int nxc = 1 << lxc, nyc = 1 << lyc, nzc = 1 << lzc;
+  const int64_t sy = L.nx, sz = (int64_t)L.nx * L.ny;
+  const int64_t total = (int64_t)1 << (lxc + lyc + lzc + LOG);
+  // whole warps take part in the shuffles: the bound is rounded up, and lanes past the end repeat the last cell
+  for (int64_t t0 = gtid(); (t0 & ~(int64_t)31) < total; t0 += gstride()) {
+    const int64_t t = t0 < total ? t0 : total - 1;
+    const int64_t I = t >> LOG;
+    const int q = (int)(t & ((1 << LOG) - 1));
+    const int c3[3] = {(int)(I & (nxc - 1)), (int)((I >> lxc) & (nyc - 1)), (int)(I >> (lxc + lyc))};
+    double su = 0.0, sr = 0.0;
+    if constexpr (FAX < 0) {
+      const int i = 2 * c3[0] + (q & 1), j = 2 * c3[1] + ((q >> 1) & 1), l = 2 * c3[2] + (q >> 2);
+      const int64_t idx = (int64_t)l * sz + (int64_t)j * sy + i;
+      su = u[idx];
+      sr = L.per ? residual_point<double, 3, true>(u, f, L, idx, i, j, l)
+                 : residual_point<double, 3, false>(u, f, L, idx, i, j, l);
+    } else {
+      constexpr int T1 = FAX == 0 ? 1 : 0, T2 = FAX == 2 ? 1 : 2;
+      const bool wall = wall_slot<FAX>(c3[0], c3[1], c3[2], nxc, nyc, nzc);
+      if (!wall) {
+#pragma unroll 1
+        for (int w = 0; w < 3; ++w) {
+          int f3[3];
+          f3[FAX] = 2 * c3[FAX] + w;
+          f3[T1] = 2 * c3[T1] + (q & 1);
+          f3[T2] = 2 * c3[T2] + (q >> 1);
+          const int64_t idx = (int64_t)f3[2] * sz + (int64_t)f3[1] * sy + f3[0];
+          const double wt = w == 1 ? 0.5 : 0.25;
+          su = fma(wt, u[idx], su);
+          if (!frozen(L, f3[0], f3[1], f3[2]))
+            sr = fma(wt, residual_point<double, 3>(u, f, L, idx, f3[0], f3[1], f3[2]), sr);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < (1 << LOG); o <<= 1) {
+      su += __shfl_xor_sync(0xffffffffu, su, o);
+      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+    }
+    if (q == 0 && t0 < total) {
+      const double scale = FAX < 0 ? 0.125 : 0.25;
+      uc[I] = su * scale;
+      uc0[I] = su * scale;
+      fc[I] = sr * scale;
+    }
+  }
+}
+
 // 3D float32 cell levels with constant kappa, no periodic axis and a multiple of 4 cells per row: the
 // residual-restriction of k_restrict_resid with one thread per 4 x 2 x 2 block of fine cells (two
 // coarse cells), every row of the block and of its y and z neighbours read as one 16-byte vector.

@@ -80,6 +80,9 @@ constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smo
 // instructions per cell (512^3: 1.64 ms against 1.22) and keeps the small grids, where both are bound by latency.
 constexpr int64_t kIr4MaxCells2D = (int64_t)1 << 22;
 constexpr int64_t kIr4MinCells3D = (int64_t)1 << 21;
+// Largest 3D float64 level whose residual-restriction is spread over lanes (64 x 32 x 32: the same as one thread per coarse
+// cell; below 12 us -> 7, 256 x 128 x 64: 28 us -> 49, its reads being of 2 cells at a time).
+constexpr int64_t kLanesMaxCells3D = (int64_t)1 << 16;
 constexpr int64_t kCol3dMinCells = (int64_t)1 << 21;  // smallest 3D level of the column-streaming kernels
 // Smallest 2D level of the sweep-fused kernels: above the register-tile kernels (whose blocks recompute half again as
 // many cells; 4096^2 level of an 8192^2 run, pre-smoothing: 68 us against 89, 2048^2: 29 against 28, 1024^2: 18
@@ -668,7 +671,7 @@ void launch_residual(fas_ctx* c, const LevelDesc<T>& L, int level, T* r, const T
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
   Prof pr(c, FAS_K_RESIDUAL, level, (double)n);
   if constexpr (std::is_same<T, double>::value) {
-    if (c->p.path != 1 && !L.varkappa && L.nx % 4 == 0) {
+    if ((c->p.path != 1 || L.fax >= 0) && !L.varkappa && L.nx % 4 == 0) {
       k_residual4<DIM, false><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r, u, f, L, E);
       return;
     }
@@ -739,6 +742,17 @@ fas_status vcycle_basic_from(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T
           blocks = true;
         }
       }
+      if constexpr (std::is_same<T, double>::value && DIM == 3) {
+        if (!L.varkappa && n <= kLanesMaxCells3D) {
+          with_fax(c, [&](auto tag) {
+            constexpr int FAX = decltype(tag)::value;
+            constexpr int lanes = FAX < 0 ? 8 : 4;
+            k_restrict_resid_lanes<FAX><<<grid_for(c, nc * lanes), kBlock, 0, c->stream>>>(H.u[l + 1], H.u0[l + 1],
+                                                                                         H.f[l + 1], u, f, L);
+          });
+          blocks = true;
+        }
+      }
       if (!blocks) with_fax(c, [&](auto tag) {
         constexpr int FAX = decltype(tag)::value;
         k_restrict_resid<T, DIM, FAX><<<grid_for(c, nc), kBlock, 0, c->stream>>>(H.u[l + 1], H.u0[l + 1],
@@ -793,7 +807,7 @@ fas_status vcycle_tile(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T* ftop
     Prof pr(c, family(l, FAS_K_SMOOTH), l, (double)c->shape[l].cells());
     STATUS_TRY(tried(launch_tile_pre<T>(top ? (zero_init ? nullptr : utop) : H.u[l], top ? ftop : H.rc[l],
                                         t ? H.f[l] : nullptr, H.u2[l], H.u[l + 1], l + 1 < lc ? H.rc[l + 1] : H.f[l + 1],
-                                        H.desc[l], p.nu1, p.ordering, t, H.tile_bits[l], c->sm_count, c->stream),
+                                        H.desc[l], p.nu1, p.ordering, t, H.tile_bits[l], p.seg_rows, c->sm_count, c->stream),
                      "tile pre"));
   }
   {
@@ -809,14 +823,14 @@ fas_status vcycle_tile(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T* ftop
     if constexpr (std::is_same<T, double>::value) {
       if (top && norm) {
         STATUS_TRY(tried(launch_tile_post_norm(H.u2[l], ftop, H.u[l + 1], utop, H.desc[l], p.nu2, p.ordering,
-                                               H.tile_bits[l], *norm, c->sm_count, c->stream),
+                                               H.tile_bits[l], *norm, p.seg_rows, c->sm_count, c->stream),
                          "tile post"));
         continue;
       }
     }
     STATUS_TRY(tried(launch_tile_post<T>(H.u2[l], t ? H.f[l] : ftop, H.u[l + 1], top ? utop : H.u[l],
                                          l == 0 ? u64 : nullptr, H.desc[l], p.nu2, p.ordering,
-                                         t && sizeof(T) == 8, H.tile_bits[l], c->sm_count, c->stream),
+                                         t && sizeof(T) == 8, H.tile_bits[l], p.seg_rows, c->sm_count, c->stream),
                      "tile post"));
   }
   return FAS_OK;
@@ -916,7 +930,7 @@ void launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b
   const LevelDesc<double>& L = c->h64.desc[0];
   const int64_t n = c->shape[0].cells();
   Prof pr(c, FAS_K_IR, 0, (double)n);
-  const bool group = c->p.path != 1 && !L.varkappa && L.nx % 4 == 0;
+  const bool group = !L.varkappa && L.nx % 4 == 0;  // on every path: r32 does not depend on it
   if (group && c->p.dim == 2 && n <= kIr4MaxCells2D)
     k_residual4<2, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
   else if (group && c->p.dim == 3 && n >= kIr4MinCells3D)
@@ -942,8 +956,8 @@ void enqueue_residual_norm(fas_ctx* c, const double* u, const double* b, const N
     launch_ir_residual(c, c->h32.f[0], u, b, E);
   } else if (H.tiled && H.ntile > 0) {
     Prof pr(c, FAS_K_RESIDUAL, 0, (double)c->shape[0].cells());
-    launch_tile_post_norm(u, b, nullptr, nullptr, H.desc[0], 0, c->p.ordering, H.tile_bits[0], E, c->sm_count,
-                          c->stream);
+    launch_tile_post_norm(u, b, nullptr, nullptr, H.desc[0], 0, c->p.ordering, H.tile_bits[0], E, c->p.seg_rows,
+                          c->sm_count, c->stream);
   } else if (c->p.dim == 2)
     launch_residual<double, 2>(c, c->h64.desc[0], 0, nullptr, u, b, E);
   else
@@ -1612,7 +1626,7 @@ fas_status fas_create(const fas_params* pin, void* stream, fas_ctx** out) {
   };
   int64_t nparts = c->max_blocks;
   if (p.dim == 2 && p.nu2 >= 1 && p.nu2 <= kTileMaxNu)
-    nparts = std::max<int64_t>(nparts, tile_norm_blocks(c->shape[0].nx, c->shape[0].ny, p.nu2, c->sm_count));
+    nparts = std::max<int64_t>(nparts, tile_norm_blocks(c->shape[0].nx, c->shape[0].ny, p.nu2));
   if (cudaMalloc(&c->partials, nparts * sizeof(double)) != cudaSuccess) return bail(fail(FAS_ENOMEM, "partials"));
   if (cudaMalloc(&c->d_scalar, 8 * sizeof(double)) != cudaSuccess) return bail(fail(FAS_ENOMEM, "scalars"));
   if (cudaMalloc(&c->ir_ticket, 4 * sizeof(unsigned)) != cudaSuccess ||
@@ -1937,7 +1951,7 @@ fas_status fas_autotune(fas_ctx* c, double* u, const double* f, fas_tune_result*
       }
   }
   const bool mixed = c->p.precision == FAS_MIXED;
-  const bool fused = mixed && c->h32.nfast > 0;
+  const bool fused = mixed && (c->h32.nfast > 0 || c->h32.ntile > 0);
   const int inners[3] = {1, 2, 3};
   const int segs[5] = {0, 16, 32, 64, 128};
   const int n_inner = mixed ? 3 : 1, n_seg = fused ? 5 : 1;

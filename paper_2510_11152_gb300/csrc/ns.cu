@@ -62,16 +62,16 @@ __device__ __forceinline__ void ns_coords(const NsGrid& G, int64_t idx, int* k) 
 // component is continued oddly, face -k = -face k and face n+k = -face n-k. `line` is the linear
 // index of slot 0 on the line through the point.
 __device__ __forceinline__ double normal_value(const double* __restrict__ phi, int64_t line, int64_t st, int n, int F) {
-  double sgn = 1.0;
+  bool flip = false;
   if (F < 0) {
     F = -F;
-    sgn = -1.0;
+    flip = true;
   } else if (F > n) {
     F = 2 * n - F;
-    sgn = -1.0;
+    flip = true;
   }
   const double v = F == 0 ? 0.0 : phi[line + (int64_t)(F - 1) * st];
-  return sgn * v;
+  return flip ? -v : v;  // a select, not a multiplication on the FP64 pipe
 }
 
 // Value of a component along a tangential axis at cell c (up to two cells beyond either wall): a
@@ -83,20 +83,18 @@ __device__ __forceinline__ double tangential_value(const double* __restrict__ ph
   return phi[line + (int64_t)c * st];
 }
 
-// Third-order WENO of Jiang and Shu for a derivative from three consecutive first differences, the
-// upwind one first: the two candidate slopes (3b - a)/2 and (b + c)/2 weighted by the ideal weights
-// 1/3 and 2/3 over the square of eps + their smoothness (b - a)^2, (c - b)^2. With the weights
-// alpha_k = d_k / q_k^2 brought to the common denominator 3 q0^2 q1^2 the combination is
-// (q1^2 p0 + 2 q0^2 p1) / (q1^2 + 2 q0^2): one division instead of three (float64 division is a long
-// sequence on the FP64 pipe).
-__device__ __forceinline__ double weno3(double a, double b, double c) {
-  const double p0 = 0.5 * (3.0 * b - a);
-  const double p1 = 0.5 * (b + c);
-  const double b0 = (b - a) * (b - a);
-  const double b1 = (c - b) * (c - b);
-  const double q0 = kWenoEps + b0, q1 = kWenoEps + b1;
-  const double w0 = q1 * q1, w1 = 2.0 * (q0 * q0);
-  return (w0 * p0 + w1 * p1) / (w0 + w1);
+// Third-order WENO of Jiang and Shu for a derivative from three consecutive differences, the upwind one first:
+// the two candidate slopes (3b - a)/2 and (b + c)/2 weighted by the ideal weights 1/3 and 2/3 over the
+// square of eps + their smoothness (b - a)^2, (c - b)^2. With the weights alpha_k = d_k / q_k^2 brought to the
+// common denominator 3 q0^2 q1^2 and both candidates written from b, the combination is
+//     b + (q1^2 (b - a) + 2 q0^2 (c - b)) / (2 (q1^2 + 2 q0^2)):
+// one division instead of three. The weights do not change when all differences and sqrt(eps) are scaled, so the
+// differences stay undivided (eps h^2 for eps), and the derivative is this value over h.
+__device__ __forceinline__ double weno3(double a, double b, double c, double eps) {
+  const double da = b - a, dc = c - b;
+  const double q0 = fma(da, da, eps), q1 = fma(dc, dc, eps);
+  const double w0 = q1 * q1, w1 = q0 * (q0 + q0);
+  return fma(0.5, fma(w0, da, w1 * dc) / (w0 + w1), b);
 }
 
 // x / h, as a multiplication by the exact reciprocal when h is a power of two (then bitwise equal)
@@ -118,6 +116,7 @@ __global__ void k_ns_source(double* __restrict__ f, const double* __restrict__ U
   const double* __restrict__ phi = vel[C];
   const double h = G.h;
   const InvH dh{G.h, G.hinv, G.hpow2};
+  const double weps = kWenoEps * (h * h);
   for (int64_t idx = ns_tid(); idx < G.cells; idx += ns_stride()) {
     int k[3];
     ns_coords(G, idx, k);
@@ -148,20 +147,17 @@ __global__ void k_ns_source(double* __restrict__ f, const double* __restrict__ U
         const double* __restrict__ A = vel[a];
         const int64_t sa = G.st[a], sc = G.st[C];
         const bool in = k[a] > 0;
-        const double lo = 0.5 * ((in ? A[idx - sa] : 0.0) + A[idx]);
-        const double hi = 0.5 * ((in ? A[idx - sa + sc] : 0.0) + A[idx + sc]);
-        adv = 0.5 * (lo + hi);
+        adv = 0.25 * (((in ? A[idx - sa] : 0.0) + A[idx]) + ((in ? A[idx - sa + sc] : 0.0) + A[idx + sc]));
       }
       // only the upwind WENO3 derivative is used: the left-biased one (differences d1, d2, d3) where
       // the advecting velocity is positive, the right-biased one (d4, d3, d2) elsewhere
       const bool up = adv > 0.0;
-      const double d2 = dh(v[2] - v[1]), d3 = dh(v[3] - v[2]);
-      const double dx = up ? dh(v[1] - v[0]) : dh(v[4] - v[3]);
-      const double dd = weno3(dx, up ? d2 : d3, up ? d3 : d2);
-      conv = conv + adv * dd;
+      const double d2 = v[2] - v[1], d3 = v[3] - v[2];
+      const double dx = up ? v[1] - v[0] : v[4] - v[3];
+      conv = fma(adv, weno3(dx, up ? d2 : d3, up ? d3 : d2, weps), conv);
     }
-    const double gp = dh(P[idx + G.st[C]] - P[idx]);
-    double v = phi[idx] - dt * conv - dt * gp;
+    // conv and the pressure difference are both over h
+    double v = phi[idx] - dt * dh(conv + (P[idx + G.st[C]] - P[idx]));
     if (F) v = v + dt * F[idx];
     if (C != DIM - 1 && k[DIM - 1] == G.n[DIM - 1] - 1) v = v + 2.0 * beta * lid_c / (h * h);
     f[idx] = v;
@@ -187,6 +183,7 @@ __global__ void k_ns_source2(double* __restrict__ f, const double* __restrict__ 
   const double* __restrict__ co = old[C];
   const double h = G.h;
   const InvH dh{G.h, G.hinv, G.hpow2};
+  const double weps = kWenoEps * (h * h);
   for (int64_t idx = ns_tid(); idx < G.cells; idx += ns_stride()) {
     int k[3];
     ns_coords(G, idx, k);
@@ -207,15 +204,16 @@ __global__ void k_ns_source2(double* __restrict__ f, const double* __restrict__ 
 #pragma unroll
         for (int s = -2; s <= 2; ++s) {
           int F2 = k[a] + 1 + s;  // face index, odd continuation beyond the walls
-          double sg = 1.0;
+          bool flip = false;
           if (F2 < 0) {
             F2 = -F2;
-            sg = -1.0;
+            flip = true;
           } else if (F2 > n) {
             F2 = 2 * n - F2;
-            sg = -1.0;
+            flip = true;
           }
-          v[s + 2] = F2 == 0 ? 0.0 : sg * cbar(line + (int64_t)(F2 - 1) * st);
+          const double cv = F2 == 0 ? 0.0 : cbar(line + (int64_t)(F2 - 1) * st);
+          v[s + 2] = flip ? -cv : cv;
         }
         const double lo = k[a] > 0 ? cc[idx - st] : 0.0;
         lap += (lo - 2.0 * c0) + cc[idx + st];
@@ -241,20 +239,17 @@ __global__ void k_ns_source2(double* __restrict__ f, const double* __restrict__ 
         auto A = [&](int64_t q) { return a < C ? 0.5 * (Ao[q] + Ac[q]) : 0.5 * (3.0 * Ac[q] - Ao[q]); };
         const int64_t sa = G.st[a], sc = G.st[C];
         const bool in = k[a] > 0;
-        const double lo = 0.5 * ((in ? A(idx - sa) : 0.0) + A(idx));
-        const double hi = 0.5 * ((in ? A(idx - sa + sc) : 0.0) + A(idx + sc));
-        adv = 0.5 * (lo + hi);
+        adv = 0.25 * (((in ? A(idx - sa) : 0.0) + A(idx)) + ((in ? A(idx - sa + sc) : 0.0) + A(idx + sc)));
       }
       // only the upwind WENO3 derivative is used: the left-biased one (differences d1, d2, d3) where
       // the advecting velocity is positive, the right-biased one (d4, d3, d2) elsewhere
       const bool up = adv > 0.0;
-      const double d2 = dh(v[2] - v[1]), d3 = dh(v[3] - v[2]);
-      const double dx = up ? dh(v[1] - v[0]) : dh(v[4] - v[3]);
-      const double dd = weno3(dx, up ? d2 : d3, up ? d3 : d2);
-      conv = conv + adv * dd;
+      const double d2 = v[2] - v[1], d3 = v[3] - v[2];
+      const double dx = up ? v[1] - v[0] : v[4] - v[3];
+      conv = fma(adv, weno3(dx, up ? d2 : d3, up ? d3 : d2, weps), conv);
     }
-    const double gp = dh(P[idx + G.st[C]] - P[idx]);
-    double v = c0 - dt * conv + beta * dh(dh(lap)) - dt * gp;
+    // conv and the pressure difference are both over h
+    double v = c0 - dt * dh(conv + (P[idx + G.st[C]] - P[idx])) + beta * dh(dh(lap));
     if (F) v = v + dt * F[idx];
     if (C != DIM - 1 && k[DIM - 1] == G.n[DIM - 1] - 1) v = v + 2.0 * (2.0 * beta * lid_c / (h * h));
     f[idx] = v;

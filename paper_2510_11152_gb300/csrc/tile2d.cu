@@ -886,8 +886,10 @@ cudaError_t post_launch(const TileArgs<T>& a, const LevelDesc<T>& L, cudaStream_
   return cudaGetLastError();
 }
 
-// Rows per region: 64 (the fewest recomputed halo rows) where such blocks fill the GPU, otherwise 32.
-bool tall_regions(int nx, int ny, int halo, int sm_count) {
+// Rows per region: 64 (the fewest recomputed halo rows) where such blocks fill the GPU, otherwise 32; `rows` > 0 asks
+// for one of the two.
+bool tall_regions(int nx, int ny, int halo, int rows, int sm_count) {
+  if (rows > 0) return rows > 32;
   const int ox = kTileCols - 2 * halo, oy = 64 - 2 * halo;
   return (int64_t)((nx + ox - 1) / ox) * ((ny + oy - 1) / oy) >= sm_count;
 }
@@ -914,7 +916,7 @@ int tile_fixed_bits(const LevelDesc<double>& L, int nu) {
 
 template <typename T>
 cudaError_t launch_tile_pre(const T* uin, const T* fin, T* fout, T* uout, T* uc, T* rc, const LevelDesc<T>& L, int nu,
-                            int ordering, bool tau, int bits, int sm_count, cudaStream_t stream) {
+                            int ordering, bool tau, int bits, int rows, int sm_count, cudaStream_t stream) {
   if (nu < 1 || nu > kTileMaxNu || (tau && !uin)) return cudaErrorInvalidValue;
   TileArgs<T> a{};
   a.uin = uin;
@@ -927,7 +929,7 @@ cudaError_t launch_tile_pre(const T* uin, const T* fin, T* fout, T* uout, T* uc,
   a.ordering = ordering;
   a.halo = 2 * nu + 2;
   a.bits = bits;
-  const bool tall = tall_regions(L.nx, L.ny, a.halo, sm_count);
+  const bool tall = tall_regions(L.nx, L.ny, a.halo, rows, sm_count);
   constexpr int R = kTileR<T>, W = 64 / R, S = kTileRShort<T>, WS = 32 / S;
   if (tau) return tall ? pre_launch<T, R, W, true, true>(a, L, stream) : pre_launch<T, S, WS, true, true>(a, L, stream);
   if (uin) return tall ? pre_launch<T, R, W, true, false>(a, L, stream) : pre_launch<T, S, WS, true, false>(a, L, stream);
@@ -936,7 +938,7 @@ cudaError_t launch_tile_pre(const T* uin, const T* fin, T* fout, T* uout, T* uc,
 
 template <typename T>
 cudaError_t launch_tile_post(const T* uin, const T* f, const T* uc, T* uout, double* u64, const LevelDesc<T>& L, int nu,
-                             int ordering, bool scaled, int bits, int sm_count, cudaStream_t stream) {
+                             int ordering, bool scaled, int bits, int rows, int sm_count, cudaStream_t stream) {
   if (nu < 1 || nu > kTileMaxNu || (u64 && sizeof(T) == 8)) return cudaErrorInvalidValue;
   TileArgs<T> a{};
   a.uin = uin;
@@ -950,7 +952,7 @@ cudaError_t launch_tile_post(const T* uin, const T* f, const T* uc, T* uout, dou
   a.bits = bits;
   a.scaled = scaled;
   constexpr int R = kTileR<T>, W = 64 / R, S = kTileRShort<T>, WS = 32 / S;
-  return tall_regions(L.nx, L.ny, a.halo, sm_count) ? post_launch<T, R, W, false>(a, L, stream)
+  return tall_regions(L.nx, L.ny, a.halo, rows, sm_count) ? post_launch<T, R, W, false>(a, L, stream)
                                                     : post_launch<T, S, WS, false>(a, L, stream);
 }
 
@@ -958,7 +960,7 @@ cudaError_t launch_tile_post(const T* uin, const T* f, const T* uc, T* uout, dou
 int norm_halo(int nu) { return 2 * nu + 2; }
 
 cudaError_t launch_tile_post_norm(const double* uin, const double* f, const double* uc, double* uout,
-                                  const LevelDesc<double>& L, int nu, int ordering, int bits, const NormEnd& norm,
+                                  const LevelDesc<double>& L, int nu, int ordering, int bits, const NormEnd& norm, int rows,
                                   int sm_count, cudaStream_t stream) {
   if (nu < 0 || nu > kTileMaxNu) return cudaErrorInvalidValue;
   TileArgs<double> a{};
@@ -972,14 +974,14 @@ cudaError_t launch_tile_post_norm(const double* uin, const double* f, const doub
   a.bits = bits;
   a.norm = norm;
   constexpr int R = kTileR<double>, W = 64 / R, S = kTileRShort<double>, WS = 32 / S;
-  return tall_regions(L.nx, L.ny, a.halo, sm_count) ? post_launch<double, R, W, true>(a, L, stream)
+  return tall_regions(L.nx, L.ny, a.halo, rows, sm_count) ? post_launch<double, R, W, true>(a, L, stream)
                                                     : post_launch<double, S, WS, true>(a, L, stream);
 }
 
-int tile_norm_blocks(int nx, int ny, int nu, int sm_count) {
+int tile_norm_blocks(int nx, int ny, int nu) {
   int most = 0;
   for (const int n : {0, nu}) {
-    const int h = norm_halo(n), ox = kTileCols - 2 * h, oy = (tall_regions(nx, ny, h, sm_count) ? 64 : 32) - 2 * h;
+    const int h = norm_halo(n), ox = kTileCols - 2 * h, oy = 32 - 2 * h;
     most = std::max(most, ((nx + ox - 1) / ox) * ((ny + oy - 1) / oy));
   }
   return most;
@@ -1009,11 +1011,11 @@ cudaError_t tile2d_prepare() {
   return err;
 }
 
-#define TILE_INSTANCE(T)                                                                                             \
+#define TILE_INSTANCE(T)                                                                                              \
   template cudaError_t launch_tile_pre<T>(const T*, const T*, T*, T*, T*, T*, const LevelDesc<T>&, int, int, bool, int, \
-                                          int, cudaStream_t);                                                        \
-  template cudaError_t launch_tile_post<T>(const T*, const T*, const T*, T*, double*, const LevelDesc<T>&, int, int,  \
-                                           bool, int, int, cudaStream_t);                                            \
+                                          int, int, cudaStream_t);                                                    \
+  template cudaError_t launch_tile_post<T>(const T*, const T*, const T*, T*, double*, const LevelDesc<T>&, int, int,   \
+                                           bool, int, int, int, cudaStream_t);                                        \
   template cudaError_t launch_tile_coarse<T>(const TileCoarse<T>&, T*, const T*, cudaStream_t);
 TILE_INSTANCE(float)
 TILE_INSTANCE(double)

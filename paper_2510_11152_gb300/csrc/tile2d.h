@@ -21,24 +21,24 @@ int tile_fixed_bits(const LevelDesc<double>& L, int nu);
 // Pre-smoothing of a level: uout = S^nu(uin) (uin = 0 when uin is null), uc = R(uout), rc = R(f - A uout).
 // tau: f = fin + A uin is formed first (fin holding R(r) of the finer level). fout (tau only) receives
 // the right-hand side for launch_tile_post: f itself in float32, b f (the point equation's
-// right-hand side, b = h^2 / D) in float64.
+// right-hand side, b = h^2 / D) in float64. rows: rows per region (0: by size; up to 32: 32; more: 64).
 template <typename T>
 cudaError_t launch_tile_pre(const T* uin, const T* fin, T* fout, T* uout, T* uc, T* rc, const LevelDesc<T>& L, int nu,
-                            int ordering, bool tau, int bits, int sm_count, cudaStream_t stream);
+                            int ordering, bool tau, int bits, int rows, int sm_count, cudaStream_t stream);
 
 // Post-smoothing: e = S^nu(uin + P(uc - R(uin))); uout = e, or u64 += e when u64 is given (uout unused).
 // scaled: f holds b f as written by launch_tile_pre with tau.
 template <typename T>
 cudaError_t launch_tile_post(const T* uin, const T* f, const T* uc, T* uout, double* u64, const LevelDesc<T>& L, int nu,
-                             int ordering, bool scaled, int bits, int sm_count, cudaStream_t stream);
+                             int ordering, bool scaled, int bits, int rows, int sm_count, cudaStream_t stream);
 
 // launch_tile_post in float64 on a level whose f is not scaled, with the norm of the residual f - A uout at
 // its end. uc null with nu 0: no correction; uout null: the norm only. norm.partials holds at least
 // tile_norm_blocks values.
 cudaError_t launch_tile_post_norm(const double* uin, const double* f, const double* uc, double* uout,
-                                  const LevelDesc<double>& L, int nu, int ordering, int bits, const NormEnd& norm,
+                                  const LevelDesc<double>& L, int nu, int ordering, int bits, const NormEnd& norm, int rows,
                                   int sm_count, cudaStream_t stream);
-int tile_norm_blocks(int nx, int ny, int nu, int sm_count);
+int tile_norm_blocks(int nx, int ny, int nu);
 
 // The V-cycle of levels l0..nlev-1, all of at most tile_coarse_cells per axis, in one CTA. utop / ftop: level l0 in
 // device memory (utop updated in place); tau: ftop holds R(r), and f = ftop + A utop is formed first.
