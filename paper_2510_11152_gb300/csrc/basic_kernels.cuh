@@ -792,6 +792,25 @@ __global__ void k_kappa_weights(T* wx, T* wy, T* wz, T* rD, T* Dh, const double*
   }
 }
 
+// The fractions a_f = w_f / D of a 2D float64 level in units of 2^-62 (LevelDesc::aq), and *bad set where they are not the
+// weights of an average: a negative one, a sum above 1, or a diagonal far from 1.
+static __global__ void k_kappa_frac(long long* aq, LevelDesc<double> L, int* bad) {
+  const int64_t n = (int64_t)L.nx * L.ny;
+  for (int64_t idx = gtid(); idx < n; idx += gstride()) {
+    const int i = (int)(idx & (L.nx - 1)), j = (int)(idx >> L.lx);
+    const double rd = L.rD[idx];
+    const double a[4] = {i > 0 ? L.wx[idx - 1] * rd : 0.0, i < L.nx - 1 ? L.wx[idx] * rd : 0.0,
+                         j > 0 ? L.wy[idx - L.nx] * rd : 0.0, j < L.ny - 1 ? L.wy[idx] * rd : 0.0};
+    const double b = L.h2 * rd;
+    bool ok = ((a[0] + a[1]) + (a[2] + a[3])) <= 1.0 + 1e-12 && b > 1e-90 && b < 1e90 && L.Dh[idx] < 1e90;
+    for (int k = 0; k < 4; ++k) {
+      ok = ok && a[k] >= 0.0 && a[k] <= 1.0;
+      aq[k * n + idx] = ok ? __double2ll_rn(a[k] * 4611686018427387904.0) : 0;
+    }
+    if (!ok) *bad = 1;
+  }
+}
+
 // ------------------------------------------------------------------------------------------------
 // Arguments of the single-CTA V-cycle over levels l0..nlev-1 (the small levels, which cannot fill the
 // GPU): the same recursion as the host driver, with __syncthreads() between dependent steps. Level l0

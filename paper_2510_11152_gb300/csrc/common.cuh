@@ -46,6 +46,8 @@ struct LevelDesc {
   const T* wz;     // same along z (0 at l = nz-1)
   const T* rD;     // 1 / D
   const T* Dh;     // D / h^2
+  const long long* aq;  // w_f / D in units of 2^-62 of the west, east, y-1, y+1 face of every cell, four arrays one after
+                        // the other (2D float64 levels in block fixed point, tile2d.cu; null otherwise)
   T alpha;         // alpha of A u = alpha u - beta div(kappa grad u)
   T a[kClasses], b[kClasses], d[kClasses];
   short alo[kClasses];         // a 2^64 beyond float64's a (block fixed point, tile2d.cu)

@@ -301,6 +301,29 @@ fas_status coarse_inverse(const fas_ctx* c, const LevelShape& s, const std::vect
   return FAS_OK;
 }
 
+// The fixed-point fractions of every level of a 2D float64 hierarchy with per-cell diffusivity. A level whose weights
+// are not those of an average, or one without room for the arrays, keeps float64 arithmetic (aq null).
+fas_status kappa_fractions(fas_ctx* c, Hier<double>& H) {
+  int* bad = nullptr;
+  STATUS_TRY(dev_alloc(H, &bad, c->nlev));
+  CUDA_TRY(cudaMemsetAsync(bad, 0, c->nlev * sizeof(int), c->stream));
+  std::vector<long long*> aq(c->nlev, nullptr);
+  for (int l = 0; l < c->nlev; ++l) {
+    const int64_t n = c->shape[l].cells();
+    if (n > INT32_MAX || dev_alloc(H, &aq[l], 4 * n) != FAS_OK) {
+      cudaGetLastError();
+      aq[l] = nullptr;
+      continue;
+    }
+    k_kappa_frac<<<grid_for(c, n), kBlock, 0, c->stream>>>(aq[l], H.desc[l], bad + l);
+  }
+  std::vector<int> hb(c->nlev, 0);
+  CUDA_TRY(cudaMemcpyAsync(hb.data(), bad, c->nlev * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(cudaStreamSynchronize(c->stream));
+  for (int l = 0; l < c->nlev; ++l) H.desc[l].aq = hb[l] ? nullptr : aq[l];
+  return FAS_OK;
+}
+
 // Build one hierarchy: descriptors for every level, buffers when `buffers`, variable-kappa arrays.
 template <typename T>
 fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers) {
@@ -440,13 +463,15 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
     // tile kernel
     H.tiled = false;
     H.ntile = 0;
-    if (p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL && p.nu1 >= 1 && p.nu1 <= kTileMaxNu &&
+    if (p.dim == 2 && p.path != 1 && p.location == FAS_CELL && p.nu1 >= 1 && p.nu1 <= kTileMaxNu &&
         p.nu2 >= 1 && p.nu2 <= kTileMaxNu) {
       int lc = 0;
       const int most = tile_coarse_cells<T>();
       while (lc < c->nlev && (c->shape[lc].nx > most || c->shape[lc].ny > most)) ++lc;
-      H.tiled = lc < c->nlev;
+      H.tiled = lc < c->nlev && !(p.kappa && c->shape[0].cells() > INT32_MAX);  // cells by 32-bit index there
       H.ntile = H.tiled ? lc : 0;
+      if constexpr (std::is_same<T, double>::value)
+        if (H.tiled && p.kappa) STATUS_TRY(kappa_fractions(c, H));
     }
     // sweep-fused 2D path (float32 only): consecutive levels from the finest that the fused kernels
     // handle and that are larger than the single-CTA switch level
@@ -502,6 +527,7 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       A.nuc = nuc;
       A.ordering = p.ordering;
       A.tau = H.ntile > 0;
+      A.varkappa = p.kappa != nullptr;
     }
     // sweep-fused 3D smoothing (float32): a second buffer on every level that the fused sweep handles
     // (its sweeps ping-pong between the two) and that is large enough for it to pay: measured at

@@ -136,20 +136,32 @@ __device__ __forceinline__ int64_t to_fixed_mul(double f, Mant b, Scale s) {
 // arithmetic policies. V: the value held in registers. F holds f (RawF) or b f (Scaled*).
 // ------------------------------------------------------------------------------------------------
 
+// The four neighbours of a cell: west, east, row - 1, row + 1 (0 where there is none).
+template <typename V>
+struct Nb4 {
+  V w, e, s, n;
+  __device__ __forceinline__ V sum() const { return (w + e) + (s + n); }
+};
+
 // The per-operation kernels' float32 expressions.
 struct RawF {
+  static constexpr bool kVar = false;
   using T = float;
   using V = float;
+  using N = Nb4<V>;
   struct A { float a, b; };
   const LevelDesc<float>& L;
   __device__ __forceinline__ A coef(int cls) const { return A{L.a[cls], L.b[cls]}; }
   __device__ __forceinline__ V in(float x) const { return x; }
   __device__ __forceinline__ V in_f(float x, int, bool, bool) const { return x; }
   __device__ __forceinline__ float out(V x) const { return x; }
-  __device__ __forceinline__ V update(V nb, V f, A c) const { return fmaf(c.a, nb, c.b * f); }
-  __device__ __forceinline__ V tau(V f, V u, V nb, A, int cls) const { return f + fmaf(L.d[cls], u, -L.c * nb); }
-  __device__ __forceinline__ V resid(V f, V u, V nb, A, int cls) const {
-    return fmaf(L.c, nb, fmaf(-L.d[cls], u, f));
+  __device__ __forceinline__ float out_f(V x) const { return x; }
+  __device__ __forceinline__ V update(N nb, V f, A c) const { return fmaf(c.a, nb.sum(), c.b * f); }
+  __device__ __forceinline__ V tau(V f, V u, N nb, A, int cls) const {
+    return f + fmaf(L.d[cls], u, -L.c * nb.sum());
+  }
+  __device__ __forceinline__ V resid(V f, V u, N nb, A, int cls) const {
+    return fmaf(L.c, nb.sum(), fmaf(-L.d[cls], u, f));
   }
   __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return ((a + b) + (c + d)) * 0.25f; }
   __device__ __forceinline__ float out_avg(V a, V b, V c, V d) const { return avg(a, b, c, d); }
@@ -158,17 +170,20 @@ struct RawF {
 
 // Float64 arithmetic on the scaled point equation (regions that fixed point does not take).
 struct ScaledD {
+  static constexpr bool kVar = false;
   using T = double;
   using V = double;
+  using N = Nb4<V>;
   struct A { double a; };
   const LevelDesc<double>& L;
   __device__ __forceinline__ A coef(int cls) const { return A{L.a[cls]}; }
   __device__ __forceinline__ V in(double x) const { return x; }
   __device__ __forceinline__ V in_f(double x, int cls, bool, bool scaled) const { return scaled ? x : L.b[cls] * x; }
   __device__ __forceinline__ double out(V x) const { return x; }
-  __device__ __forceinline__ V update(V nb, V f, A c) const { return fma(c.a, nb, f); }
-  __device__ __forceinline__ V tau(V f, V u, V nb, A c, int) const { return f + fma(-c.a, nb, u); }
-  __device__ __forceinline__ V resid(V f, V u, V nb, A c, int) const { return fma(c.a, nb, f - u); }
+  __device__ __forceinline__ double out_f(V x) const { return x; }
+  __device__ __forceinline__ V update(N nb, V f, A c) const { return fma(c.a, nb.sum(), f); }
+  __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + fma(-c.a, nb.sum(), u); }
+  __device__ __forceinline__ V resid(V f, V u, N nb, A c, int) const { return fma(c.a, nb.sum(), f - u); }
   __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return ((a + b) + (c + d)) * 0.25; }
   __device__ __forceinline__ double out_avg(V a, V b, V c, V d) const { return avg(a, b, c, d); }
   __device__ __forceinline__ double out_avg_r(V a, V b, V c, V d, int ca, int cb, int cc, int cd) const {
@@ -183,13 +198,17 @@ struct ScaledD {
 // multiply 2 N by a / 2.
 template <bool INNER>
 struct ScaledX {
+  static constexpr bool kVar = false;
   using T = double;
   using V = int64_t;
+  using N = Nb4<V>;
   using A = Frac;
   const LevelDesc<double>& L;
   Scale s;
   Mant be, bo;  // b of the thread's even and odd column away from the y boundaries
-  __device__ __forceinline__ A coef(int cls) const { return INNER ? frac_of(L.a[cls], L.alo[cls]) : frac_of(0.5 * L.a[cls], L.alo[cls] >> 1); }
+  __device__ __forceinline__ A coef(int cls) const {
+    return INNER ? frac_of(L.a[cls], L.alo[cls]) : frac_of(0.5 * L.a[cls], L.alo[cls] >> 1);
+  }
   __device__ __forceinline__ V times(V nb, A c) const { return mul_frac(INNER ? nb : nb + nb, c); }
   __device__ __forceinline__ V in(double x) const { return to_fixed(x, s); }
   __device__ __forceinline__ V in_f(double x, int cls, bool odd, bool scaled) const {
@@ -197,9 +216,10 @@ struct ScaledX {
     return to_fixed_mul(x, !INNER && (cls & 12) ? mant_of(L.b[cls]) : (!INNER && odd ? bo : be), s);
   }
   __device__ __forceinline__ double out(V x) const { return from_fixed(x, s); }
-  __device__ __forceinline__ V update(V nb, V f, A c) const { return times(nb, c) + f; }
-  __device__ __forceinline__ V tau(V f, V u, V nb, A c, int) const { return f + (u - times(nb, c)); }
-  __device__ __forceinline__ V resid(V f, V u, V nb, A c, int) const { return (f - u) + times(nb, c); }
+  __device__ __forceinline__ double out_f(V x) const { return from_fixed(x, s); }
+  __device__ __forceinline__ V update(N nb, V f, A c) const { return times(nb.sum(), c) + f; }
+  __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + (u - times(nb.sum(), c)); }
+  __device__ __forceinline__ V resid(V f, V u, N nb, A c, int) const { return (f - u) + times(nb.sum(), c); }
   __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return (((a + b) + (c + d)) + 2) >> 2; }
   __device__ __forceinline__ double out_avg(V a, V b, V c, V d) const { return from_fixed((a + b) + (c + d), s, 2); }
   __device__ __forceinline__ double out_avg_r(V a, V b, V c, V d, int ca, int cb, int cc, int cd) const {
@@ -216,6 +236,126 @@ struct ScaledX {
   __device__ __forceinline__ float norm_value(V r, int cls, float fac) const {
     // by halves: the 64-bit integer conversion runs at the FP64 pipe's rate
     return fmaf((float)(int)(r >> 32), 4294967296.f, (float)(uint32_t)r) * fac;
+  }
+};
+
+// ---- per-cell diffusivity: the face weights and the diagonal of a cell come from the level's arrays, by the cell's
+// index (id; -1 outside the domain, where all coefficients are 0)
+
+struct VarF {  // float32, the per-operation kernels' expressions
+  static constexpr bool kVar = true;
+  using T = float;
+  using V = float;
+  using N = Nb4<V>;
+  struct A { float w, e, s, n, rd; };
+  const LevelDesc<float>& L;
+  __device__ __forceinline__ A coef(int id) const {
+    if (id < 0) return A{};
+    const int i = id & (L.nx - 1), j = id >> L.lx;
+    return A{i > 0 ? L.wx[id - 1] : 0.f, i < L.nx - 1 ? L.wx[id] : 0.f, j > 0 ? L.wy[id - L.nx] : 0.f,
+             j < L.ny - 1 ? L.wy[id] : 0.f, L.rD[id]};
+  }
+  __device__ __forceinline__ float nsum(N nb, A c) const {
+    return fmaf(c.n, nb.n, fmaf(c.s, nb.s, fmaf(c.e, nb.e, fmaf(c.w, nb.w, 0.f))));
+  }
+  __device__ __forceinline__ V in(float x) const { return x; }
+  __device__ __forceinline__ V in_f(float x, int, bool, bool) const { return x; }
+  __device__ __forceinline__ float out(V x) const { return x; }
+  __device__ __forceinline__ float out_f(V x) const { return x; }
+  __device__ __forceinline__ V update(N nb, V f, A c) const { return fmaf(L.h2, f, nsum(nb, c)) * c.rd; }
+  __device__ __forceinline__ V tau(V f, V u, N nb, A c, int id) const {
+    return f + fmaf(L.Dh[id], u, -L.ih2 * nsum(nb, c));
+  }
+  __device__ __forceinline__ V resid(V f, V u, N nb, A c, int id) const {
+    return id < 0 ? 0.f : fmaf(L.ih2, nsum(nb, c), fmaf(-L.Dh[id], u, f));
+  }
+  __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return ((a + b) + (c + d)) * 0.25f; }
+  __device__ __forceinline__ float out_avg(V a, V b, V c, V d) const { return avg(a, b, c, d); }
+  __device__ __forceinline__ float out_avg_r(V a, V b, V c, V d, int, int, int, int) const { return avg(a, b, c, d); }
+};
+
+// In float64 the cell's equation divided by its diagonal, u = sum_f a_f u_f + b f with a_f = w_f / D.
+struct VarD {
+  static constexpr bool kVar = true;
+  using T = double;
+  using V = double;
+  using N = Nb4<V>;
+  struct A { double w, e, s, n; };
+  const LevelDesc<double>& L;
+  __device__ __forceinline__ A coef(int id) const {
+    if (id < 0) return A{};
+    const int i = id & (L.nx - 1), j = id >> L.lx;
+    const double rd = L.rD[id];
+    return A{i > 0 ? L.wx[id - 1] * rd : 0.0, i < L.nx - 1 ? L.wx[id] * rd : 0.0, j > 0 ? L.wy[id - L.nx] * rd : 0.0,
+             j < L.ny - 1 ? L.wy[id] * rd : 0.0};
+  }
+  __device__ __forceinline__ double nsum(N nb, A c) const {
+    return fma(c.n, nb.n, fma(c.s, nb.s, fma(c.e, nb.e, c.w * nb.w)));
+  }
+  __device__ __forceinline__ V in(double x) const { return x; }
+  __device__ __forceinline__ V in_f(double x, int id, bool, bool scaled) const {
+    return scaled || id < 0 ? x : (L.h2 * L.rD[id]) * x;
+  }
+  __device__ __forceinline__ double out(V x) const { return x; }
+  __device__ __forceinline__ double out_f(V x) const { return x; }
+  __device__ __forceinline__ V update(N nb, V f, A c) const { return nsum(nb, c) + f; }
+  __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + (u - nsum(nb, c)); }
+  __device__ __forceinline__ V resid(V f, V u, N nb, A c, int) const { return (f - u) + nsum(nb, c); }
+  __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return ((a + b) + (c + d)) * 0.25; }
+  __device__ __forceinline__ double out_avg(V a, V b, V c, V d) const { return avg(a, b, c, d); }
+  __device__ __forceinline__ double dh(int id) const { return id < 0 ? 0.0 : L.Dh[id]; }
+  __device__ __forceinline__ double out_avg_r(V a, V b, V c, V d, int ia, int ib, int ic, int id) const {
+    return ((dh(ia) * a + dh(ib) * b) + (dh(ic) * c + dh(id) * d)) * 0.25;
+  }
+  __device__ __forceinline__ float norm_factor(int, float ns) const { return ns; }
+  __device__ __forceinline__ float norm_value(V r, int id, float fac) const { return (float)(dh(id) * r) * fac; }
+};
+
+// Block fixed point with the four a_f as 64-bit fractions (LevelDesc::aq, a 2^62). A value u of X units is held as
+// 4 X, so that a fraction of 62 bits gives X units; updated values are whole units.
+struct VarX {
+  static constexpr bool kVar = true;
+  using T = double;
+  using V = int64_t;
+  using N = Nb4<V>;
+  struct A { Frac w, e, s, n; };
+  const LevelDesc<double>& L;
+  Scale s;   // of f and of the residual
+  Scale s4;  // of u: two bits more
+  static __device__ __forceinline__ Frac unpack(long long a) {
+    const int lo = (int)(uint32_t)a;
+    return Frac{(int)((a - (long long)lo) >> 32), lo};
+  }
+  __device__ __forceinline__ A coef(int id) const {
+    if (id < 0) return A{};
+    const int64_t n = (int64_t)L.nx * L.ny;
+    return A{unpack(L.aq[id]), unpack(L.aq[n + id]), unpack(L.aq[2 * n + id]), unpack(L.aq[3 * n + id])};
+  }
+  __device__ __forceinline__ int64_t nsum(N nb, A c) const {
+    return (mul_frac(nb.w, c.w) + mul_frac(nb.e, c.e)) + (mul_frac(nb.s, c.s) + mul_frac(nb.n, c.n));
+  }
+  static __device__ __forceinline__ int64_t units(V u) { return (u + 2) >> 2; }
+  __device__ __forceinline__ V in(double x) const { return to_fixed(x, s4); }
+  __device__ __forceinline__ V in_f(double x, int id, bool, bool scaled) const {
+    return scaled || id < 0 ? to_fixed(x, s) : to_fixed_mul(x, mant_of(L.h2 * L.rD[id]), s);
+  }
+  __device__ __forceinline__ double out(V x) const { return from_fixed(x, s4); }
+  __device__ __forceinline__ double out_f(V x) const { return from_fixed(x, s); }
+  __device__ __forceinline__ V update(N nb, V f, A c) const { return (nsum(nb, c) + f) << 2; }
+  __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + (units(u) - nsum(nb, c)); }
+  __device__ __forceinline__ V resid(V f, V u, N nb, A c, int) const { return (f - units(u)) + nsum(nb, c); }
+  __device__ __forceinline__ V avg(V a, V b, V c, V d) const { return units((units(a) + units(b)) + (units(c) + units(d))) << 2; }
+  __device__ __forceinline__ double out_avg(V a, V b, V c, V d) const {
+    return from_fixed((units(a) + units(b)) + (units(c) + units(d)), s, 2);
+  }
+  __device__ __forceinline__ double dh(int id) const { return id < 0 ? 0.0 : L.Dh[id]; }
+  __device__ __forceinline__ double out_avg_r(V a, V b, V c, V d, int ia, int ib, int ic, int id) const {
+    return ((dh(ia) * from_fixed(a, s) + dh(ib) * from_fixed(b, s)) +
+            (dh(ic) * from_fixed(c, s) + dh(id) * from_fixed(d, s))) * 0.25;
+  }
+  __device__ __forceinline__ float norm_factor(int, float ns) const { return (float)(from_fixed(1, s) * (double)ns); }
+  __device__ __forceinline__ float norm_value(V r, int id, float fac) const {
+    return fmaf((float)(int)(r >> 32), 4294967296.f, (float)(uint32_t)r) * fac * f64_to_f32_rn_bits(dh(id));
   }
 };
 
@@ -267,7 +407,12 @@ struct Region {
 
   __device__ __forceinline__ Region(const P& p, const Place& pl, Edge<V>* ed)
       : pol(p), g(pl), edge(ed), lane(threadIdx.x & 31), warp(threadIdx.x >> 5) {
-    if (INNER) {
+    if constexpr (P::kVar) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) co[r][k] = p.coef(id(r, k));
+    } else if constexpr (INNER) {
       co[0][0] = p.coef(0);
     } else {
       // cells outside the domain get coefficients 0: with f = 0 their value then stays 0
@@ -291,7 +436,9 @@ struct Region {
   static __device__ __forceinline__ constexpr bool odd(int r) { return r & 1; }
   // the cell of colour k is the odd column
   static __device__ __forceinline__ constexpr bool odd_col(int r, int k) { return (k == 1) != odd(r); }
-  __device__ __forceinline__ int cls(int r, int k) const {
+  // what the policy knows the cell by: its boundary class, or its index
+  __device__ __forceinline__ int id(int r, int k) const {
+    if (P::kVar) return g.col_in && g.row_in(r) ? (g.y + r) * g.nx + g.x + (odd_col(r, k) ? 1 : 0) : -1;
     return INNER ? 0 : ((odd_col(r, k) ? g.xfo : g.xfe) | g.yf(r));
   }
   __device__ __forceinline__ A coef(int r, int k) const { return INNER ? co[0][0] : co[INNER ? 0 : r][k]; }
@@ -300,15 +447,22 @@ struct Region {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       u[r][k] = pol.in(uw[odd_col(r, k)]);
-      f[r][k] = pol.in_f(fw[odd_col(r, k)], cls(r, k), odd_col(r, k), scaled);
+      f[r][k] = pol.in_f(fw[odd_col(r, k)], id(r, k), odd_col(r, k), scaled);
     }
   }
-  // the (even, odd) column of row r of x
+  // the (even, odd) column of row r of u, of f
   template <typename T2>
-  __device__ __forceinline__ T2 pair(const V (&x)[R][2], int r) const {
+  __device__ __forceinline__ T2 pair_u(int r) const {
     T2 v;
-    v.x = pol.out(x[r][odd(r)]);
-    v.y = pol.out(x[r][!odd(r)]);
+    v.x = pol.out(u[r][odd(r)]);
+    v.y = pol.out(u[r][!odd(r)]);
+    return v;
+  }
+  template <typename T2>
+  __device__ __forceinline__ T2 pair_f(int r) const {
+    T2 v;
+    v.x = pol.out_f(f[r][odd(r)]);
+    v.y = pol.out_f(f[r][!odd(r)]);
     return v;
   }
   __device__ __forceinline__ V above(int r, int k) const {  // row r - 1
@@ -319,12 +473,13 @@ struct Region {
     if (r < R - 1) return u[r < R - 1 ? r + 1 : 0][k];
     return edge[g.wd].v[0][k][lane];
   }
-  // sum of the existing neighbours of cell (r, k): (west + east) + (row - 1 + row + 1)
-  __device__ __forceinline__ V nbsum(int r, int k) const {
+  // the neighbours of cell (r, k)
+  __device__ __forceinline__ Nb4<V> nb(int r, int k) const {
     const V own = u[r][1 - k];
     V far = shfl_v(own, odd_col(r, k) ? g.srcE : g.srcW);
     if (!INNER && (odd_col(r, k) ? g.noE : g.noW)) far = V(0);
-    return (own + far) + (above(r, 1 - k) + below(r, 1 - k));
+    const V a = above(r, 1 - k), b = below(r, 1 - k);
+    return odd_col(r, k) ? Nb4<V>{own, far, a, b} : Nb4<V>{far, own, a, b};
   }
   __device__ __forceinline__ void publish(int k) {
     edge[warp].v[0][k][lane] = u[0][k];
@@ -341,7 +496,7 @@ struct Region {
   __device__ __forceinline__ void phase() {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      u[r][K] = pol.update(nbsum(r, K), f[r][K], coef(r, K));
+      u[r][K] = pol.update(nb(r, K), f[r][K], coef(r, K));
     }
     publish(K);
     meet();
@@ -359,12 +514,12 @@ struct Region {
     for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const V nb = nbsum(r, k);
-        if (INNER || (g.col_in && g.row_in(r))) f[r][k] = pol.tau(f[r][k], u[r][k], nb, coef(r, k), cls(r, k));
+        const Nb4<V> b = nb(r, k);
+        if (INNER || (g.col_in && g.row_in(r))) f[r][k] = pol.tau(f[r][k], u[r][k], b, coef(r, k), id(r, k));
       }
   }
   __device__ __forceinline__ V rho(int r, int k) const {
-    return pol.resid(f[r][k], u[r][k], nbsum(r, k), coef(r, k), cls(r, k));
+    return pol.resid(f[r][k], u[r][k], nb(r, k), coef(r, k), id(r, k));
   }
   // u += P(uc - R(u)) for row pair q
   __device__ __forceinline__ void correct(int q, V cv) {
@@ -381,7 +536,7 @@ struct Region {
     const int r = 2 * q;
     const V r00 = rho(r, 0), r01 = rho(r, 1), r10 = rho(r + 1, 1), r11 = rho(r + 1, 0);  // (row, column)
     *cu = pol.out_avg(u[r][0], u[r][1], u[r + 1][1], u[r + 1][0]);
-    *cr = pol.out_avg_r(r00, r01, r10, r11, cls(r, 0), cls(r, 1), cls(r + 1, 1), cls(r + 1, 0));
+    *cr = pol.out_avg_r(r00, r01, r10, r11, id(r, 0), id(r, 1), id(r + 1, 1), id(r + 1, 0));
   }
 };
 
@@ -517,6 +672,28 @@ __device__ __forceinline__ int raw_exp(const Raw<double, R>& w, int Eb, bool sca
   return e;
 }
 
+// The same with a per-cell b = h^2 / D.
+template <bool POST, int R>
+__device__ __forceinline__ int raw_exp_var(const Raw<double, R>& w, const LevelDesc<double>& L, const Place& g, bool scaled) {
+  int e = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      e = max(e, exp_field(w.u[r][c]));
+      const int ef = exp_field(w.f[r][c]);
+      if (scaled || ef == 0 || ef == 0x7FF || !(g.col_in && g.active && g.row_in(r)))
+        e = max(e, ef);
+      else
+        e = max(e, max(1, min(0x7FE, ef + exp_field(L.h2 * L.rD[(g.y + r) * g.nx + g.x + c]) - 1022)));
+      if (POST && (r & 1) == 0 && c == 0) e = max(e, exp_field(w.c[r >> 1]));
+    }
+  return e;
+}
+__device__ __forceinline__ VarX var_x(const LevelDesc<double>& L, Scale s) {
+  return VarX{L, s, Scale{s.top, s.bits + 2}};
+}
+
 template <bool TAU, bool INNER, int R, typename P, typename T, typename SM>
 __device__ __forceinline__ void pre_run(const P& pol, const TileArgs<T>& a, const Place& g, const RowMap& rm, SM& sm,
                                         const Raw<T, R>& w, int rows) {
@@ -542,8 +719,8 @@ __device__ __forceinline__ void pre_run(const P& pol, const TileArgs<T>& a, cons
       const int64_t off = (int64_t)y * g.nx + g.x;
 #pragma unroll
       for (int d = 0; d < 2; ++d) {
-        *reinterpret_cast<T2*>(a.uout + off + d * g.nx) = Q.template pair<T2>(Q.u, 2 * k + d);
-        if (TAU) *reinterpret_cast<T2*>(a.fout + off + d * g.nx) = Q.template pair<T2>(Q.f, 2 * k + d);
+        *reinterpret_cast<T2*>(a.uout + off + d * g.nx) = Q.template pair_u<T2>(2 * k + d);
+        if (TAU) *reinterpret_cast<T2*>(a.fout + off + d * g.nx) = Q.template pair_f<T2>(2 * k + d);
       }
       const int64_t co = (int64_t)(y >> 1) * (g.nx >> 1) + (g.x >> 1);
       a.uc[co] = cu;
@@ -582,8 +759,8 @@ __device__ __forceinline__ float post_run(const P& pol, const TileArgs<T>& a, co
       const bool wr = lane_out && q >= a.halo && q < rows - a.halo && y >= 0 && y < rm.ny;
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const int cls = Q.cls(r, k);
-        const float v = pol.norm_value(Q.rho(r, k), cls, cls ? pol.norm_factor(cls, ns) : fac0);
+        const int id = Q.id(r, k);
+        const float v = pol.norm_value(Q.rho(r, k), id, !P::kVar && id ? pol.norm_factor(id, ns) : fac0);
         if (wr) acc = fmaf(v, v, acc);
       }
     }
@@ -594,7 +771,7 @@ __device__ __forceinline__ float post_run(const P& pol, const TileArgs<T>& a, co
     const int q = R * warp + r, y = g.y + r;
     if (lane_out && q >= a.halo && q < rows - a.halo && y >= 0 && y < rm.ny) {
       const int64_t off = (int64_t)y * g.nx + g.x;
-      const T2 v = Q.template pair<T2>(Q.u, r);
+      const T2 v = Q.template pair_u<T2>(r);
       if constexpr (sizeof(T) == 4) {
         if (a.u64) {  // the refinement step's float64 update
           double2* p = reinterpret_cast<double2*>(a.u64 + off);
@@ -611,7 +788,7 @@ __device__ __forceinline__ float post_run(const P& pol, const TileArgs<T>& a, co
   return acc;
 }
 
-template <typename T, int R, int NW, bool HAS_U, bool TAU>
+template <typename T, int R, int NW, bool HAS_U, bool TAU, bool VAR>
 __global__ void __launch_bounds__(32 * NW) k_tile_pre(const __grid_constant__ TileArgs<T> a,
                                                       const __grid_constant__ LevelDesc<T> L) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
@@ -623,7 +800,15 @@ __global__ void __launch_bounds__(32 * NW) k_tile_pre(const __grid_constant__ Ti
   Raw<T, R> w;
   load_raw<HAS_U, false>(w, a, g, rm, L.per & 1);
   constexpr int rows = R * NW;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (VAR && sizeof(T) == 4) {
+    pre_run<TAU, false>(VarF{L}, a, g, rm, sm, w, rows);
+  } else if constexpr (VAR) {
+    Scale s;
+    if (choose_scale(raw_exp_var<false>(w, L, g, false), a.bits, sm.wmax, NW, &s))
+      pre_run<TAU, false>(var_x(L, s), a, g, rm, sm, w, rows);
+    else
+      pre_run<TAU, false>(VarD{L}, a, g, rm, sm, w, rows);
+  } else if constexpr (sizeof(T) == 4) {
     const RawF pol{L};
     if (inner)
       pre_run<TAU, true>(pol, a, g, rm, sm, w, rows);
@@ -643,7 +828,7 @@ __global__ void __launch_bounds__(32 * NW) k_tile_pre(const __grid_constant__ Ti
   }
 }
 
-template <typename T, int R, int NW, bool RES>
+template <typename T, int R, int NW, bool RES, bool VAR>
 __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ TileArgs<T> a,
                                                        const __grid_constant__ LevelDesc<T> L) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
@@ -656,7 +841,15 @@ __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ T
   load_raw<true, true>(w, a, g, rm, L.per & 1);
   constexpr int rows = R * NW;
   float acc;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (VAR && sizeof(T) == 4) {
+    acc = post_run<false, false>(VarF{L}, a, g, rm, sm, w, rows);
+  } else if constexpr (VAR) {
+    Scale s;
+    if (choose_scale(raw_exp_var<true>(w, L, g, a.scaled), a.bits, sm.wmax, NW, &s))
+      acc = post_run<RES, false>(var_x(L, s), a, g, rm, sm, w, rows);
+    else
+      acc = post_run<RES, false>(VarD{L}, a, g, rm, sm, w, rows);
+  } else if constexpr (sizeof(T) == 4) {
     const RawF pol{L};
     if (inner)
       acc = post_run<false, true>(pol, a, g, rm, sm, w, rows);
@@ -750,10 +943,10 @@ __device__ __forceinline__ void coarse_level(const P& pol, const Place& g, int p
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int off = (g.y + r) * g.nx + g.x;
-    const T2 v = Q.template pair<T2>(Q.u, r);
+    const T2 v = Q.template pair_u<T2>(r);
     if (g.col_in) *reinterpret_cast<T2*>(su + off) = v;
     if (PASS == Pass::kDown) {
-      const T2 b = Q.template pair<T2>(Q.f, r);
+      const T2 b = Q.template pair_f<T2>(r);
       if (g.col_in) *reinterpret_cast<T2*>(sf + off) = b;
     }
   }
@@ -789,14 +982,23 @@ __device__ __forceinline__ void coarse_load(Raw<T, kCoarseR>& w, const Place& g,
   }
 }
 
-template <Pass PASS, typename T, typename SM>
+template <Pass PASS, bool VAR, typename T, typename SM>
 __device__ __forceinline__ void coarse_step(const LevelDesc<T>& L, SM& sm, const TileCoarse<T>& A, const T* u,
                                             const T* f, const T* c, bool tau, bool scaled, int nu, T* su, T* sf, T* cu,
                                             T* cf) {
   const Place g = coarse_place<T>(L.nx, L.ny, L.per);
   Raw<T, kCoarseR> w;
   coarse_load(w, g, u, f, c);
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (VAR && sizeof(T) == 4) {
+    if (g.active) coarse_level<PASS>(VarF{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+  } else if constexpr (VAR) {
+    Scale s;
+    if (choose_scale(raw_exp_var<PASS == Pass::kUp>(w, L, g, scaled), A.bits, sm.wmax, kCoarseWarps<T>, &s)) {
+      if (g.active) coarse_level<PASS>(var_x(L, s), g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+    } else if (g.active) {
+      coarse_level<PASS>(VarD{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+    }
+  } else if constexpr (sizeof(T) == 4) {
     if (g.active) coarse_level<PASS>(RawF{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
   } else {
     Scale s;
@@ -811,7 +1013,7 @@ __device__ __forceinline__ void coarse_step(const LevelDesc<T>& L, SM& sm, const
   __syncthreads();
 }
 
-template <typename T>
+template <typename T, bool VAR>
 __global__ void __launch_bounds__(32 * kCoarseWarps<T>) k_tile_coarse(const __grid_constant__ TileCoarse<T> A, T* utop,
                                                                       const T* ftop) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
@@ -832,7 +1034,7 @@ __global__ void __launch_bounds__(32 * kCoarseWarps<T>) k_tile_coarse(const __gr
   auto F = [&](int l) { return fields + A.off[l] + (desc[l].nx * desc[l].ny + 3) / 4 * 4; };
   for (int l = A.l0; l < last; ++l) {
     const bool top = l == A.l0;
-    coarse_step<Pass::kDown>(desc[l], sm, A, top ? utop : U(l), top ? ftop : F(l), (const T*)nullptr, !top || A.tau,
+    coarse_step<Pass::kDown, VAR>(desc[l], sm, A, top ? utop : U(l), top ? ftop : F(l), (const T*)nullptr, !top || A.tau,
                              false, A.nu1, U(l), F(l), U(l + 1), F(l + 1));
   }
   {
@@ -861,28 +1063,28 @@ __global__ void __launch_bounds__(32 * kCoarseWarps<T>) k_tile_coarse(const __gr
       }
       __syncthreads();
     } else {
-      coarse_step<Pass::kLast>(L, sm, A, top ? utop : U(last), top ? ftop : F(last), (const T*)nullptr, tau, false,
+      coarse_step<Pass::kLast, VAR>(L, sm, A, top ? utop : U(last), top ? ftop : F(last), (const T*)nullptr, tau, false,
                                A.nuc, top ? utop : U(last), (T*)nullptr, (T*)nullptr, (T*)nullptr);
     }
   }
   for (int l = last - 1; l >= A.l0; --l)
-    coarse_step<Pass::kUp>(desc[l], sm, A, U(l), F(l), U(l + 1), false, sizeof(T) == 8, A.nu2,
+    coarse_step<Pass::kUp, VAR>(desc[l], sm, A, U(l), F(l), U(l + 1), false, sizeof(T) == 8, A.nu2,
                            l == A.l0 ? utop : U(l), (T*)nullptr, (T*)nullptr, (T*)nullptr);
 }
 
-template <typename T, int R, int NW, bool HAS_U, bool TAU>
+template <typename T, int R, int NW, bool HAS_U, bool TAU, bool VAR = false>
 cudaError_t pre_launch(const TileArgs<T>& a, const LevelDesc<T>& L, cudaStream_t stream) {
   const int ox = kTileCols - 2 * a.halo, oy = R * NW - 2 * a.halo;
   const dim3 grid((L.nx + ox - 1) / ox, (L.ny + oy - 1) / oy);
-  k_tile_pre<T, R, NW, HAS_U, TAU><<<grid, 32 * NW, sizeof(TileSmem<T, NW>), stream>>>(a, L);
+  k_tile_pre<T, R, NW, HAS_U, TAU, VAR><<<grid, 32 * NW, sizeof(TileSmem<T, NW>), stream>>>(a, L);
   return cudaGetLastError();
 }
 
-template <typename T, int R, int NW, bool RES>
+template <typename T, int R, int NW, bool RES, bool VAR = false>
 cudaError_t post_launch(const TileArgs<T>& a, const LevelDesc<T>& L, cudaStream_t stream) {
   const int ox = kTileCols - 2 * a.halo, oy = R * NW - 2 * a.halo;
   const dim3 grid((L.nx + ox - 1) / ox, (L.ny + oy - 1) / oy);
-  k_tile_post<T, R, NW, RES><<<grid, 32 * NW, sizeof(TileSmem<T, NW>), stream>>>(a, L);
+  k_tile_post<T, R, NW, RES, VAR><<<grid, 32 * NW, sizeof(TileSmem<T, NW>), stream>>>(a, L);
   return cudaGetLastError();
 }
 
@@ -897,9 +1099,10 @@ bool tall_regions(int nx, int ny, int halo, int rows, int sm_count) {
 }  // namespace
 
 int tile_fixed_bits(const LevelDesc<double>& L, int nu) {
-  if (L.varkappa || L.fax >= 0 || L.nz != 1 || nu < 1 || nu > kTileMaxNu) return 0;
-  if (!(L.alpha >= 0.0) || !(L.c > 0.0)) return 0;
-  for (int cls = 0; cls < 16; ++cls) {
+  if (L.fax >= 0 || L.nz != 1 || nu < 1 || nu > kTileMaxNu) return 0;
+  if (L.varkappa && !L.aq) return 0;  // the level's weights were checked when aq was formed
+  if (!L.varkappa && (!(L.alpha >= 0.0) || !(L.c > 0.0))) return 0;
+  for (int cls = 0; cls < 16 && !L.varkappa; ++cls) {
     const int nb = 4 - (cls & 1) - ((cls >> 1) & 1) - ((cls >> 2) & 1) - ((cls >> 3) & 1);
     if ((cls & 3) == 3 || (cls & 12) == 12) continue;  // no cell touches both ends of an axis
     if (!(L.a[cls] > 0.0) || !(L.a[cls] * nb <= 1.0 + 1e-12) || !(L.a[cls] <= 0.5)) return 0;
@@ -929,6 +1132,10 @@ cudaError_t launch_tile_pre(const T* uin, const T* fin, T* fout, T* uout, T* uc,
   a.ordering = ordering;
   a.halo = 2 * nu + 2;
   a.bits = bits;
+  if (L.varkappa) {  // 32-row regions: the coefficients take the registers of two more rows
+    if (tau) return pre_launch<T, 2, 16, true, true, true>(a, L, stream);
+    return uin ? pre_launch<T, 2, 16, true, false, true>(a, L, stream) : pre_launch<T, 2, 16, false, false, true>(a, L, stream);
+  }
   const bool tall = tall_regions(L.nx, L.ny, a.halo, rows, sm_count);
   constexpr int R = kTileR<T>, W = 64 / R, S = kTileRShort<T>, WS = 32 / S;
   if (tau) return tall ? pre_launch<T, R, W, true, true>(a, L, stream) : pre_launch<T, S, WS, true, true>(a, L, stream);
@@ -951,6 +1158,7 @@ cudaError_t launch_tile_post(const T* uin, const T* f, const T* uc, T* uout, dou
   a.halo = 2 * nu;
   a.bits = bits;
   a.scaled = scaled;
+  if (L.varkappa) return post_launch<T, 2, 16, false, true>(a, L, stream);
   constexpr int R = kTileR<T>, W = 64 / R, S = kTileRShort<T>, WS = 32 / S;
   return tall_regions(L.nx, L.ny, a.halo, rows, sm_count) ? post_launch<T, R, W, false>(a, L, stream)
                                                     : post_launch<T, S, WS, false>(a, L, stream);
@@ -973,6 +1181,7 @@ cudaError_t launch_tile_post_norm(const double* uin, const double* f, const doub
   a.halo = norm_halo(nu);
   a.bits = bits;
   a.norm = norm;
+  if (L.varkappa) return post_launch<double, 2, 16, true, true>(a, L, stream);
   constexpr int R = kTileR<double>, W = 64 / R, S = kTileRShort<double>, WS = 32 / S;
   return tall_regions(L.nx, L.ny, a.halo, rows, sm_count) ? post_launch<double, R, W, true>(a, L, stream)
                                                     : post_launch<double, S, WS, true>(a, L, stream);
@@ -994,7 +1203,10 @@ size_t coarse_bytes(const TileCoarse<T>& A) {
 
 template <typename T>
 cudaError_t launch_tile_coarse(const TileCoarse<T>& A, T* utop, const T* ftop, cudaStream_t stream) {
-  k_tile_coarse<T><<<1, 32 * kCoarseWarps<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
+  if (A.varkappa)
+    k_tile_coarse<T, true><<<1, 32 * kCoarseWarps<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
+  else
+    k_tile_coarse<T, false><<<1, 32 * kCoarseWarps<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
   return cudaGetLastError();
 }
 
@@ -1003,10 +1215,12 @@ cudaError_t tile2d_prepare() {
   static cudaError_t err = cudaSuccess;
   std::call_once(once, [] {
     const int most = 200 * 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_tile_coarse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_tile_coarse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    err = e;
+    const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    for (cudaError_t e : {cudaFuncSetAttribute(k_tile_coarse<float, false>, a, most),
+                          cudaFuncSetAttribute(k_tile_coarse<float, true>, a, most),
+                          cudaFuncSetAttribute(k_tile_coarse<double, false>, a, most),
+                          cudaFuncSetAttribute(k_tile_coarse<double, true>, a, most)})
+      if (err == cudaSuccess) err = e;
   });
   return err;
 }

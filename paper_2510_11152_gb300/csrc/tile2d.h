@@ -47,7 +47,7 @@ template <typename T>
 struct TileCoarse {
   const LevelDesc<T>* desc;  // device array, one per level
   const T* cinv;
-  int l0, nlev, nu1, nu2, nuc, ordering, tau;
+  int l0, nlev, nu1, nu2, nuc, ordering, tau, varkappa;
   int bits;                  // tile_fixed_bits for the largest of nu1, nu2, nuc
   int off[kMaxLevels];       // element offset of each level's u in shared memory; f follows it
   int total;                 // elements

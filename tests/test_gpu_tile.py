@@ -87,3 +87,26 @@ def test_tile_float64_nonfinite(cuda_lib, bad):
     with pytest.raises(fas.FasError) as e:
         fas.fas_solve(ctx, _t(np.zeros(shape)), _t(f))
     assert e.value.status == fas.FAS_ENONFINITE
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("shape,bc,nu,contrast", [
+    ((128, 128), (N_,) * 4, 2, 1.0), ((32, 64), (D_, N_, N_, D_), 2, 1.0), ((16, 16), (N_,) * 4, 1, 1.0),
+    ((256, 64), (D_,) * 4, 3, 1e4), ((64, 512), (N_, D_, D_, N_), 2, 1e4), ((256, 512), (N_,) * 4, 4, 1e2)])
+def test_tile_kernels_per_cell_diffusivity(cuda_lib, shape, bc, nu, contrast, precision):
+    """The same with a per-cell diffusivity (weights as 62-bit fractions in float64), up to a jump of 1e4."""
+    fas = cuda_lib
+    u0, f = random_field(shape, 651, -1, 1), noisy_cos_mode(shape, 652)
+    kappa = _t(0.5 + random_field(shape, 653) * np.where(np.arange(shape[1]) < shape[1] // 3, contrast, 1.0)[None, :])
+    out = []
+    for path in (0, 1):
+        ctx = fas.fas_create(fas.make_params(shape, 1.0 / max(shape), beta=2e-3, path=path, bc=bc, nu1=nu, nu2=nu,
+                                             precision=precision), kappa=kappa)
+        u, ft = _t(u0), _t(f)
+        for _ in range(3):
+            fas.fas_vcycle(ctx, u, ft)
+        out.append(u.cpu().numpy())
+    if precision == 1:
+        np.testing.assert_array_equal(out[0], out[1])
+    else:
+        assert np.max(np.abs(out[0] - out[1])) <= 1e-12 * np.max(np.abs(out[1]))
