@@ -706,7 +706,10 @@ __device__ __forceinline__ void pre_run(const P& pol, const TileArgs<T>& a, cons
   Q.publish(0);
   Q.publish(1);
   __syncthreads();
-  if (TAU) Q.tau();  // f changes, u does not: the edges stay valid, and no barrier is needed
+  if (TAU) {
+    Q.tau();
+    __syncthreads();  // it reads the edges of both colours: the first phase must not publish its colour before
+  }
   Q.smooth(a.nu, a.ordering);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool lane_out = g.x >= 0 && g.x < g.nx && 2 * lane >= a.halo && 2 * lane < kTileCols - a.halo;
@@ -937,7 +940,10 @@ __device__ __forceinline__ void coarse_level(const P& pol, const Place& g, int p
   Q.publish(0);
   Q.publish(1);
   Q.meet();
-  if (PASS != Pass::kUp && tau) Q.tau();
+  if (PASS != Pass::kUp && tau) {
+    Q.tau();
+    Q.meet();  // before the first phase publishes its colour
+  }
   Q.smooth(nu, ordering);
   const int lane = threadIdx.x & 31;
 #pragma unroll

@@ -110,3 +110,14 @@ def test_tile_kernels_per_cell_diffusivity(cuda_lib, shape, bc, nu, contrast, pr
         np.testing.assert_array_equal(out[0], out[1])
     else:
         assert np.max(np.abs(out[0] - out[1])) <= 1e-12 * np.max(np.abs(out[1]))
+
+
+@pytest.mark.parametrize("shape,nu", [((128, 128), 2), ((256, 256), 2), ((512, 1024), 3)])
+def test_tile_kernels_repeat(cuda_lib, shape, nu):
+    """A warp that is late in the tau correction must not see the first phase of the others: twenty runs of three
+    float32 cycles, bit for bit."""
+    u0, f = random_field(shape, 661, -1, 1), noisy_cos_mode(shape, 662)
+    kw = dict(nu1=nu, nu2=nu, precision=1, inner_cycles=2)
+    b = _cycles(cuda_lib, shape, 1, u0, f, **kw)
+    for _ in range(20):
+        np.testing.assert_array_equal(_cycles(cuda_lib, shape, 0, u0, f, **kw), b)
