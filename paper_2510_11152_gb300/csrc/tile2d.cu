@@ -876,19 +876,30 @@ __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ T
 
 // ------------------------------------------------------------------------------------------------
 // levels of at most 64 x 64 (float64: 32 x 32) cells: a V-cycle in one block
+//
+// A pass over such a level is bound by the chain of instructions of one thread, with a barrier per phase.
+// float32: two rows per warp, as in the grid-wide kernels (from 64 x 64: 14 us). float64: an update is some thirty
+// integer instructions, so a thread owns one pair of cells, whatever the level's width, and takes all but one of
+// a cell's neighbours from shared memory. With two rows per warp half the lanes of a 32 x 32 level were idle and
+// the others had twice the instructions: a V-cycle from 32 x 32 took 30.3 us, and takes 22.2. In float32 the same
+// split gained nothing (18.0 us either way, with the event's 4 us).
 // ------------------------------------------------------------------------------------------------
 
-constexpr int kCoarseR = 2;  // rows per warp: the pass over a level is one warp's chain of instructions
+constexpr int kCoarseR = 2;  // float32: rows per warp
 template <typename T>
-constexpr int kCoarseWarps = tile_coarse_cells<T>() / kCoarseR;
+constexpr int kCoarseThreads = sizeof(T) == 4 ? 32 * tile_coarse_cells<T>() / kCoarseR
+                                              : tile_coarse_cells<T>() * tile_coarse_cells<T>() / 2;
 
 template <typename T>
-struct CoarseSmem {
-  typename std::conditional<sizeof(T) == 4, Edge<float>, Edge<int64_t>>::type edge[kCoarseWarps<T> + 1];
-  int wmax[kCoarseWarps<T>];
+struct CoarseSmem {  // the rows of the warps (one more: zeros)
+  Edge<float> edge[kCoarseThreads<T> / 32 + 1];
+};
+template <>
+struct CoarseSmem<double> {
+  int64_t v[2][kCoarseThreads<double> + 8];  // the cells of each colour by pair, and a zero after the level's last pair
+  int wmax[kCoarseThreads<double> / 32];
 };
 
-template <typename T>
 __device__ __forceinline__ Place coarse_place(int nx, int ny, int per) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool px = per & 1, py = per & 2;
@@ -907,8 +918,8 @@ __device__ __forceinline__ Place coarse_place(int nx, int ny, int per) {
   g.srcE = (lane + 1) & (np - 1);
   g.noW = !px && lane == 0;
   g.noE = !px && lane == np - 1;
-  g.wu = warp > 0 ? warp - 1 : (py ? nwa - 1 : kCoarseWarps<T>);
-  g.wd = warp + 1 < nwa ? warp + 1 : (py ? 0 : kCoarseWarps<T>);
+  g.wu = warp > 0 ? warp - 1 : (py ? nwa - 1 : kCoarseThreads<float> / 32);
+  g.wd = warp + 1 < nwa ? warp + 1 : (py ? 0 : kCoarseThreads<float> / 32);
   return g;
 }
 
@@ -988,43 +999,207 @@ __device__ __forceinline__ void coarse_load(Raw<T, kCoarseR>& w, const Place& g,
   }
 }
 
-template <Pass PASS, bool VAR, typename T, typename SM>
-__device__ __forceinline__ void coarse_step(const LevelDesc<T>& L, SM& sm, const TileCoarse<T>& A, const T* u,
-                                            const T* f, const T* c, bool tau, bool scaled, int nu, T* su, T* sf, T* cu,
-                                            T* cf) {
-  const Place g = coarse_place<T>(L.nx, L.ny, L.per);
-  Raw<T, kCoarseR> w;
-  coarse_load(w, g, u, f, c);
-  if constexpr (VAR && sizeof(T) == 4) {
-    if (g.active) coarse_level<PASS>(VarF{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
-  } else if constexpr (VAR) {
-    Scale s;
-    if (choose_scale(raw_exp_var<PASS == Pass::kUp>(w, L, g, scaled), A.bits, sm.wmax, kCoarseWarps<T>, &s)) {
-      if (g.active) coarse_level<PASS>(var_x(L, s), g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
-    } else if (g.active) {
-      coarse_level<PASS>(VarD{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+// The thread's cells in float64: pair threadIdx.x of the level (row by row), columns 2 x and 2 x + 1. The slots are
+// indexes into CoarseSmem::v, n for a neighbour beyond a boundary. Sizes are powers of two, at least 2.
+struct Pair {
+  int np, n, x, row, idx;
+  int west, east, up, down;
+  bool in;
+  int xfe, xfo, yf, ylast;
+  int bar;  // threads that meet at a phase's barrier
+  __device__ __forceinline__ Pair(const LevelDesc<double>& L) {
+    const bool px = L.per & 1, py = L.per & 2;
+    np = L.nx >> 1;
+    n = np * L.ny;
+    idx = threadIdx.x;
+    in = idx < n;
+    x = idx & (np - 1);
+    row = idx >> (L.lx - 1);
+    xfe = !px && x == 0 ? 1 : 0;
+    xfo = !px && x == np - 1 ? 2 : 0;
+    ylast = py ? 0 : 8;
+    yf = py ? 0 : ((row == 0) << 2) | ((row == L.ny - 1) << 3);
+    west = x > 0 ? idx - 1 : (px ? idx + np - 1 : n);
+    east = x < np - 1 ? idx + 1 : (px ? idx - x : n);
+    up = row > 0 ? idx - np : (py ? idx + (L.ny - 1) * np : n);
+    down = row < L.ny - 1 ? idx + np : (py ? idx - (L.ny - 1) * np : n);
+    bar = max(32, n);
+  }
+  __device__ __forceinline__ bool odd() const { return row & 1; }
+  // the cell of colour k (1: x + y odd) is the odd column
+  __device__ __forceinline__ bool odd_col(int k) const { return (k == 1) != odd(); }
+  __device__ __forceinline__ void meet() const {
+    if (bar == 32) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"r"(bar) : "memory");
+  }
+};
+
+// As above for one pair per thread, in float64.
+template <Pass PASS, typename P>
+__device__ __forceinline__ void pair_level(const P& pol, const Pair& g, CoarseSmem<double>& sm, const double2 uw,
+                                           const double2 fw, double cw, bool tau, bool scaled, int nu, int ordering,
+                                           double* su, double* sf, double* cu, double* cf) {
+  using V = typename P::V;
+  using A = typename P::A;
+  static_assert(sizeof(V) == 8, "");
+  auto* v = reinterpret_cast<V(*)[kCoarseThreads<double> + 8]>(sm.v);
+  auto id = [&](int k) {
+    const bool o = g.odd_col(k);
+    if (P::kVar) return g.in ? 2 * g.idx + (o ? 1 : 0) : -1;
+    return (o ? g.xfo : g.xfe) | g.yf;
+  };
+  V u[2], f[2];
+  A co[2];
+  int far[2];  // the neighbour in the adjacent pair
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const bool o = g.odd_col(k);
+    u[k] = pol.in(o ? uw.y : uw.x);
+    f[k] = pol.in_f(o ? fw.y : fw.x, id(k), o, scaled);
+    co[k] = g.in ? pol.coef(id(k)) : A{};
+    far[k] = o ? g.east : g.west;
+  }
+  auto publish = [&](int k) {
+    if (g.in) v[k][g.idx] = u[k];
+  };
+  if (threadIdx.x < 2) v[threadIdx.x][g.n] = V(0);
+  publish(0);
+  publish(1);
+  g.meet();
+  if (PASS == Pass::kUp) {  // R(u) with the other row of the row pair
+    const int partner = g.in ? (g.odd() ? g.idx - g.np : g.idx + g.np) : g.n;
+    const V p0 = v[0][partner], p1 = v[1][partner];
+    // avg takes (even row: even, odd column), (odd row: even, odd column)
+    const V d = pol.in(cw) - (g.odd() ? pol.avg(p0, p1, u[1], u[0]) : pol.avg(u[0], u[1], p1, p0));
+    g.meet();
+    u[0] += d;
+    u[1] += d;
+    publish(0);
+    publish(1);
+    g.meet();
+  }
+  auto nb = [&](int k) {
+    const V own = u[1 - k], away = v[1 - k][far[k]], a = v[1 - k][g.up], b = v[1 - k][g.down];
+    return g.odd_col(k) ? Nb4<V>{own, away, a, b} : Nb4<V>{away, own, a, b};
+  };
+  if (PASS != Pass::kUp && tau) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (g.in) f[k] = pol.tau(f[k], u[k], nb(k), co[k], id(k));
+    g.meet();  // before the first phase publishes its colour
+  }
+  auto phase = [&](auto kc) {
+    constexpr int K = decltype(kc)::value;
+    if (g.in) u[K] = pol.update(nb(K), f[K], co[K]);
+    publish(K);
+    g.meet();
+  };
+  for (int t = 0; t < 2 * nu; ++t) {
+    const int c0 = first_colour(ordering, t >> 1);
+    if ((t & 1) ? !c0 : c0)
+      phase(std::integral_constant<int, 1>());
+    else
+      phase(std::integral_constant<int, 0>());
+  }
+  const bool r = g.odd();  // the even column's colour
+  if (g.in) {
+    const double a = pol.out(u[0]), b = pol.out(u[1]);
+    reinterpret_cast<double2*>(su)[g.idx] = r ? make_double2(b, a) : make_double2(a, b);
+    if (PASS == Pass::kDown) {
+      const double c = pol.out_f(f[0]), d = pol.out_f(f[1]);
+      reinterpret_cast<double2*>(sf)[g.idx] = r ? make_double2(d, c) : make_double2(c, d);
     }
-  } else if constexpr (sizeof(T) == 4) {
-    if (g.active) coarse_level<PASS>(RawF{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
-  } else {
-    Scale s;
-    const Mant be = mant_of(L.b[g.xfe]), bo = mant_of(L.b[g.xfo]);
-    if (choose_scale(raw_exp<PASS == Pass::kUp>(w, max(be.E, bo.E) + 1, scaled), A.bits, sm.wmax, kCoarseWarps<T>, &s)) {
-      if (g.active)
-        coarse_level<PASS>(ScaledX<false>{L, s, be, bo}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
-    } else if (g.active) {
-      coarse_level<PASS>(ScaledD{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+  }
+  if (PASS == Pass::kDown) {  // the even rows' threads take the odd rows' cells: u, then the residuals in its place
+    V rho[2], pu[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      rho[k] = g.in ? pol.resid(f[k], u[k], nb(k), co[k], id(k)) : V(0);
+      pu[k] = g.in && !r ? v[k][g.idx + g.np] : V(0);
+    }
+    g.meet();
+    if (g.in && r) {
+      v[0][g.idx] = rho[0];
+      v[1][g.idx] = rho[1];
+    }
+    g.meet();
+    if (g.in && !r) {
+      const V q0 = v[0][g.idx + g.np], q1 = v[1][g.idx + g.np];
+      auto id2 = [&](bool o) {  // the odd row's cells
+        if (P::kVar) return 2 * (g.idx + g.np) + (o ? 1 : 0);
+        return (o ? g.xfo : g.xfe) | (g.idx + 2 * g.np >= g.n ? g.ylast : 0);
+      };
+      const int c = (g.row >> 1) * g.np + g.x;
+      cu[c] = pol.out_avg(u[0], u[1], pu[1], pu[0]);
+      cf[c] = pol.out_avg_r(rho[0], rho[1], q1, q0, id(0), id(1), id2(false), id2(true));
+    }
+  }
+}
+
+template <Pass PASS, bool VAR>
+__device__ __forceinline__ void coarse_step(const LevelDesc<float>& L, CoarseSmem<float>& sm, const TileCoarse<float>& A,
+                                            const float* u, const float* f, const float* c, bool tau, bool scaled,
+                                            int nu, float* su, float* sf, float* cu, float* cf) {
+  const Place g = coarse_place(L.nx, L.ny, L.per);
+  Raw<float, kCoarseR> w;
+  coarse_load(w, g, u, f, c);
+  using P = typename std::conditional<VAR, VarF, RawF>::type;
+  if (g.active) coarse_level<PASS>(P{L}, g, L.per, sm, w, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+  __syncthreads();
+}
+
+template <Pass PASS, bool VAR>
+__device__ __forceinline__ void coarse_step(const LevelDesc<double>& L, CoarseSmem<double>& sm,
+                                            const TileCoarse<double>& A, const double* u, const double* f,
+                                            const double* c, bool tau, bool scaled, int nu, double* su, double* sf,
+                                            double* cu, double* cf) {
+  const Pair g(L);
+  double2 uw{}, fw{};
+  double cw = 0.0;
+  if (g.in) {
+    uw = reinterpret_cast<const double2*>(u)[g.idx];
+    fw = reinterpret_cast<const double2*>(f)[g.idx];
+    if (PASS == Pass::kUp) cw = c[(g.row >> 1) * g.np + g.x];
+  }
+  // the largest exponent of the thread's values (u, c and an upper bound of b f)
+  int e = PASS == Pass::kUp ? exp_field(cw) : 0;
+  const Mant be = VAR ? Mant{} : mant_of(L.b[g.xfe]), bo = VAR ? Mant{} : mant_of(L.b[g.xfo]);
+#pragma unroll
+  for (int o = 0; o < 2; ++o) {
+    e = max(e, exp_field(o ? uw.y : uw.x));
+    const int ef = exp_field(o ? fw.y : fw.x);
+    if (scaled || ef == 0 || ef == 0x7FF) {
+      e = max(e, ef);
+    } else {  // a nonzero f: the pair is in the domain
+      const int eb = VAR ? exp_field(L.h2 * L.rD[2 * g.idx + o]) : max(be.E, bo.E) + 1;
+      e = max(e, max(1, min(0x7FE, ef + eb - 1022)));
+    }
+  }
+  Scale s;
+  const bool fixed = choose_scale(e, A.bits, sm.wmax, kCoarseThreads<double> / 32, &s);
+  if ((int)threadIdx.x < g.bar) {
+    auto run = [&](const auto& pol) {
+      pair_level<PASS>(pol, g, sm, uw, fw, cw, tau, scaled, nu, A.ordering, su, sf, cu, cf);
+    };
+    if constexpr (VAR) {
+      if (fixed) run(var_x(L, s));
+      else run(VarD{L});
+    } else {
+      if (fixed) run(ScaledX<false>{L, s, be, bo});
+      else run(ScaledD{L});
     }
   }
   __syncthreads();
 }
 
 template <typename T, bool VAR>
-__global__ void __launch_bounds__(32 * kCoarseWarps<T>) k_tile_coarse(const __grid_constant__ TileCoarse<T> A, T* utop,
+__global__ void __launch_bounds__(kCoarseThreads<T>) k_tile_coarse(const __grid_constant__ TileCoarse<T> A, T* utop,
                                                                       const T* ftop) {
   extern __shared__ __align__(16) unsigned char tile_smem[];
   auto& sm = *reinterpret_cast<CoarseSmem<T>*>(tile_smem);
-  if (threadIdx.x < 128) reinterpret_cast<T*>(&sm.edge[kCoarseWarps<T>])[threadIdx.x] = T(0);
+  if constexpr (sizeof(T) == 4) {
+    if (threadIdx.x < 128) reinterpret_cast<T*>(&sm.edge[kCoarseThreads<T> / 32])[threadIdx.x] = T(0);
+  }
   T* fields = reinterpret_cast<T*>(tile_smem + (sizeof(CoarseSmem<T>) + 15) / 16 * 16);
   LevelDesc<T>* desc = reinterpret_cast<LevelDesc<T>*>(fields + A.total) - A.l0;
   {
@@ -1210,9 +1385,9 @@ size_t coarse_bytes(const TileCoarse<T>& A) {
 template <typename T>
 cudaError_t launch_tile_coarse(const TileCoarse<T>& A, T* utop, const T* ftop, cudaStream_t stream) {
   if (A.varkappa)
-    k_tile_coarse<T, true><<<1, 32 * kCoarseWarps<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
+    k_tile_coarse<T, true><<<1, kCoarseThreads<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
   else
-    k_tile_coarse<T, false><<<1, 32 * kCoarseWarps<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
+    k_tile_coarse<T, false><<<1, kCoarseThreads<T>, coarse_bytes(A), stream>>>(A, utop, ftop);
   return cudaGetLastError();
 }
 
