@@ -457,7 +457,6 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
         STATUS_TRY(dev_alloc(H, &H.u[l], n));
         STATUS_TRY(dev_alloc(H, &H.f[l], n));
       }
-      if (l > 0) STATUS_TRY(dev_alloc(H, &H.u0[l], n));
     }
     // register-tile path: 2D cell levels of either precision whose coarsest levels fit the single-block
     // tile kernel
@@ -470,8 +469,6 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       while (lc < c->nlev && (c->shape[lc].nx > most || c->shape[lc].ny > most)) ++lc;
       H.tiled = lc < c->nlev && !(p.kappa && c->shape[0].cells() > INT32_MAX);  // cells by 32-bit index there
       H.ntile = H.tiled ? lc : 0;
-      if constexpr (std::is_same<T, double>::value)
-        if (H.tiled && p.kappa) STATUS_TRY(kappa_fractions(c, H));
     }
     // sweep-fused 2D path (float32 only): consecutive levels from the finest that the fused kernels
     // handle and that are larger than the single-CTA switch level
@@ -494,16 +491,23 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       STATUS_TRY(dev_alloc(H, &H.u2[l], c->shape[l].cells()));
       if (l + 1 < H.nfast) STATUS_TRY(dev_alloc(H, &H.rc[l + 1], c->shape[l + 1].cells()));
     }
+    const size_t mark = H.owned.size();
     for (int l = H.nfast; l < H.ntile && H.tiled; ++l) {
-      // without room for the second buffers the levels run the per-operation kernels
+      // without room for the second buffers the levels run the per-operation kernels, and their room is given back
       if (dev_alloc(H, &H.u2[l], c->shape[l].cells()) != FAS_OK ||
           (l > 0 && dev_alloc(H, &H.rc[l], c->shape[l].cells()) != FAS_OK)) {
         cudaGetLastError();
+        for (; H.owned.size() > mark; H.owned.pop_back()) cudaFree(H.owned.back());
+        for (int k = H.nfast; k <= l; ++k) H.u2[k] = H.rc[k] = nullptr;
         H.tiled = false;
         H.ntile = 0;
       }
     }
+    for (int l = 1; l < c->nlev && !H.tiled; ++l)  // the per-operation kernels' restricted start
+      STATUS_TRY(dev_alloc(H, &H.u0[l], c->shape[l].cells()));
     if (H.tiled) {
+      if constexpr (std::is_same<T, double>::value)
+        if (p.kappa) STATUS_TRY(kappa_fractions(c, H));
       TileCoarse<T>& A = H.tile_coarse;
       std::memset(&A, 0, sizeof(A));
       H.tile_bits.assign(c->nlev, 0);
