@@ -55,7 +55,7 @@ typedef enum {
  * relation for it; here the ghost of the first cell is the last cell and vice versa, and the face
  * between them is an interior face). Both faces of an axis must be PERIODIC or neither; periodic axes
  * need cell-centred unknowns and a constant kappa (FAS_EUNSUPPORTED otherwise) and run the
- * per-operation kernels. With alpha = 0 and no Dirichlet face the operator is singular and is handled
+ * register-tile kernels in 2D, the per-operation or (large float32 levels) column kernels in 3D. With alpha = 0 and no Dirichlet face the operator is singular and is handled
  * like the all-Neumann pressure solve (mean-free right-hand side, mean removed after every cycle). */
 typedef enum { FAS_BC_NEUMANN = 0, FAS_BC_DIRICHLET = 1, FAS_BC_PERIODIC = 2 } fas_bc;
 typedef enum { FAS_FP64 = 0, FAS_MIXED = 1 } fas_precision;
@@ -90,11 +90,13 @@ typedef struct {
   int precision;         /* fas_precision: FP64, or FP32 inner cycles in FP64 refinement        */
   int inner_cycles;      /* FAS_MIXED: FP32 V-cycles per refinement step (default 1)          */
   int use_graph;         /* 1: capture repeated launch sequences in CUDA graphs (default 1)     */
-  int path;              /* 0: sweep-fused kernels where the level allows and they pay (default);
+  int path;              /* 0: fused kernels where the level allows and they pay (default);
                           * 1: one kernel per operation everywhere, the 3D restriction and tau
                           *    correction one cell per thread (reference path);
                           * 2: sweep-fused kernels on every level they handle, whatever its size */
-  int seg_rows;          /* rows per warp segment in the fused 2D kernels (0: default 128)      */
+  int seg_rows;          /* rows per warp segment in the sweep-fused 2D kernels (0: up to 128), and
+                          * region height of the register-tile kernels: 0 by size, up to 32: 32
+                          * rows, more: 64 */
   int location;          /* fas_location (default FAS_CELL). Face grids need kappa == NULL and
                           * coarse_exact 0; they run the per-operation kernels                  */
   int ordering;          /* fas_ordering of the X-MCGS sweeps (default FAS_ORDER_FORWARD)       */
@@ -103,8 +105,8 @@ typedef struct {
 /* X-MCGS sweep orderings (Sec. 2.3, the smoother comparison). FORWARD ("1234-1234"): every sweep
  * updates the parity sets in the paper's order, sets 1-2 (2D; 1-4 in 3D: odd index sum) then the
  * rest. SYMMETRIC ("1234-4321"): the sweeps of each smoothing step alternate forward and backward
- * (sets in reverse order), the symmetric Gauss-Seidel analogue; cell-centred unknowns only, and it
- * runs the per-operation kernels. */
+ * (sets in reverse order), the symmetric Gauss-Seidel analogue; cell-centred unknowns only. It runs the
+ * register-tile kernels in 2D and the per-operation kernels in 3D. */
 typedef enum { FAS_ORDER_FORWARD = 0, FAS_ORDER_SYMMETRIC = 1 } fas_ordering;
 
 /* Per-solve report. res0/res are ||f - A u||_2 before the first and after the last cycle
@@ -193,7 +195,7 @@ fas_status fas_solve_batched(fas_ctx* const* ctxs, int count, double* const* u, 
                              fas_info* infos, void* stream);
 
 /* Autotuning of a context's launch parameters: float32 cycles per refinement step (mixed precision,
- * 1..3) and the row-segment length of the sweep-fused kernels (auto, 16, 32, 64, 128), chosen by
+ * 1..3) and seg_rows (auto, 16, 32, 64, 128; see fas_params), chosen by
  * the time of full solves of f from u = 0 (u is overwritten; a scratch field of the finest size).
  * Results are cached per (dim, n, precision) for the process, so contexts of a size already tuned
  * take the cached choice without timing. out (may be NULL) receives the choice and its time. */

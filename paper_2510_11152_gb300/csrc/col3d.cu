@@ -20,9 +20,11 @@
 // each side; 2 nu in post-smoothing), and only the interior is written, to buffers other than the
 // inputs. The expressions per point are those of basic_kernels.cuh: bit for bit the per-operation path.
 //
-// What bounds it: issue slots (about 55 instructions per output cell and launch at nu = 2) a little
-// above the memory floor of 13.5 bytes per cell. The alternative it replaces at nu = 2 is two passes of the
-// sweep-fused kernel (stream3d.cu) or four colour launches, and a pass for the restriction.
+// What bounds it: issue slots and latency at 16 warps per SM (the registers of one block fill it). 512^3,
+// nu = 2, zero start: 0.70 ms, about 110 instructions per output cell (halo cells included), issue slots 63 % busy,
+// 8.8 bytes of DRAM traffic per cell, 1.7 TB/s. With a start field and the tau correction up to 0.95 ms, post-
+// smoothing 0.72 ms. The two passes of the sweep-fused kernel (stream3d.cu) that it replaces took 1.17 ms, the
+// restriction after them 0.28 ms. One body for plain warps (constants in registers) and one for the rest: 869 -> 835 us.
 #include "col3d.h"
 
 #include <algorithm>
