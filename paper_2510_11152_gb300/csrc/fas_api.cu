@@ -451,13 +451,6 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
     H.u.assign(c->nlev, nullptr);
     H.f.assign(c->nlev, nullptr);
     H.u0.assign(c->nlev, nullptr);
-    for (int l = 0; l < c->nlev; ++l) {
-      const int64_t n = c->shape[l].cells();
-      if (l > 0 || level0_buffers) {
-        STATUS_TRY(dev_alloc(H, &H.u[l], n));
-        STATUS_TRY(dev_alloc(H, &H.f[l], n));
-      }
-    }
     // register-tile path: 2D cell levels of either precision whose coarsest levels fit the single-block
     // tile kernel
     H.tiled = false;
@@ -470,6 +463,12 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       H.tiled = lc < c->nlev && !(p.kappa && c->shape[0].cells() > INT32_MAX);  // cells by 32-bit index there
       H.ntile = H.tiled ? lc : 0;
     }
+    auto level_buffers = [&](int l) -> fas_status {
+      STATUS_TRY(dev_alloc(H, &H.u[l], c->shape[l].cells()));
+      return dev_alloc(H, &H.f[l], c->shape[l].cells());
+    };
+    // (the single-block tile kernel holds the levels below its first in shared memory)
+    for (int l = level0_buffers ? 0 : 1; l < c->nlev && (!H.tiled || l <= H.ntile); ++l) STATUS_TRY(level_buffers(l));
     // sweep-fused 2D path (float32 only): consecutive levels from the finest that the fused kernels
     // handle and that are larger than the single-CTA switch level
     H.nfast = 0;
@@ -503,8 +502,10 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
         H.ntile = 0;
       }
     }
-    for (int l = 1; l < c->nlev && !H.tiled; ++l)  // the per-operation kernels' restricted start
+    for (int l = 1; l < c->nlev && !H.tiled; ++l) {  // the per-operation kernels: also the restricted start
+      if (!H.u[l]) STATUS_TRY(level_buffers(l));
       STATUS_TRY(dev_alloc(H, &H.u0[l], c->shape[l].cells()));
+    }
     if (H.tiled) {
       if constexpr (std::is_same<T, double>::value)
         if (p.kappa) STATUS_TRY(kappa_fractions(c, H));
