@@ -112,6 +112,13 @@ __device__ __forceinline__ double from_fixed(int64_t X, Scale s, int k = 0) {
   return f64_of_units(X, s.top - s.bits - k + 63);
 }
 
+// X as a float, by halves (the 64-bit integer conversion runs at the FP64 pipe's rate). The low half is signed: an
+// unsigned one would lie just below 2^32 for a small negative X, where a float has a spacing of 256.
+__device__ __forceinline__ float float_of(int64_t X) {
+  const int lo = (int)(uint32_t)X;
+  return fmaf((float)(int)((X - lo) >> 32), 4294967296.f, (float)lo);
+}
+
 // b as a 64-bit significand (leading one at bit 63) and its biased exponent.
 struct Mant {
   uint32_t hi, lo;
@@ -241,8 +248,7 @@ struct ScaledX {
     return (float)(L.d[cls] * from_fixed(1, s) * (double)ns);
   }
   __device__ __forceinline__ float norm_value(V r, int cls, float fac) const {
-    // by halves: the 64-bit integer conversion runs at the FP64 pipe's rate
-    return fmaf((float)(int)(r >> 32), 4294967296.f, (float)(uint32_t)r) * fac;
+    return float_of(r) * fac;
   }
 };
 
@@ -362,7 +368,7 @@ struct VarX {
   }
   __device__ __forceinline__ float norm_factor(int, float ns) const { return (float)(from_fixed(1, s) * (double)ns); }
   __device__ __forceinline__ float norm_value(V r, int id, float fac) const {
-    return fmaf((float)(int)(r >> 32), 4294967296.f, (float)(uint32_t)r) * fac * f64_to_f32_rn_bits(dh(id));
+    return float_of(r) * fac * f64_to_f32_rn_bits(dh(id));
   }
 };
 
