@@ -142,13 +142,18 @@ __device__ __forceinline__ int exp_field(double x) {
 }
 
 // X in units of 2^(base - 1086), rounded to the nearest float64 (ties to even); the caller's base keeps the
-// result normal (base - 63 .. base are the exponent fields it may get, less one).
-__device__ __forceinline__ double f64_of_units(int64_t X, int base) {
+// result normal (base - 63 .. base are the exponent fields it may get, less one). *stored (nullable): the rounded value,
+// in units.
+__device__ __forceinline__ double f64_of_units(int64_t X, int base, int64_t* stored = nullptr) {
   const uint64_t sign = (uint64_t)X & (1ull << 63);
   const uint64_t A = X < 0 ? (uint64_t)(-X) : (uint64_t)X;
   const int z = __clzll((long long)A);
   const uint64_t n = A << z;  // leading one at bit 63
   const uint64_t q = (n >> 11) + ((((uint32_t)n & 0x7FFu) + 0x3FFu + ((uint32_t)(n >> 11) & 1u)) >> 11);
+  if (stored) {
+    const int64_t B = (int64_t)(z < 11 ? q << (11 - z) : A);  // from z = 11 on X has at most 53 bits
+    *stored = X < 0 ? -B : B;
+  }
   // q has its leading one at bit 52, which adds one to the exponent field; a carry out of the rounding
   // lands there as well
   const uint64_t r = ((uint64_t)(base - z) << 52) + q;

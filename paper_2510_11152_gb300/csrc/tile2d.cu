@@ -111,6 +111,10 @@ __device__ __forceinline__ int64_t to_fixed(double x, Scale s) {
 __device__ __forceinline__ double from_fixed(int64_t X, Scale s, int k = 0) {
   return f64_of_units(X, s.top - s.bits - k + 63);
 }
+// The same, and X becomes the value that was returned.
+__device__ __forceinline__ double round_fixed(int64_t& X, Scale s) {
+  return f64_of_units(X, s.top - s.bits + 63, &X);
+}
 
 // X as a float, by halves (the 64-bit integer conversion runs at the FP64 pipe's rate). The low half is signed: an
 // unsigned one would lie just below 2^32 for a small negative X, where a float has a spacing of 256.
@@ -194,6 +198,7 @@ struct ScaledD {
   __device__ __forceinline__ V in(double x) const { return x; }
   __device__ __forceinline__ V in_f(double x, int cls, bool, bool scaled) const { return scaled ? x : L.b[cls] * x; }
   __device__ __forceinline__ double out(V x) const { return x; }
+  __device__ __forceinline__ double out_round(V& x) const { return x; }
   __device__ __forceinline__ double out_f(V x) const { return x; }
   __device__ __forceinline__ V update(N nb, V f, A c) const { return fma(c.a, nb.sum(), f); }
   __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + fma(-c.a, nb.sum(), u); }
@@ -230,6 +235,7 @@ struct ScaledX {
     return to_fixed_mul(x, !INNER && (cls & 12) ? mant_of(L.b[cls]) : (!INNER && odd ? bo : be), s);
   }
   __device__ __forceinline__ double out(V x) const { return from_fixed(x, s); }
+  __device__ __forceinline__ double out_round(V& x) const { return round_fixed(x, s); }  // x: as stored
   __device__ __forceinline__ double out_f(V x) const { return from_fixed(x, s); }
   __device__ __forceinline__ V update(N nb, V f, A c) const { return times(nb.sum(), c) + f; }
   __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + (u - times(nb.sum(), c)); }
@@ -310,6 +316,7 @@ struct VarD {
     return scaled || id < 0 ? x : (L.h2 * L.rD[id]) * x;
   }
   __device__ __forceinline__ double out(V x) const { return x; }
+  __device__ __forceinline__ double out_round(V& x) const { return x; }
   __device__ __forceinline__ double out_f(V x) const { return x; }
   __device__ __forceinline__ V update(N nb, V f, A c) const { return nsum(nb, c) + f; }
   __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + (u - nsum(nb, c)); }
@@ -353,6 +360,7 @@ struct VarX {
     return scaled || id < 0 ? to_fixed(x, s) : to_fixed_mul(x, mant_of(L.h2 * L.rD[id]), s);
   }
   __device__ __forceinline__ double out(V x) const { return from_fixed(x, s4); }
+  __device__ __forceinline__ double out_round(V& x) const { return round_fixed(x, s4); }
   __device__ __forceinline__ double out_f(V x) const { return from_fixed(x, s); }
   __device__ __forceinline__ V update(N nb, V f, A c) const { return (nsum(nb, c) + f) << 2; }
   __device__ __forceinline__ V tau(V f, V u, N nb, A c, int) const { return f + (units(u) - nsum(nb, c)); }
@@ -469,6 +477,13 @@ struct Region {
     T2 v;
     v.x = pol.out(u[r][odd(r)]);
     v.y = pol.out(u[r][!odd(r)]);
+    return v;
+  }
+  template <typename T2>
+  __device__ __forceinline__ T2 pair_round(int r) {  // and u is then what was returned
+    T2 v;
+    v.x = pol.out_round(u[r][odd(r)]);
+    v.y = pol.out_round(u[r][!odd(r)]);
     return v;
   }
   template <typename T2>
@@ -745,7 +760,8 @@ __device__ __forceinline__ void pre_run(const P& pol, const TileArgs<T>& a, cons
   }
 }
 
-// RES: returns the thread's sum of (ns (f - A u))^2 over its output cells.
+// RES: returns the thread's sum of (ns (f - A u))^2 over its output cells, u as it is stored: near float64's floor the
+// rounding of u is what is left of the residual. So u is rounded and stored first; halo cells are rounded as well.
 template <bool RES, bool INNER, int R, typename P, typename T, typename SM>
 __device__ __forceinline__ float post_run(const P& pol, const TileArgs<T>& a, const Place& g, const RowMap& rm, SM& sm,
                                          const Raw<T, R>& w, int rows) {
@@ -765,14 +781,27 @@ __device__ __forceinline__ float post_run(const P& pol, const TileArgs<T>& a, co
   Q.smooth(a.nu, a.ordering);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool lane_out = g.x >= 0 && g.x < g.nx && 2 * lane >= a.halo && 2 * lane < kTileCols - a.halo;
+  auto writes = [&](int r) {
+    const int q = R * warp + r, y = g.y + r;
+    return lane_out && q >= a.halo && q < rows - a.halo && y >= 0 && y < rm.ny;
+  };
   float acc = 0.f;
   if constexpr (RES) {
+    if (a.uout) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const T2 v = Q.template pair_round<T2>(r);
+        if (writes(r)) *reinterpret_cast<T2*>(a.uout + (int64_t)(g.y + r) * g.nx + g.x) = v;
+      }
+      Q.publish(0);  // the last phase's barrier lies behind: nobody reads the edges
+      Q.publish(1);
+      __syncthreads();
+    }
     const float ns = a.norm.nsp ? *a.norm.nsp : 1.f;
     const float fac0 = pol.norm_factor(0, ns);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const int q = R * warp + r, y = g.y + r;
-      const bool wr = lane_out && q >= a.halo && q < rows - a.halo && y >= 0 && y < rm.ny;
+      const bool wr = writes(r);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const int id = Q.id(r, k);
@@ -780,13 +809,12 @@ __device__ __forceinline__ float post_run(const P& pol, const TileArgs<T>& a, co
         if (wr) acc = fmaf(v, v, acc);
       }
     }
-    if (!a.uout) return acc;
+    return acc;
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int q = R * warp + r, y = g.y + r;
-    if (lane_out && q >= a.halo && q < rows - a.halo && y >= 0 && y < rm.ny) {
-      const int64_t off = (int64_t)y * g.nx + g.x;
+    if (writes(r)) {
+      const int64_t off = (int64_t)(g.y + r) * g.nx + g.x;
       const T2 v = Q.template pair_u<T2>(r);
       if constexpr (sizeof(T) == 4) {
         if (a.u64) {  // the refinement step's float64 update
