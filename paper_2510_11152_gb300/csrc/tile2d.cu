@@ -22,8 +22,8 @@
 // smoothing can reach (a N is an average: each phase adds at most max |B|), so the unit in the last
 // place is 2^-56 of the region's largest value or below, finer than the float64 rounding of that value.
 // The scaled residual rho = B - u + a N = (f - A u) / d needs no cancellation-prone products. Regions whose
-// rows differ by more than 2^10 in magnitude, or hold a non-finite value or exponents far from 1, take
-// float64 arithmetic.
+// threads' patches of cells (2 columns x 2 or 4 rows) differ by more than 2^10 in magnitude, or that hold a non-finite
+// value or exponents far from 1, take float64 arithmetic: a patch in fixed point keeps at least 44 of its bits.
 //
 // What bounds float64: the integer pipe (61 % of its peak, issue slots 54 %, DRAM 17 %) at one block of 16 warps per
 // SM. 4096 x 2048, two sweeps: pre-smoothing 150 us, where four colour launches of 49 us and a residual-restriction
@@ -49,7 +49,7 @@ constexpr int kTileR = 4;
 template <typename T>
 constexpr int kTileRShort = 2;
 constexpr int kTileCols = 64;   // columns per region
-constexpr int kRowSpread = 10;  // binades between the rows of a region that fixed point still takes
+constexpr int kSpread = 10;     // binades between the threads' cells of a region that fixed point still takes
 
 template <typename T>
 struct Vec2;
@@ -569,21 +569,23 @@ struct Region {
 };
 
 // Decide the arithmetic of a float64 region: the largest biased exponent of its values, and whether
-// fixed point may be used. etop: the thread's largest exponent over its values (0: all zero). Every
-// thread of the block takes part; `active` warps count (of nwarps).
+// fixed point may be used: not where the largest value of one thread's patch of cells (2 columns x R rows) lies more
+// than kSpread binades below another's, whichever way the field decays. etop: the thread's largest exponent over its
+// values (0: all zero, which does not limit the scale). Every thread of the block takes part; the first nwarps
+// warps count.
 __device__ __forceinline__ bool choose_scale(int etop, int bits, int* wmax, int nwarps, Scale* s) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m = (int)__reduce_max_sync(kFullMask, (unsigned)etop);
+  const int n = (int)__reduce_min_sync(kFullMask, etop ? (unsigned)etop : 0xFFFu);
   __syncthreads();  // the previous use of wmax is over
-  if (lane == 0) wmax[warp] = m;
+  if (lane == 0) wmax[warp] = (n << 12) | m;
   __syncthreads();
-  int v = lane < nwarps ? wmax[lane] : 0;
-  const int top = (int)__reduce_max_sync(kFullMask, (unsigned)v);
-  if (v == 0) v = top;  // a warp of zeros does not limit the scale
-  const int low = (int)__reduce_min_sync(kFullMask, (unsigned)v);
+  const int v = lane < nwarps ? wmax[lane] : 0xFFF << 12;
+  const int top = (int)__reduce_max_sync(kFullMask, (unsigned)v & 0xFFFu);
+  const int low = (int)__reduce_min_sync(kFullMask, (unsigned)v >> 12);
   s->top = top == 0 ? 1023 : top;
   s->bits = bits;
-  return bits > 0 && s->top >= 300 && s->top <= 1800 && top - low <= kRowSpread;
+  return bits > 0 && s->top >= 300 && s->top <= 1800 && top - low <= kSpread;
 }
 
 // ------------------------------------------------------------------------------------------------
