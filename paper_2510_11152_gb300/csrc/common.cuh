@@ -190,21 +190,6 @@ __device__ __forceinline__ double block_sum(double v) {
   return v;
 }
 
-// The same from one float per thread: the warps' sums in float (the 31 float64 additions of a warp sum hold the FP64 pipe
-// for 2500 cycles per block of 16 warps), then double.
-__device__ __forceinline__ double block_sum_f(float v) {
-  __shared__ double warp_part[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  __syncthreads();  // protect warp_part against a previous use
-  if (lane == 0) warp_part[w] = (double)v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < nw; ++k) s += warp_part[k];
-  return s;
-}
-
 __device__ __forceinline__ float warp_sum_f(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;

@@ -914,7 +914,7 @@ __global__ void __launch_bounds__(32 * NW) k_tile_post(const __grid_constant__ T
     }
   }
   if constexpr (RES)
-    norm_end(a.norm, block_sum_f(acc), blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    norm_end(a.norm, block_sum((double)acc), blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
 
 // ------------------------------------------------------------------------------------------------
