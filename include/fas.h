@@ -221,11 +221,12 @@ fas_status fas_residual(fas_ctx* ctx, int level, const double* u, const double* 
  * S = sum_nb u_nb - M u (M the diagonal's neighbour count plus boundary multiplicities) is summed
  * in integer arithmetic on the significands and rounded once. The sum is exact where the values of a
  * group of four cells of a row (from a multiple of 4) and of their neighbours lie within 2^6 (2D) or 2^5
- * (3D) of one another; wider groups cut values at 2^-59 (2D) or 2^-58 (3D) of the group's largest, below
- * the rounding of a float64 sum. Large 2D levels (more than 2^22 cells, nx a multiple of 128) and small 3D
- * ones (fewer than 2^21 cells, nx a multiple of 128, ny of 8) use kernels that keep to the exact sum within
- * 2^5 (2D: decided per row of 128 cells of one sign; 3D: per four cells) and take the float64 expression of
- * fas_residual elsewhere, as all do for non-finite values; levels whose nx is not a multiple of 4 decide
+ * (3D) of one another; wider groups cut values at 2^-59 (2D) or 2^-58 (3D) of the group's largest, as long as
+ * the largest value of every cell's own stencil lies within 2^3 of that, and take the float64 expression of
+ * fas_residual otherwise: no cell is less accurate than that expression. Large 2D levels (more than 2^22 cells,
+ * nx a multiple of 128) and small 3D ones (fewer than 2^21 cells, nx a multiple of 128, ny of 8) use kernels that
+ * keep to the exact sum within 2^5 (2D: decided per row of 128 cells of one sign; 3D: per four cells) and take the
+ * float64 expression elsewhere, as all do for non-finite values; levels whose nx is not a multiple of 4 decide
  * per cell. r32 is reproducible bit for bit;
  * norm2 sums float32 partials whose grouping depends on how the GPU scheduled the work, so its last
  * bits may vary between calls. u, f DEVICE float64, r32 DEVICE float32, nx*ny(*nz) each. */

@@ -345,12 +345,20 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
       T acc[2];
       bool done = false;
       if constexpr (std::is_same<T, double>::value && DIM == 3) {
-        // both sums by integers at one scale (bits64.cuh), the common value converted once
-        int top = max(max(exp_field(x0v), exp_field(x1v)), exp_field(x2v));
+        // both sums by integers at one scale (bits64.cuh), the common value converted once; at a scale each where the
+        // two cells' neighbours differ much in magnitude
+        int own[2];
+        const int mid = exp_field(x1v);
 #pragma unroll
         for (int q = 0; q < 2; ++q)
-          top = max(top, max(max(exp_field(sv[q]), exp_field(nv[q])), max(exp_field(bo[q]), exp_field(to[q]))));
-        if (sum_range(top)) {
+          own[q] = max(max(mid, exp_field(q ? x2v : x0v)),
+                       max(max(exp_field(sv[q]), exp_field(nv[q])), max(exp_field(bo[q]), exp_field(to[q]))));
+        int top = max(own[0], own[1]);
+        if (min(own[0], own[1]) < top - kGroupSpread) {
+#pragma unroll
+          for (int q = 0; q < 2; ++q) acc[q] = sum6(q ? x1v : x0v, q ? x2v : x1v, sv[q], nv[q], bo[q], to[q]);
+          done = true;
+        } else if (sum_range(top)) {
           const int64_t m = sum_units(x1v, top);
 #pragma unroll
           for (int q = 0; q < 2; ++q)
@@ -627,14 +635,23 @@ struct Group4 {
       if (l < nz - 1 || pz) t.ld(u + (l < nz - 1 ? idx + sz : idx - (nz - 1) * sz));
     }
   }
-  __device__ __forceinline__ int top() const {
-    int m = max(exp_field(w), exp_field(e));
+  // the largest biased exponent of the group's values, and the smallest of its cells' own (of a cell and its neighbours)
+  __device__ __forceinline__ void exponents(int* top, int* low) const {
+    int x[6];
+    x[0] = exp_field(w);
+    x[5] = exp_field(e);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k + 1] = exp_field(c.v[k]);
+    int hi = 0, lo = 0x7FF;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      m = max(m, max(exp_field(c.v[k]), max(exp_field(s.v[k]), exp_field(n.v[k]))));
+      int m = max(max(x[k], x[k + 1]), max(x[k + 2], max(exp_field(s.v[k]), exp_field(n.v[k]))));
       if (DIM == 3) m = max(m, max(exp_field(b.v[k]), exp_field(t.v[k])));
+      hi = max(hi, m);
+      lo = min(lo, m);
     }
-    return m;
+    *top = hi;
+    *low = lo;
   }
   // the neighbours' float64 sum, in the order of nbsum_t
   __device__ __forceinline__ double sum_f64(int k) const {
@@ -650,13 +667,14 @@ struct Group4 {
 //        (exact, rounded once, when the group's values lie within 2^6 (2D) or 2^5 (3D) of one another; cut below
 //        2^-59 (2^-58) of the largest otherwise);
 //   not IR: r (nullable) = fma(c, N, fma(-d, u, f)), N the neighbour sum.
+// Where a cell's own stencil lies more than 2^kGroupSpread below the group's largest value, the group takes float64.
 // About 90 (2D) and 110 (3D) instructions per cell; a thread per cell with its own conversions took 250, the 3D
 // plane-streaming kernel (ir_strip.cu) 247.
 template <int DIM, bool IR>
 __global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<IR, float, double>::type* r, const double* u,
                                                    const double* f, const __grid_constant__ LevelDesc<double> L,
                                                    const __grid_constant__ NormEnd E) {
-  constexpr int BITS = DIM == 2 ? 59 : 58;  // |S| <= (2 DIM + M) 2^BITS < 2^63, M <= 4 DIM
+  constexpr int BITS = !IR ? kSumBits : DIM == 2 ? 59 : 58;  // |S| <= (2 DIM + M) 2^BITS < 2^63, M <= 4 DIM
   const int nx = L.nx, ny = L.ny, nz = L.nz;
   const int lg = L.lx - 2;
   const int64_t ngroups = (int64_t)1 << (lg + L.ly + L.lz);
@@ -672,9 +690,10 @@ __global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<
     q.load(u, idx, x0, j, l, L);
     Quad<double> fq;
     fq.ld(f + idx);
-    int top = q.top();
+    int top, low;
+    q.exponents(&top, &low);
     double rv[4];
-    if (sum_range(top)) {
+    if (low >= top - kGroupSpread && sum_range(top)) {
       int64_t C[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) C[k] = sum_units<BITS>(q.c.v[k], top);
@@ -692,7 +711,7 @@ __global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<
           rv[k] = fma(L.c, sum_value<BITS>(S, top), fma(-L.d[cls], q.c.v[k], fq.v[k]));
         }
       }
-    } else {  // all zero, non-finite values, or values near the ends of the float64 range
+    } else {  // cells of different magnitude, non-finite values, or values near the ends of the float64 range
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         rv[k] = fma(L.c, q.sum_f64(k), fma(-L.d[bclass<DIM>(x0 + k, j, l, nx, ny, nz)], q.c.v[k], fq.v[k]));

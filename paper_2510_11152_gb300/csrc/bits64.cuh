@@ -165,6 +165,10 @@ __device__ __forceinline__ double f64_of_units(int64_t X, int base, int64_t* sto
 // values within 2^7 of the largest; the unit is 2^-60 of it, where a float64 addition rounds at 2^-53 of its
 // result's magnitude). Up to six such values add up without overflow; the sum is rounded once.
 constexpr int kSumBits = 60;
+// Several sums at one scale (the neighbour sums of adjacent cells): only while every sum's own largest value lies within
+// 2^kGroupSpread of the group's. Cutting its up to six values then costs a sum at most 6 2^-57 of its own largest value,
+// no more than float64 additions may.
+constexpr int kGroupSpread = 3;
 // Scale of a sum from the values' largest biased exponent: all zeros take any; false (float64 additions instead) near
 // the ends of the float64 range and for infinities and NaN.
 __device__ __forceinline__ bool sum_range(int& top) {
