@@ -83,7 +83,11 @@ constexpr int64_t kIr4MinCells3D = (int64_t)1 << 21;
 // Largest 3D float64 level whose residual-restriction is spread over lanes (64 x 32 x 32: the same as one thread per coarse
 // cell; below 12 us -> 7, 256 x 128 x 64: 28 us -> 49, its reads being of 2 cells at a time).
 constexpr int64_t kLanesMaxCells3D = (int64_t)1 << 16;
-constexpr int64_t kCol3dMinCells = (int64_t)1 << 21;  // smallest 3D level of the column-streaming kernels
+// Smallest 3D level of the column-streaming kernels. A block walks its planes one after the other, and smaller levels
+// have too few blocks and planes: a cycle on a 128^3 grid takes 166 us without them on level 0 and 184 with, 512 x 64 x 64
+// (planes x rows x columns) 167 against 202, 256 x 32 x 512 225 against 240, 512 x 64 x 256 359 against 399; from 2^24 on
+// they win for every shape measured (256^3: 755 us without, 585 with; 1024 x 128 x 128: 754, 668).
+constexpr int64_t kCol3dMinCells = (int64_t)1 << 24;
 // Smallest 2D level of the sweep-fused kernels: above the register-tile kernels (whose blocks recompute half again as
 // many cells; 4096^2 level of an 8192^2 run, pre-smoothing: 68 us against 89, 2048^2: 29 against 28, 1024^2: 18
 // against 8), and in hierarchies that those do not take.
