@@ -105,8 +105,19 @@ __device__ __forceinline__ bool norm_end(const NormEnd& E, double part, int bloc
   __syncthreads();
   if (!last) return false;
   __threadfence();
+  // loads in batches: one after the other, the ten per thread that a full grid's 2432 partials take cost 6 us
+  constexpr int kBatch = 8;
   double v = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += __ldcg(E.partials + b);
+  for (int b0 = threadIdx.x; b0 < nblocks; b0 += kBatch * blockDim.x) {
+    double x[kBatch];
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int b = b0 + k * (int)blockDim.x;
+      x[k] = b < nblocks ? __ldcg(E.partials + b) : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) v += x[k];
+  }
   v = block_sum(v);
   if (threadIdx.x != 0) return false;
   *E.ticket = 0u;
