@@ -18,7 +18,7 @@ namespace fasmg {
 // paper's sets 1,2 in 2D, sets 1-4 in 3D); colour 0: even (sets 3,4 / 5-8). With the 0-based indices
 // used here the 1-based sum is the 0-based sum plus DIM. Every cell of a colour has only other-colour
 // neighbours, so all of them update at once from the current values.
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ void smooth_colour_range(T* u, const T* f, const LevelDesc<T>& L, int colour,
                                                     int64_t t0, int64_t stride) {
   const int lhx = L.lx - 1;
@@ -30,12 +30,12 @@ __device__ __forceinline__ void smooth_colour_range(T* u, const T* f, const Leve
     const int i = 2 * k + ((colour + DIM + j + l) & 1);
     const int64_t idx = ((int64_t)l * L.ny + j) * L.nx + i;
     if (L.fax >= 0 && frozen(L, i, j, l)) continue;
-    u[idx] = point_update<T, DIM, PER>(u, f, L, idx, i, j, l);
+    u[idx] = point_update<T, DIM, PER, INT>(u, f, L, idx, i, j, l);
   }
 }
 
 // ---- r = f - A u (Sec. 2.2) over a range of cells; returns the thread's sum of (scale*r)^2.
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ float residual_range(T* r, const T* u, const T* f, const LevelDesc<T>& L,
                                                 float nscale, int64_t t0, int64_t stride) {
   // nscale: power-of-two factor applied before squaring (keeps float squares in range)
@@ -45,7 +45,7 @@ __device__ __forceinline__ float residual_range(T* r, const T* u, const T* f, co
     const int i = (int)(idx & (L.nx - 1));
     const int j = (int)((idx >> L.lx) & (L.ny - 1));
     const int l = (int)(idx >> (L.lx + L.ly));
-    const T rv = (L.fax >= 0 && frozen(L, i, j, l)) ? T(0) : residual_point<T, DIM, PER>(u, f, L, idx, i, j, l);
+    const T rv = (L.fax >= 0 && frozen(L, i, j, l)) ? T(0) : residual_point<T, DIM, PER, INT>(u, f, L, idx, i, j, l);
     if (r) r[idx] = rv;
     const float rs = (float)rv * nscale;
     acc = fmaf(rs, rs, acc);
@@ -87,7 +87,7 @@ __device__ __forceinline__ void restrict_range(T* uc, T* uc0, T* fc, const T* u,
 }
 
 // ---- tau correction (Algorithm 1, coarse source term): fc <- fc + A_c uc, fc holding R(r).
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ void tau_range(T* fc, const T* uc, const LevelDesc<T>& Lc, int64_t t0,
                                           int64_t stride) {
   const int64_t n = (int64_t)Lc.nx * Lc.ny * Lc.nz;
@@ -96,7 +96,7 @@ __device__ __forceinline__ void tau_range(T* fc, const T* uc, const LevelDesc<T>
     const int j = (int)((idx >> Lc.lx) & (Lc.ny - 1));
     const int l = (int)(idx >> (Lc.lx + Lc.ly));
     if (Lc.fax >= 0 && frozen(Lc, i, j, l)) continue;
-    fc[idx] = fc[idx] + apply_point<T, DIM, PER>(uc, Lc, idx, i, j, l);
+    fc[idx] = fc[idx] + apply_point<T, DIM, PER, INT>(uc, Lc, idx, i, j, l);
   }
 }
 
@@ -267,9 +267,9 @@ __device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * block
 template <typename T, int DIM>
 __global__ void k_smooth_colour(T* u, const T* f, LevelDesc<T> L, int colour) {
   if (L.per)
-    smooth_colour_range<T, DIM, true>(u, f, L, colour, gtid(), gstride());
+    smooth_colour_range<T, DIM, true, true>(u, f, L, colour, gtid(), gstride());
   else
-    smooth_colour_range<T, DIM, false>(u, f, L, colour, gtid(), gstride());
+    smooth_colour_range<T, DIM, false, true>(u, f, L, colour, gtid(), gstride());
 }
 
 // One colour phase with a thread per group of 4 consecutive cells of a row (nx a multiple of 4,
@@ -356,7 +356,7 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
         int top = max(own[0], own[1]);
         if (min(own[0], own[1]) < top - kGroupSpread) {
 #pragma unroll
-          for (int q = 0; q < 2; ++q) acc[q] = sum6(q ? x1v : x0v, q ? x2v : x1v, sv[q], nv[q], bo[q], to[q]);
+          for (int q = 0; q < 2; ++q) acc[q] = sum6<true>(q ? x1v : x0v, q ? x2v : x1v, sv[q], nv[q], bo[q], to[q]);
           done = true;
         } else if (sum_range(top)) {
           const int64_t m = sum_units(x1v, top);
@@ -403,8 +403,8 @@ __global__ void __launch_bounds__(256, 3) k_smooth_colour4(T* u, const T* f, Lev
 // r (nullable) = f - A u, and the norm of the residual (scaled by s = *E.nsp before squaring).
 template <typename T, int DIM>
 __global__ void k_residual(T* r, const T* u, const T* f, LevelDesc<T> L, const __grid_constant__ NormEnd E) {
-  const float acc = L.per ? residual_range<T, DIM, true>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride())
-                          : residual_range<T, DIM, false>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride());
+  const float acc = L.per ? residual_range<T, DIM, true, true>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride())
+                          : residual_range<T, DIM, false, true>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride());
   norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
@@ -424,9 +424,9 @@ __global__ void k_restrict(T* uc, T* uc0, T* fc, const T* u, const T* r, int nxf
 template <typename T, int DIM>
 __global__ void k_tau(T* fc, const T* uc, LevelDesc<T> Lc) {
   if (Lc.per)
-    tau_range<T, DIM, true>(fc, uc, Lc, gtid(), gstride());
+    tau_range<T, DIM, true, true>(fc, uc, Lc, gtid(), gstride());
   else
-    tau_range<T, DIM, false>(fc, uc, Lc, gtid(), gstride());
+    tau_range<T, DIM, false, true>(fc, uc, Lc, gtid(), gstride());
 }
 
 template <typename T, int DIM>
@@ -602,8 +602,8 @@ __global__ void k_ir_residual(float* r32, const double* u, const double* b, Leve
         }
       }
       if (!done)
-        r = L.per ? residual_point<double, DIM, true>(u, b, L, idx, i, j, l)
-                  : residual_point<double, DIM, false>(u, b, L, idx, i, j, l);
+        r = L.per ? residual_point<double, DIM, true, true>(u, b, L, idx, i, j, l)
+                  : residual_point<double, DIM, false, true>(u, b, L, idx, i, j, l);
       rv = f64_to_f32_rn_bits(r);
     }
     r32[idx] = rv;
@@ -866,7 +866,7 @@ __device__ void coarse_smooth(T* u, const T* f, const LevelDesc<T>& L, int sweep
 // Single-CTA V-cycle with every level held in shared memory: levels l0..nlev-1 of u and f, and the
 // restricted start u0 of the coarser ones. Same steps and same per-point arithmetic as the grid-wide
 // kernels (the residual is evaluated per child inside the restriction instead of being stored
-// first), so the results are identical; the latency of each dependent step is a shared-memory round
+// first), so the results are identical but for the rounding of 3D float64 neighbour sums (sum6); the latency of each dependent step is a shared-memory round
 // trip instead of an L2 one.
 // ------------------------------------------------------------------------------------------------
 struct SmemLayout {
@@ -874,7 +874,7 @@ struct SmemLayout {
   int64_t total;                                                      // elements
 };
 
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ void restrict_resid_range(T* uc, T* uc0, T* fc, const T* u, const T* f,
                                                      const LevelDesc<T>& L, int64_t t0, int64_t stride) {
   const int nxf = L.nx, nyf = L.ny, nzf = L.nz;
@@ -896,7 +896,7 @@ __device__ __forceinline__ void restrict_resid_range(T* uc, T* uc0, T* fc, const
     for (int k = 0; k < (DIM == 3 ? 8 : 4); ++k) {
       const int di = k & 1, dj = (k >> 1) & 1, dl = (k >> 2) & 1;
       const int64_t idx = base + di + dj * sy + dl * sz;
-      r[k] = residual_point<T, DIM, PER>(u, f, L, idx, i0 + di, j0 + dj, l0 + dl);
+      r[k] = residual_point<T, DIM, PER, INT>(u, f, L, idx, i0 + di, j0 + dj, l0 + dl);
     }
     // same association as avg_children: (c00 + c01) + (c10 + c11) [+ the upper z layer]
     T sr = (r[0] + r[1]) + (r[2] + r[3]);
@@ -912,7 +912,7 @@ __device__ __forceinline__ void restrict_resid_range(T* uc, T* uc0, T* fc, const
 // Face-grid counterpart: the fine residual is evaluated at each fine face the Appendix D weights
 // touch (the three normal slots overlap between neighbouring coarse faces, so some are evaluated
 // twice); the arithmetic per value equals that of k_residual followed by k_restrict_face.
-template <typename T, int DIM, int FAX>
+template <typename T, int DIM, int FAX, bool INT = false>
 __device__ __forceinline__ void restrict_resid_face_range(T* uc, T* uc0, T* fc, const T* u, const T* f,
                                                           const LevelDesc<T>& L, int64_t t0, int64_t stride) {
   const int nxf = L.nx, nyf = L.ny;
@@ -920,7 +920,7 @@ __device__ __forceinline__ void restrict_resid_face_range(T* uc, T* uc0, T* fc, 
   const int64_t nc = (int64_t)nxc * nyc * nzc;
   const int lxc = L.lx - 1, lyc = L.ly - 1;
   auto resid = [&](int64_t q, int i, int j, int l) {
-    return frozen(L, i, j, l) ? T(0) : residual_point<T, DIM>(u, f, L, q, i, j, l);
+    return frozen(L, i, j, l) ? T(0) : residual_point<T, DIM, false, INT>(u, f, L, q, i, j, l);
   };
   for (int64_t I = t0; I < nc; I += stride) {
     const int ic = (int)(I & (nxc - 1));
@@ -941,11 +941,11 @@ template <typename T, int DIM, int FAX>
 __global__ void k_restrict_resid(T* uc, T* uc0, T* fc, const T* u, const T* f, LevelDesc<T> L) {
   if constexpr (FAX < 0) {
     if (L.per)
-      restrict_resid_range<T, DIM, true>(uc, uc0, fc, u, f, L, gtid(), gstride());
+      restrict_resid_range<T, DIM, true, true>(uc, uc0, fc, u, f, L, gtid(), gstride());
     else
-      restrict_resid_range<T, DIM, false>(uc, uc0, fc, u, f, L, gtid(), gstride());
+      restrict_resid_range<T, DIM, false, true>(uc, uc0, fc, u, f, L, gtid(), gstride());
   } else
-    restrict_resid_face_range<T, DIM, FAX>(uc, uc0, fc, u, f, L, gtid(), gstride());
+    restrict_resid_face_range<T, DIM, FAX, true>(uc, uc0, fc, u, f, L, gtid(), gstride());
 }
 
 // The same for 3D float64 levels with constant kappa, with the fine residuals of a coarse cell spread over the lanes of
@@ -971,8 +971,8 @@ __global__ void __launch_bounds__(256) k_restrict_resid_lanes(double* uc, double
       const int i = 2 * c3[0] + (q & 1), j = 2 * c3[1] + ((q >> 1) & 1), l = 2 * c3[2] + (q >> 2);
       const int64_t idx = (int64_t)l * sz + (int64_t)j * sy + i;
       su = u[idx];
-      sr = L.per ? residual_point<double, 3, true>(u, f, L, idx, i, j, l)
-                 : residual_point<double, 3, false>(u, f, L, idx, i, j, l);
+      sr = L.per ? residual_point<double, 3, true, true>(u, f, L, idx, i, j, l)
+                 : residual_point<double, 3, false, true>(u, f, L, idx, i, j, l);
     } else {
       constexpr int T1 = FAX == 0 ? 1 : 0, T2 = FAX == 2 ? 1 : 2;
       const bool wall = wall_slot<FAX>(c3[0], c3[1], c3[2], nxc, nyc, nzc);
@@ -987,7 +987,7 @@ __global__ void __launch_bounds__(256) k_restrict_resid_lanes(double* uc, double
           const double wt = w == 1 ? 0.5 : 0.25;
           su = fma(wt, u[idx], su);
           if (!frozen(L, f3[0], f3[1], f3[2]))
-            sr = fma(wt, residual_point<double, 3>(u, f, L, idx, f3[0], f3[1], f3[2]), sr);
+            sr = fma(wt, residual_point<double, 3, false, true>(u, f, L, idx, f3[0], f3[1], f3[2]), sr);
         }
       }
     }

@@ -68,11 +68,13 @@ __device__ __forceinline__ bool frozen(const LevelDesc<T>& L, int i, int j, int 
   return (L.fax == 0 && i == L.nx - 1) || (L.fax == 1 && j == L.ny - 1) || (L.fax == 2 && l == L.nz - 1);
 }
 
-// The six neighbours' sum of a 3D cell, (w + e) + (s + n) + (bo + to). In float64 by integers (bits64.cuh): five
-// float64 additions keep the FP64 pipe busy for 320 issue slots, the integer sum takes about 90.
-template <typename T>
+// The six neighbours' sum of a 3D cell, (w + e) + (s + n) + (bo + to). INT: in float64 by integers (bits64.cuh). Five
+// float64 additions keep the FP64 pipe busy for 320 issue slots, the integer sum takes about 90, so the kernels that fill
+// the GPU use it; the single-block kernels wait for one thread's chain, which is shorter in float64 (a V-cycle from 8^3:
+// 27 us, 47 with integers).
+template <bool INT, typename T>
 __device__ __forceinline__ T sum6(T w, T e, T s, T n, T bo, T to) {
-  if constexpr (std::is_same<T, double>::value) {
+  if constexpr (INT && std::is_same<T, double>::value) {
     int top = max(max(max(exp_field(w), exp_field(e)), max(exp_field(s), exp_field(n))),
                         max(exp_field(bo), exp_field(to)));
     if (sum_range(top))
@@ -86,7 +88,7 @@ __device__ __forceinline__ T sum6(T w, T e, T s, T n, T bo, T to) {
 // Sum of the existing neighbours of cell (i, j, l) at linear index idx (constant kappa); on a periodic
 // axis (bit of per) the neighbour across the boundary is the wrapped cell. PER = false is the code for
 // levels without periodic axes.
-template <typename T, int DIM, bool PER>
+template <typename T, int DIM, bool PER, bool INT>
 __device__ __forceinline__ T nbsum_t(const T* __restrict__ u, int64_t idx, int i, int j, int l, int nx, int ny,
                                      int nz, int per) {
   const int64_t sy = nx, sz = (int64_t)nx * ny;
@@ -98,7 +100,7 @@ __device__ __forceinline__ T nbsum_t(const T* __restrict__ u, int64_t idx, int i
     if (DIM == 3) {
       T bo = l > 0 ? u[idx - sz] : T(0);
       T to = l < nz - 1 ? u[idx + sz] : T(0);
-      return sum6(w, e, s, n, bo, to);
+      return sum6<INT>(w, e, s, n, bo, to);
     }
     return (w + e) + (s + n);
   } else {
@@ -110,7 +112,7 @@ __device__ __forceinline__ T nbsum_t(const T* __restrict__ u, int64_t idx, int i
     if (DIM == 3) {
       T bo = (l > 0 || (per & 4)) ? u[l > 0 ? idx - sz : idx + (nz - 1) * sz] : T(0);
       T to = (l < nz - 1 || (per & 4)) ? u[l < nz - 1 ? idx + sz : idx - (nz - 1) * sz] : T(0);
-      return sum6(w, e, s, n, bo, to);
+      return sum6<INT>(w, e, s, n, bo, to);
     }
     return (w + e) + (s + n);
   }
@@ -135,7 +137,7 @@ __device__ __forceinline__ T nbsum_w(const T* __restrict__ u, const LevelDesc<T>
 
 // Gauss-Seidel point update of cell (i, j, l): the new value from the current neighbours. PER: the
 // level may have periodic axes (the kernels choose the instantiation once from the descriptor).
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ T point_update(const T* __restrict__ u, const T* __restrict__ f,
                                           const LevelDesc<T>& L, int64_t idx, int i, int j, int l) {
   if (L.varkappa) {
@@ -143,12 +145,12 @@ __device__ __forceinline__ T point_update(const T* __restrict__ u, const T* __re
     return fma(L.h2, f[idx], nw) * L.rD[idx];
   }
   const int cls = bclass<DIM>(i, j, l, L.nx, L.ny, L.nz);
-  T nb = nbsum_t<T, DIM, PER>(u, idx, i, j, l, L.nx, L.ny, L.nz, L.per);
+  T nb = nbsum_t<T, DIM, PER, INT>(u, idx, i, j, l, L.nx, L.ny, L.nz, L.per);
   return fma(L.a[cls], nb, L.b[cls] * f[idx]);
 }
 
 // (A u) at cell (i, j, l).
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ T apply_point(const T* __restrict__ u, const LevelDesc<T>& L, int64_t idx, int i,
                                          int j, int l) {
   if (L.varkappa) {
@@ -156,12 +158,12 @@ __device__ __forceinline__ T apply_point(const T* __restrict__ u, const LevelDes
     return fma(L.Dh[idx], u[idx], -L.ih2 * nw);
   }
   const int cls = bclass<DIM>(i, j, l, L.nx, L.ny, L.nz);
-  T nb = nbsum_t<T, DIM, PER>(u, idx, i, j, l, L.nx, L.ny, L.nz, L.per);
+  T nb = nbsum_t<T, DIM, PER, INT>(u, idx, i, j, l, L.nx, L.ny, L.nz, L.per);
   return fma(L.d[cls], u[idx], -L.c * nb);
 }
 
 // Residual f - A u at cell (i, j, l).
-template <typename T, int DIM, bool PER = false>
+template <typename T, int DIM, bool PER = false, bool INT = false>
 __device__ __forceinline__ T residual_point(const T* __restrict__ u, const T* __restrict__ f,
                                             const LevelDesc<T>& L, int64_t idx, int i, int j, int l) {
   if (L.varkappa) {
@@ -169,7 +171,7 @@ __device__ __forceinline__ T residual_point(const T* __restrict__ u, const T* __
     return fma(L.ih2, nw, fma(-L.Dh[idx], u[idx], f[idx]));
   }
   const int cls = bclass<DIM>(i, j, l, L.nx, L.ny, L.nz);
-  T nb = nbsum_t<T, DIM, PER>(u, idx, i, j, l, L.nx, L.ny, L.nz, L.per);
+  T nb = nbsum_t<T, DIM, PER, INT>(u, idx, i, j, l, L.nx, L.ny, L.nz, L.per);
   return fma(L.c, nb, fma(-L.d[cls], u[idx], f[idx]));
 }
 
