@@ -88,6 +88,11 @@ constexpr int64_t kLanesMaxCells3D = (int64_t)1 << 16;
 // (planes x rows x columns) 167 against 202, 256 x 32 x 512 225 against 240, 512 x 64 x 256 359 against 399; from 2^24 on
 // they win for every shape measured (256^3: 755 us without, 585 with; 1024 x 128 x 128: 754, 668).
 constexpr int64_t kCol3dMinCells = (int64_t)1 << 24;
+// Largest grid with a per-cell diffusivity whose hierarchy runs the register-tile kernels in float64: they read eight
+// more words per cell (the fractions), and on larger grids the per-operation kernels are faster (a cycle of a solve on 1024^2:
+// 285 us against 288 per operation, 512^2: 123 against 179; but 2048 x 1024: 480 against 453, 2048^2: 843 against 667). In
+// float32 (cells by 32-bit index) they win throughout.
+constexpr int64_t kTileMaxCellsKappa = (int64_t)1 << 20;
 // Smallest 2D level of the sweep-fused kernels: above the register-tile kernels (whose blocks recompute half again as
 // many cells; 4096^2 level of an 8192^2 run, pre-smoothing: 68 us against 89, 2048^2: 29 against 28, 1024^2: 18
 // against 8), and in hierarchies that those do not take.
@@ -464,7 +469,8 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       int lc = 0;
       const int most = tile_coarse_cells<T>();
       while (lc < c->nlev && (c->shape[lc].nx > most || c->shape[lc].ny > most)) ++lc;
-      H.tiled = lc < c->nlev && !(p.kappa && c->shape[0].cells() > INT32_MAX);  // cells by 32-bit index there
+      const int64_t most_cells = !p.kappa ? INT64_MAX : sizeof(T) == 8 ? kTileMaxCellsKappa : INT32_MAX;
+      H.tiled = lc < c->nlev && c->shape[0].cells() <= most_cells;
       H.ntile = H.tiled ? lc : 0;
     }
     auto level_buffers = [&](int l) -> fas_status {
