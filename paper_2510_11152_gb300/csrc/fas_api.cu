@@ -554,12 +554,15 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
         while (H.ncol < H.switch_level && col3d_supported(H.desc[H.ncol], p.nu1) &&
                col3d_supported(H.desc[H.ncol], p.nu2) && c->shape[H.ncol].cells() >= kCol3dMinCells)
           H.ncol++;
+        const size_t first = H.owned.size();
         for (int l = 0; l < H.ncol; ++l)
           if (dev_alloc(H, &H.u2[l], c->shape[l].cells()) != FAS_OK ||
               (l > 0 && dev_alloc(H, &H.rc[l], c->shape[l].cells()) != FAS_OK)) {
             cudaGetLastError();
+            for (; H.owned.size() > first; H.owned.pop_back()) cudaFree(H.owned.back());
             H.ncol = 0;
             std::fill(H.u2.begin(), H.u2.end(), nullptr);
+            std::fill(H.rc.begin(), H.rc.end(), nullptr);
           }
       }
       if (p.dim == 3 && p.path != 1 && H.ncol == 0 && p.ordering == FAS_ORDER_FORWARD && p.nu1 + p.nu2 >= 2)
