@@ -28,7 +28,6 @@
 #include "col3d.h"
 
 #include <algorithm>
-#include <mutex>
 
 #include "cp_async.cuh"
 
@@ -482,15 +481,12 @@ cudaError_t launch_col3d_post(const float* uin, const float* f, const float* uc,
 }
 
 cudaError_t col3d_prepare() {
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  std::call_once(once, [] {
-    for (cudaError_t e : {col_attr<1, false, true, false>(), col_attr<1, false, false, false>(),
-                          col_attr<1, true, false, false>(), col_attr<1, false, false, true>(),
-                          col_attr<2, false, true, false>(), col_attr<2, false, false, false>(),
-                          col_attr<2, true, false, false>(), col_attr<2, false, false, true>()})
-      if (err == cudaSuccess) err = e;
-  });
+  cudaError_t err = cudaSuccess;
+  for (cudaError_t e : {col_attr<1, false, true, false>(), col_attr<1, false, false, false>(),
+                        col_attr<1, true, false, false>(), col_attr<1, false, false, true>(),
+                        col_attr<2, false, true, false>(), col_attr<2, false, false, false>(),
+                        col_attr<2, true, false, false>(), col_attr<2, false, false, true>()})
+    if (err == cudaSuccess) err = e;
   return err;
 }
 

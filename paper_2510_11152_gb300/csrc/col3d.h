@@ -19,7 +19,7 @@ cudaError_t launch_col3d_pre(const float* uin, const float* fin, float* fout, fl
 cudaError_t launch_col3d_post(const float* uin, const float* f, const float* uc, float* uout,
                               const LevelDesc<float>& L, int nu, int sm_count, cudaStream_t stream);
 
-// Shared-memory attributes (once per process; before launching or capturing).
+// Shared-memory attributes on the current device (before launching or capturing).
 cudaError_t col3d_prepare();
 
 }  // namespace fasmg

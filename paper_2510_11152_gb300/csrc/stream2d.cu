@@ -544,19 +544,15 @@ cudaError_t pre_attr() {
   return e;
 }
 
-// Shared-memory size attributes of every fused kernel, set once before any launch or stream capture.
+// Shared-memory size attributes of every fused kernel, set before any launch or stream capture (they belong to the
+// current device).
 cudaError_t stream2d_prepare() {
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  std::call_once(once, [] {
-    const int big = (int)(sizeof(Ring<true>) * kWarps);
-    cudaError_t e = cudaFuncSetAttribute(k_post<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_post<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    if (e == cudaSuccess) e = pre_attr<1>();
-    if (e == cudaSuccess) e = pre_attr<2>();
-    err = e;
-  });
-  return err;
+  const int big = (int)(sizeof(Ring<true>) * kWarps);
+  cudaError_t e = cudaFuncSetAttribute(k_post<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_post<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = pre_attr<1>();
+  if (e == cudaSuccess) e = pre_attr<2>();
+  return e;
 }
 
 template <int NS, bool UPD>

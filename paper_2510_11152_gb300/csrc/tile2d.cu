@@ -33,7 +33,6 @@
 
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 #include <type_traits>
 
 #include "basic_kernels.cuh"
@@ -1435,17 +1434,14 @@ cudaError_t launch_tile_coarse(const TileCoarse<T>& A, T* utop, const T* ftop, c
 }
 
 cudaError_t tile2d_prepare() {
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  std::call_once(once, [] {
-    const int most = 200 * 1024;
-    const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    for (cudaError_t e : {cudaFuncSetAttribute(k_tile_coarse<float, false>, a, most),
-                          cudaFuncSetAttribute(k_tile_coarse<float, true>, a, most),
-                          cudaFuncSetAttribute(k_tile_coarse<double, false>, a, most),
-                          cudaFuncSetAttribute(k_tile_coarse<double, true>, a, most)})
-      if (err == cudaSuccess) err = e;
-  });
+  const int most = 200 * 1024;
+  const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t err = cudaSuccess;
+  for (cudaError_t e : {cudaFuncSetAttribute(k_tile_coarse<float, false>, a, most),
+                        cudaFuncSetAttribute(k_tile_coarse<float, true>, a, most),
+                        cudaFuncSetAttribute(k_tile_coarse<double, false>, a, most),
+                        cudaFuncSetAttribute(k_tile_coarse<double, true>, a, most)})
+    if (err == cudaSuccess) err = e;
   return err;
 }
 

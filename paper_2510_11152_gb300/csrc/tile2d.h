@@ -55,7 +55,7 @@ struct TileCoarse {
 template <typename T>
 cudaError_t launch_tile_coarse(const TileCoarse<T>& A, T* utop, const T* ftop, cudaStream_t stream);
 
-// Shared-memory attributes (once per process; before launching or capturing).
+// Shared-memory attributes on the current device (before launching or capturing).
 cudaError_t tile2d_prepare();
 
 }  // namespace fasmg
