@@ -831,6 +831,11 @@ int seg_for_level(const fas_ctx* c, int nx, int ny) {
   return (int)std::max<int64_t>(8, std::min<int64_t>(128, (seg + 7) / 8 * 8));
 }
 
+// The status of a launcher that reports (and thereby clears) its launch error itself.
+fas_status launched(cudaError_t e, const char* what) {
+  return e == cudaSuccess ? FAS_OK : fail(FAS_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
+}
+
 // Levels lfrom..ntile-1 through the register-tile kernels around the single-block tile kernel. Level
 // lfrom works on (utop, ftop); tau: ftop holds R(r) of a finer level, and f is formed from it (into
 // H.f[lfrom]). zero_init: the initial guess of level lfrom is 0 (utop is not read). u64 (nullable, float32
@@ -841,41 +846,39 @@ fas_status vcycle_tile(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T* ftop
                        double* u64, const NormEnd* norm = nullptr) {
   const fas_params& p = c->p;
   const int lc = H.ntile;
-  auto tried = [](cudaError_t e, const char* what) {
-    return e == cudaSuccess ? FAS_OK : fail(FAS_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
-  };
   // the small levels (from the switch level on) are timed as the coarse family, whichever kernels run them
   auto family = [&](int l, int fam) { return l >= H.switch_level && l > lfrom ? (int)FAS_K_COARSE : fam; };
   for (int l = lfrom; l < lc; ++l) {
     const bool top = l == lfrom, t = !top || tau;
     Prof pr(c, family(l, FAS_K_SMOOTH), l, (double)c->shape[l].cells());
-    STATUS_TRY(tried(launch_tile_pre<T>(top ? (zero_init ? nullptr : utop) : H.u[l], top ? ftop : H.rc[l],
-                                        t ? H.f[l] : nullptr, H.u2[l], H.u[l + 1], l + 1 < lc ? H.rc[l + 1] : H.f[l + 1],
-                                        H.desc[l], p.nu1, p.ordering, t, H.tile_bits[l], p.seg_rows, c->sm_count, c->stream),
-                     "tile pre"));
+    STATUS_TRY(launched(launch_tile_pre<T>(top ? (zero_init ? nullptr : utop) : H.u[l], top ? ftop : H.rc[l],
+                                           t ? H.f[l] : nullptr, H.u2[l], H.u[l + 1], l + 1 < lc ? H.rc[l + 1] : H.f[l + 1],
+                                           H.desc[l], p.nu1, p.ordering, t, H.tile_bits[l], p.seg_rows, c->sm_count,
+                                           c->stream),
+                        "tile pre"));
   }
   {
     Prof pr(c, FAS_K_COARSE, lc, (double)c->shape[lc].cells());
     TileCoarse<T> A = H.tile_coarse;
     A.tau = lc > lfrom || tau;
-    STATUS_TRY(tried(launch_tile_coarse<T>(A, lc == lfrom ? utop : H.u[lc], lc == lfrom ? ftop : H.f[lc], c->stream),
-                     "tile coarse"));
+    STATUS_TRY(launched(launch_tile_coarse<T>(A, lc == lfrom ? utop : H.u[lc], lc == lfrom ? ftop : H.f[lc], c->stream),
+                        "tile coarse"));
   }
   for (int l = lc - 1; l >= lfrom; --l) {
     const bool top = l == lfrom, t = !top || tau;
     Prof pr(c, family(l, (l == 0 && u64) ? FAS_K_UPDATE : FAS_K_PROLONG), l, (double)c->shape[l].cells());
     if constexpr (std::is_same<T, double>::value) {
       if (top && norm) {
-        STATUS_TRY(tried(launch_tile_post_norm(H.u2[l], ftop, H.u[l + 1], utop, H.desc[l], p.nu2, p.ordering,
-                                               H.tile_bits[l], *norm, p.seg_rows, c->sm_count, c->stream),
-                         "tile post"));
+        STATUS_TRY(launched(launch_tile_post_norm(H.u2[l], ftop, H.u[l + 1], utop, H.desc[l], p.nu2, p.ordering,
+                                                  H.tile_bits[l], *norm, p.seg_rows, c->sm_count, c->stream),
+                            "tile post"));
         continue;
       }
     }
-    STATUS_TRY(tried(launch_tile_post<T>(H.u2[l], t ? H.f[l] : ftop, H.u[l + 1], top ? utop : H.u[l],
-                                         l == 0 ? u64 : nullptr, H.desc[l], p.nu2, p.ordering,
-                                         t && sizeof(T) == 8, H.tile_bits[l], p.seg_rows, c->sm_count, c->stream),
-                     "tile post"));
+    STATUS_TRY(launched(launch_tile_post<T>(H.u2[l], t ? H.f[l] : ftop, H.u[l + 1], top ? utop : H.u[l],
+                                            l == 0 ? u64 : nullptr, H.desc[l], p.nu2, p.ordering,
+                                            t && sizeof(T) == 8, H.tile_bits[l], p.seg_rows, c->sm_count, c->stream),
+                        "tile post"));
   }
   return FAS_OK;
 }
@@ -994,18 +997,21 @@ void launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b
 }
 
 // The norm of b - A u; mixed precision also leaves r32 = (float)(b - A u) in h32.f[0]
-void enqueue_residual_norm(fas_ctx* c, const double* u, const double* b, const NormEnd& E) {
+fas_status enqueue_residual_norm(fas_ctx* c, const double* u, const double* b, const NormEnd& E) {
   const Hier<double>& H = c->h64;
   if (c->p.precision == FAS_MIXED) {
     launch_ir_residual(c, c->h32.f[0], u, b, E);
   } else if (H.tiled && H.ntile > 0) {
     Prof pr(c, FAS_K_RESIDUAL, 0, (double)c->shape[0].cells());
-    launch_tile_post_norm(u, b, nullptr, nullptr, H.desc[0], 0, c->p.ordering, H.tile_bits[0], E, c->p.seg_rows,
-                          c->sm_count, c->stream);
-  } else if (c->p.dim == 2)
+    STATUS_TRY(launched(launch_tile_post_norm(u, b, nullptr, nullptr, H.desc[0], 0, c->p.ordering, H.tile_bits[0], E,
+                                              c->p.seg_rows, c->sm_count, c->stream),
+                        "tile residual"));
+  } else if (c->p.dim == 2) {
     launch_residual<double, 2>(c, c->h64.desc[0], 0, nullptr, u, b, E);
-  else
+  } else {
     launch_residual<double, 3>(c, c->h64.desc[0], 0, nullptr, u, b, E);
+  }
+  return FAS_OK;
 }
 
 void enqueue_remove_mean(fas_ctx* c, double* x, const double* y) {
@@ -1054,8 +1060,7 @@ fas_status enqueue_prologue(fas_ctx* c, double* u, const double* f_in, bool fn_r
     fn_ready = false;
   }
   if (!fn_ready) enqueue_norm(c, f, norm_rhs(c, max_cycles));
-  enqueue_residual_norm(c, u, f, norm_to(c, kNormFirst, &c->S->nscale));
-  return FAS_OK;
+  return enqueue_residual_norm(c, u, f, norm_to(c, kNormFirst, &c->S->nscale));
 }
 
 // Enqueue one cycle, its residual norm and the stopping decision.
@@ -1070,8 +1075,7 @@ fas_status enqueue_body(fas_ctx* c, double* u, const double* f_in, cudaGraphCond
     STATUS_TRY(vcycle<double>(c, c->h64, u, f));
   }
   if (c->singular) enqueue_remove_mean(c, u, u);
-  enqueue_residual_norm(c, u, f, norm_cycle(c, h, set_cond));
-  return FAS_OK;
+  return enqueue_residual_norm(c, u, f, norm_cycle(c, h, set_cond));
 }
 
 // Heat step: b = u + dt fsrc and ||b||.

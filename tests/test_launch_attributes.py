@@ -1,5 +1,10 @@
-"""A kernel's shared-memory limit is an attribute of the kernel on one device: every fas_create sets it, on the device
-that is current then. Setting it once per process would leave the kernels of a second device without."""
+"""Launch rules that hold by the text of the sources.
+
+A kernel's shared-memory limit is an attribute of the kernel on one device: every fas_create sets it, on the device
+that is current then. Setting it once per process would leave the kernels of a second device without.
+
+The launchers of the tile, column and sweep kernels return their launch error and clear it, so a caller that drops it
+would go on with the results of an earlier launch."""
 import glob
 import os
 import re
@@ -27,3 +32,13 @@ def test_limits_are_not_set_once_per_process():
     create = api[api.index("fas_status fas_create("):api.index("fas_status fas_destroy(")]
     for name in seen - {"pre_attr", "col_attr"}:
         assert name in create, name
+
+
+def test_launch_errors_are_not_dropped():
+    with open(os.path.join(CSRC, "fas_api.cu")) as f:
+        api = f.read()
+    calls = [m for m in re.finditer(r"\blaunch_(?:tile_\w+|col3d_\w+|stream2d_\w+|sweep3d|ir_strip)(?:<T>)?\(", api)]
+    assert len(calls) >= 8
+    for m in calls:
+        before = api[max(0, m.start() - 40):m.start()]
+        assert re.search(r"(launched\(|cudaError_t e\w* =\s*|&&\s*|\be =\s*)$", before), before + m.group(0)
