@@ -92,7 +92,8 @@ typedef struct {
   int use_graph;         /* 1: capture repeated launch sequences in CUDA graphs (default 1)     */
   int path;              /* 0: fused kernels where the level allows and they pay (default);
                           * 1: one kernel per operation everywhere, the 3D restriction and tau
-                          *    correction one cell per thread (reference path);
+                          *    correction one cell per thread (reference path; 3D float64 neighbour
+                          *    sums are formed by integers on every path);
                           * 2: sweep-fused kernels on every level they handle, whatever its size */
   int seg_rows;          /* rows per warp segment in the sweep-fused 2D kernels (0: up to 128), and
                           * region height of the register-tile kernels: 0 by size, up to 32: 32

@@ -787,7 +787,8 @@ fas_status vcycle_basic_from(fas_ctx* c, Hier<T>& H, int lfrom, T* utop, const T
         }
       }
       if constexpr (std::is_same<T, double>::value && DIM == 3) {
-        if (!L.varkappa && n <= kLanesMaxCells3D) {
+        // (path 1: one coarse cell per thread)
+        if (c->p.path != 1 && !L.varkappa && n <= kLanesMaxCells3D) {
           with_fax(c, [&](auto tag) {
             constexpr int FAX = decltype(tag)::value;
             constexpr int lanes = FAX < 0 ? 8 : 4;

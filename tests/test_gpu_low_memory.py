@@ -52,11 +52,12 @@ def test_fallback_without_second_buffers(cuda_lib, shape, precision, path0):
         left = _free()
     finally:
         hog.release()
-    # all but one field of the finest level (the sweep-fused 3D kernel's, in float32) has been given back
+    # all but one field of the finest level (the sweep-fused 3D kernel's, in float32) has been given back; the smallest
+    # buffers in question take 64 MB, and free memory moves by some 20 MB between the measurements
     cells = 1
     for n in shape:
         cells *= n
-    assert left >= need - 32 * MB - basic - (4 * cells if len(shape) == 3 else 0) - 8 * MB
+    assert left >= need - 32 * MB - basic - (4 * cells if len(shape) == 3 else 0) - 40 * MB
     gen = torch.Generator("cuda").manual_seed(761)
     u0 = torch.rand(shape, dtype=torch.float64, device="cuda", generator=gen)
     f = torch.rand(shape, dtype=torch.float64, device="cuda", generator=gen)
