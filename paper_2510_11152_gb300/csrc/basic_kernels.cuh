@@ -839,10 +839,7 @@ static __global__ void k_kappa_frac(long long* aq, LevelDesc<double> L, int* bad
 template <typename T>
 struct CoarseArgs {
   const LevelDesc<T>* desc;  // device array, one per level
-  T* const* u;               // per-level buffers (entry l0 replaced by utop)
-  T* const* f;
-  T* const* u0;
-  const T* cinv;  // dense inverse of the coarsest operator, or null
+  const T* cinv;             // dense inverse of the coarsest operator, or null
   int l0, nlev, nu1, nu2, nuc;
   int ordering;  // fas_ordering
 };

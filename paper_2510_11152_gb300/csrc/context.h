@@ -29,12 +29,11 @@ struct Hier {
   bool tiled = false;
   std::vector<int> tile_bits;  // fixed-point bits of each tiled level (float64; 0: float64 arithmetic)
   TileCoarse<T> tile_coarse;   // arguments of the single-block tile kernel
+  std::vector<long long*> aq;  // per-cell diffusivity in float64: fractions of every level (LevelDesc::aq)
+  int* aq_bad = nullptr;       // and a flag per level
   int ncol = 0;            // 3D float32: levels 0..ncol-1 use the column-streaming kernels
   SmemLayout smem;         // shared-memory layout of the single-CTA kernel (levels >= switch_level)
   size_t smem_bytes = 0;
-  T** d_u = nullptr;
-  T** d_f = nullptr;
-  T** d_u0 = nullptr;
   T* cinv = nullptr;
   std::vector<void*> owned;  // every device allocation above
   bool allocated = false;

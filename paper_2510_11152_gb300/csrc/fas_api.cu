@@ -233,6 +233,7 @@ void free_hier(Hier<T>& H) {
   H.ntile = 0;
   H.tiled = false;
   H.ncol = 0;
+  H.aq.clear();
   H.d_desc = nullptr;
   H.cinv = nullptr;
   H.allocated = false;
@@ -310,26 +311,55 @@ fas_status coarse_inverse(const fas_ctx* c, const LevelShape& s, const std::vect
   return FAS_OK;
 }
 
-// The fixed-point fractions of every level of a 2D float64 hierarchy with per-cell diffusivity. A level whose weights
-// are not those of an average, or one without room for the arrays, keeps float64 arithmetic (aq null).
-fas_status kappa_fractions(fas_ctx* c, Hier<double>& H) {
-  int* bad = nullptr;
-  STATUS_TRY(dev_alloc(H, &bad, c->nlev));
-  CUDA_TRY(cudaMemsetAsync(bad, 0, c->nlev * sizeof(int), c->stream));
-  std::vector<long long*> aq(c->nlev, nullptr);
-  for (int l = 0; l < c->nlev; ++l) {
-    const int64_t n = c->shape[l].cells();
-    if (n > INT32_MAX || dev_alloc(H, &aq[l], 4 * n) != FAS_OK) {
-      cudaGetLastError();
-      aq[l] = nullptr;
-      continue;
+// The buffers of a hierarchy of the register-tile kernels, one after the other in one allocation (a tenth of the calls, and
+// fas_create is short on small grids): u and f of levels first..ntile (the single-block kernel holds the levels below its
+// first in shared memory), the second u and R(r) of levels nfast..ntile-1, and the fractions of a per-cell diffusivity
+// with a flag per level (kappa_fractions).
+template <typename T>
+fas_status tile_buffers(const fas_ctx* c, Hier<T>& H, int first) {
+  const bool fractions = c->p.kappa && sizeof(T) == 8;
+  constexpr int64_t kAlign = 512 / sizeof(T);
+  int64_t total = 0;
+  T* base = nullptr;
+  auto place = [&](auto** at, int64_t n) {  // the first pass sums up, the second one hands out
+    if (base) *at = reinterpret_cast<std::remove_reference_t<decltype(*at)>>(base + total);
+    total += (n + kAlign - 1) / kAlign * kAlign;
+  };
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1) {
+      STATUS_TRY(dev_alloc(H, &base, total));
+      total = 0;
     }
-    k_kappa_frac<<<grid_for(c, n), kBlock, 0, c->stream>>>(aq[l], H.desc[l], bad + l);
+    for (int l = 0; l <= H.ntile; ++l) {
+      const int64_t n = c->shape[l].cells();
+      if (l >= first) {
+        place(&H.u[l], n);
+        place(&H.f[l], n);
+      }
+      if (l >= H.nfast && l < H.ntile) {
+        place(&H.u2[l], n);
+        if (l > 0) place(&H.rc[l], n);
+      }
+    }
+    if (fractions) {
+      H.aq.assign(c->nlev, nullptr);
+      for (int l = 0; l < c->nlev; ++l) place(&H.aq[l], 4 * c->shape[l].cells());
+      place(&H.aq_bad, c->nlev);
+    }
   }
+  return FAS_OK;
+}
+
+// The fixed-point fractions of every level of a 2D float64 hierarchy with per-cell diffusivity. A level whose weights
+// are not those of an average keeps float64 arithmetic (aq null).
+fas_status kappa_fractions(fas_ctx* c, Hier<double>& H) {
+  CUDA_TRY(cudaMemsetAsync(H.aq_bad, 0, c->nlev * sizeof(int), c->stream));
+  for (int l = 0; l < c->nlev; ++l)
+    k_kappa_frac<<<grid_for(c, c->shape[l].cells()), kBlock, 0, c->stream>>>(H.aq[l], H.desc[l], H.aq_bad + l);
   std::vector<int> hb(c->nlev, 0);
-  CUDA_TRY(cudaMemcpyAsync(hb.data(), bad, c->nlev * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(cudaMemcpyAsync(hb.data(), H.aq_bad, c->nlev * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  for (int l = 0; l < c->nlev; ++l) H.desc[l].aq = hb[l] ? nullptr : aq[l];
+  for (int l = 0; l < c->nlev; ++l) H.desc[l].aq = hb[l] ? nullptr : H.aq[l];
   return FAS_OK;
 }
 
@@ -473,48 +503,42 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       H.tiled = lc < c->nlev && c->shape[0].cells() <= most_cells;
       H.ntile = H.tiled ? lc : 0;
     }
-    auto level_buffers = [&](int l) -> fas_status {
-      STATUS_TRY(dev_alloc(H, &H.u[l], c->shape[l].cells()));
-      return dev_alloc(H, &H.f[l], c->shape[l].cells());
-    };
-    // (the single-block tile kernel holds the levels below its first in shared memory)
-    for (int l = level0_buffers ? 0 : 1; l < c->nlev && (!H.tiled || l <= H.ntile); ++l) STATUS_TRY(level_buffers(l));
     // sweep-fused 2D path (float32 only): consecutive levels from the finest that the fused kernels
     // handle and that are larger than the single-CTA switch level
-    H.nfast = 0;
-    if (sizeof(T) == 4 && p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL &&
-        p.ordering == FAS_ORDER_FORWARD && p.nu1 >= 1 && p.nu2 >= 1 && periodic_mask(p) == 0) {
-      // below that a level's fused kernels are latency-bound (one warp streams a long segment of rows) and
-      // the register-tile kernels take it; where those do not apply (narrow hierarchies) the finest level
-      // stays fused for its float64 update and the others run per operation
-      const int64_t fused_min = H.tiled ? kFusedMinCells2D : kFusedMinCells2DUntiled;
-      while (H.nfast < H.switch_level &&
-             stream2d_supported(c->shape[H.nfast].nx, c->shape[H.nfast].ny, std::max(p.nu1, p.nu2)) &&
-             ((H.nfast == 0 && !H.tiled) || c->shape[H.nfast].cells() >= fused_min || p.path == 2) &&
-             (!H.tiled || H.nfast < H.ntile))
-        H.nfast++;
-    }
+    auto count_fused = [&]() {
+      H.nfast = 0;
+      if (sizeof(T) == 4 && p.dim == 2 && p.path != 1 && !p.kappa && p.location == FAS_CELL &&
+          p.ordering == FAS_ORDER_FORWARD && p.nu1 >= 1 && p.nu2 >= 1 && periodic_mask(p) == 0) {
+        // below that a level's fused kernels are latency-bound (one warp streams a long segment of rows) and
+        // the register-tile kernels take it; where those do not apply (narrow hierarchies) the finest level
+        // stays fused for its float64 update and the others run per operation
+        const int64_t fused_min = H.tiled ? kFusedMinCells2D : kFusedMinCells2DUntiled;
+        while (H.nfast < H.switch_level &&
+               stream2d_supported(c->shape[H.nfast].nx, c->shape[H.nfast].ny, std::max(p.nu1, p.nu2)) &&
+               ((H.nfast == 0 && !H.tiled) || c->shape[H.nfast].cells() >= fused_min || p.path == 2) &&
+               (!H.tiled || H.nfast < H.ntile))
+          H.nfast++;
+      }
+    };
+    count_fused();
     H.u2.assign(c->nlev, nullptr);
     H.rc.assign(c->nlev, nullptr);
+    const int first = level0_buffers ? 0 : 1;
+    if (H.tiled && tile_buffers(c, H, first) != FAS_OK) {
+      // without room for them the levels run the per-operation kernels
+      cudaGetLastError();
+      H.tiled = false;
+      H.ntile = 0;
+      count_fused();
+    }
+    for (int l = first; l < c->nlev && !H.tiled; ++l) {
+      STATUS_TRY(dev_alloc(H, &H.u[l], c->shape[l].cells()));
+      STATUS_TRY(dev_alloc(H, &H.f[l], c->shape[l].cells()));
+      if (l > 0) STATUS_TRY(dev_alloc(H, &H.u0[l], c->shape[l].cells()));  // the restricted start
+    }
     for (int l = 0; l < H.nfast; ++l) {
       STATUS_TRY(dev_alloc(H, &H.u2[l], c->shape[l].cells()));
       if (l + 1 < H.nfast) STATUS_TRY(dev_alloc(H, &H.rc[l + 1], c->shape[l + 1].cells()));
-    }
-    const size_t mark = H.owned.size();
-    for (int l = H.nfast; l < H.ntile && H.tiled; ++l) {
-      // without room for the second buffers the levels run the per-operation kernels, and their room is given back
-      if (dev_alloc(H, &H.u2[l], c->shape[l].cells()) != FAS_OK ||
-          (l > 0 && dev_alloc(H, &H.rc[l], c->shape[l].cells()) != FAS_OK)) {
-        cudaGetLastError();
-        for (; H.owned.size() > mark; H.owned.pop_back()) cudaFree(H.owned.back());
-        for (int k = H.nfast; k <= l; ++k) H.u2[k] = H.rc[k] = nullptr;
-        H.tiled = false;
-        H.ntile = 0;
-      }
-    }
-    for (int l = 1; l < c->nlev && !H.tiled; ++l) {  // the per-operation kernels: also the restricted start
-      if (!H.u[l]) STATUS_TRY(level_buffers(l));
-      STATUS_TRY(dev_alloc(H, &H.u0[l], c->shape[l].cells()));
     }
     if (H.tiled) {
       if constexpr (std::is_same<T, double>::value)
@@ -570,14 +594,6 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
           if (sweep3d_supported(H.desc[l]) && (c->shape[l].cells() >= kSweep3dMinCells || p.path == 2))
             STATUS_TRY(dev_alloc(H, &H.u2[l], c->shape[l].cells()));
     }
-    T** arrs[3] = {nullptr, nullptr, nullptr};
-    for (int k = 0; k < 3; ++k) STATUS_TRY(dev_alloc(H, &arrs[k], kMaxLevels));
-    H.d_u = arrs[0];
-    H.d_f = arrs[1];
-    H.d_u0 = arrs[2];
-    CUDA_TRY(cudaMemcpy(H.d_u, H.u.data(), c->nlev * sizeof(T*), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(H.d_f, H.f.data(), c->nlev * sizeof(T*), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(H.d_u0, H.u0.data(), c->nlev * sizeof(T*), cudaMemcpyHostToDevice));
     if (p.coarse_exact) {
       std::vector<double> inv;
       STATUS_TRY(coarse_inverse(c, c->shape[c->nlev - 1], cwx, cwy, cwz, cDh, inv));
@@ -729,9 +745,6 @@ fas_status launch_coarse(fas_ctx* c, Hier<T>& H, int l0, T* utop, const T* ftop)
   if (l0 != H.switch_level) return fail(FAS_ECUDA, "single-CTA kernel launched above its shared-memory level");
   CoarseArgs<T> A;
   A.desc = H.d_desc;
-  A.u = H.d_u;
-  A.f = H.d_f;
-  A.u0 = H.d_u0;
   A.cinv = H.cinv;
   A.l0 = l0;
   A.nlev = H.nlev;
@@ -1698,15 +1711,18 @@ fas_status fas_create(const fas_params* pin, void* stream, fas_ctx** out) {
   }
   if (c->singular && cudaMalloc(&c->fproj, s.cells() * sizeof(double)) != cudaSuccess)
     return bail(fail(FAS_ENOMEM, "fproj"));
-  // kernel attributes, set before any launch or stream capture
-  cudaError_t e = stream2d_prepare();
-  if (e == cudaSuccess) e = tile2d_prepare();
-  if (e == cudaSuccess) e = col3d_prepare();
-  if (e == cudaSuccess) e = ir_strip_prepare();
-  if (e == cudaSuccess) e = sweep3d_prepare();
-  for (cudaError_t ek : {coarse_attr<double, 2>(), coarse_attr<double, 3>(), coarse_attr<float, 2>(),
-                         coarse_attr<float, 3>()})
-    if (e == cudaSuccess) e = ek;
+  // kernel attributes of the kernels that this context may launch, set before any launch or stream capture
+  cudaError_t e = cudaSuccess;
+  if (p.dim == 2) {
+    e = tile2d_prepare();
+    if (e == cudaSuccess && mixed) e = stream2d_prepare();
+    if (e == cudaSuccess) e = mixed ? coarse_attr<float, 2>() : coarse_attr<double, 2>();
+  } else {
+    if (mixed) e = col3d_prepare();
+    if (e == cudaSuccess) e = ir_strip_prepare();  // fas_residual_ir takes either precision
+    if (e == cudaSuccess && mixed) e = sweep3d_prepare();
+    if (e == cudaSuccess) e = mixed ? coarse_attr<float, 3>() : coarse_attr<double, 3>();
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return bail(fail(FAS_ECUDA, std::string("fas_create: ") + cudaGetErrorString(e)));
   *out = c;
