@@ -390,10 +390,13 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
   }
 }
 
-// At least three blocks per SM: the float64 3D phase waits for its rows from L2, and with two blocks (94 registers) too
-// few are in flight (256 x 128 x 64 heat run: 8.03 -> 7.44 ms; four blocks spill: 7.95).
+// Blocks per SM: at least three in float64 3D, whose phase waits for its rows from L2 with too few in flight at two blocks (94
+// registers; 256 x 128 x 64 heat run: 8.03 -> 7.44 ms; four blocks spill: 7.95), four or five for the others, as many as their
+// single-cell form had.
 template <typename T, int DIM>
-__global__ void __launch_bounds__(256, 3) k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
+constexpr int kColour4Blocks = DIM == 3 ? (sizeof(T) == 8 ? 3 : 4) : (sizeof(T) == 8 ? 4 : 5);
+template <typename T, int DIM>
+__global__ void __launch_bounds__(256, kColour4Blocks<T, DIM>) k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
   if (L.per)
     smooth_colour4_body<T, DIM, true>(u, f, L, colour);
   else
