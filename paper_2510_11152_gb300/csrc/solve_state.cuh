@@ -97,6 +97,11 @@ __device__ __forceinline__ void norm_decide(const NormEnd& E, double norm) {
 // 0 of the last block.
 __device__ __forceinline__ bool norm_end(const NormEnd& E, double part, int block, int nblocks) {
   __shared__ int last;
+  if (nblocks == 1) {  // small grids: the block's sum is the whole one
+    if (threadIdx.x != 0) return false;
+    norm_decide(E, sqrt(part) / (E.nsp ? (double)*E.nsp : 1.0));
+    return true;
+  }
   if (threadIdx.x == 0) {
     E.partials[block] = part;
     __threadfence();
