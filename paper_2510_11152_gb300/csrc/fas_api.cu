@@ -92,6 +92,7 @@ constexpr int64_t kCol3dMinCells = (int64_t)1 << 24;
 // more words per cell (the fractions), and on larger grids the per-operation kernels are faster (a cycle of a solve on 1024^2:
 // 285 us against 288 per operation, 512^2: 123 against 179; but 2048 x 1024: 480 against 453, 2048^2: 843 against 667). In
 // float32 (cells by 32-bit index) they win throughout.
+constexpr size_t kTileBytesUnasked = (size_t)256 << 20;  // up to this size the free memory is not looked at
 constexpr int64_t kTileMaxCellsKappa = (int64_t)1 << 20;
 // Smallest 2D level of the sweep-fused kernels: above the register-tile kernels (whose blocks recompute half again as
 // many cells; 4096^2 level of an 8192^2 run, pre-smoothing: 68 us against 89, 2048^2: 29 against 28, 1024^2: 18
@@ -314,7 +315,8 @@ fas_status coarse_inverse(const fas_ctx* c, const LevelShape& s, const std::vect
 // The buffers of a hierarchy of the register-tile kernels, one after the other in one allocation (a tenth of the calls, and
 // fas_create is short on small grids): u and f of levels first..ntile (the single-block kernel holds the levels below its
 // first in shared memory), the second u and R(r) of levels nfast..ntile-1, and the fractions of a per-cell diffusivity
-// with a flag per level (kappa_fractions).
+// with a flag per level (kappa_fractions). They take 2.3 fields of the grid in float64 where the per-operation kernels take
+// one; large ones must leave as much memory again, which fields that the context allocates later may need.
 template <typename T>
 fas_status tile_buffers(const fas_ctx* c, Hier<T>& H, int first) {
   const bool fractions = c->p.kappa && sizeof(T) == 8;
@@ -327,6 +329,10 @@ fas_status tile_buffers(const fas_ctx* c, Hier<T>& H, int first) {
   };
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1) {
+      size_t room = 0, all = 0;
+      if (total * sizeof(T) > kTileBytesUnasked && cudaMemGetInfo(&room, &all) == cudaSuccess &&
+          total * sizeof(T) > room / 2)
+        return fail(FAS_ENOMEM, "buffers of the register-tile kernels");
       STATUS_TRY(dev_alloc(H, &base, total));
       total = 0;
     }

@@ -69,3 +69,33 @@ def test_fallback_without_second_buffers(cuda_lib, shape, precision, path0):
         out.append(u)
         fas.fas_destroy(c)
     assert torch.equal(out[0], out[1])
+
+
+def test_later_buffers_fit(cuda_lib):
+    """A context whose second buffers would take the room that its heat right-hand side needs later."""
+    import torch
+    fas = cuda_lib
+    shape, dt = (4096, 4096), 1e-4
+    field = 8 * shape[0] * shape[1]
+
+    def params(path):
+        return fas.make_params(shape, 1.0 / shape[-1], alpha=1.0, beta=dt, path=path)
+
+    fas.fas_destroy(fas.fas_create(params(0)))
+    need, basic = _used(fas, params(0)), _used(fas, params(1))
+    leave = need + field // 2
+    assert leave > basic + field + 32 * MB
+    gen = torch.Generator("cuda").manual_seed(762)
+    u0 = torch.rand(shape, dtype=torch.float64, device="cuda", generator=gen)
+    u, ref = u0.clone(), u0.clone()
+    hog = _Leave(leave)
+    try:
+        ctx = fas.fas_create(params(0))
+        fas.fas_heat_run(ctx, u, None, dt, 1)
+    finally:
+        hog.release()
+    fas.fas_destroy(ctx)
+    ctx = fas.fas_create(params(1))
+    fas.fas_heat_run(ctx, ref, None, dt, 1)
+    fas.fas_destroy(ctx)
+    assert torch.equal(u, ref)
