@@ -40,7 +40,7 @@ __device__ __forceinline__ float residual_range(T* r, const T* u, const T* f, co
                                                 float nscale, int64_t t0, int64_t stride) {
   // nscale: power-of-two factor applied before squaring (keeps float squares in range)
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
-  float acc = 0.f;
+  FloatSum acc;
   for (int64_t idx = t0; idx < n; idx += stride) {
     const int i = (int)(idx & (L.nx - 1));
     const int j = (int)((idx >> L.lx) & (L.ny - 1));
@@ -48,9 +48,9 @@ __device__ __forceinline__ float residual_range(T* r, const T* u, const T* f, co
     const T rv = (L.fax >= 0 && frozen(L, i, j, l)) ? T(0) : residual_point<T, DIM, PER, INT>(u, f, L, idx, i, j, l);
     if (r) r[idx] = rv;
     const float rs = (float)rv * nscale;
-    acc = fmaf(rs, rs, acc);
+    acc.add(rs * rs);
   }
-  return acc;
+  return acc.value();
 }
 
 // ---- Appendix C restriction: coarse cell = average of its 2^d children. Writes uc (and uc0, a
@@ -404,11 +404,11 @@ __global__ void __launch_bounds__(256, kColour4Blocks<T, DIM>) k_smooth_colour4(
 }
 
 // r (nullable) = f - A u, and the norm of the residual (scaled by s = *E.nsp before squaring).
-template <typename T, int DIM>
+template <typename T, int DIM, bool ONE = false>
 __global__ void k_residual(T* r, const T* u, const T* f, LevelDesc<T> L, const __grid_constant__ NormEnd E) {
   const float acc = L.per ? residual_range<T, DIM, true, true>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride())
                           : residual_range<T, DIM, false, true>(r, u, f, L, E.nsp ? *E.nsp : 1.f, gtid(), gstride());
-  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
+  norm_end<ONE>(E, block_sum((double)acc), blockIdx.x, gridDim.x);
 }
 
 // out[0] = sum of partials (no square root), used for means.
@@ -522,16 +522,17 @@ __global__ void k_sub_mean(T* x, const T* y, int64_t n, const double* sum) {
 }
 
 // heat step right-hand side: b = u + dt * fsrc (fsrc may be null: b = u), and ||b|| (float squares)
-static __global__ void k_heat_rhs(double* b, const double* u, const double* fsrc, double dt, int64_t n,
+template <bool ONE = false>
+__global__ void k_heat_rhs(double* b, const double* u, const double* fsrc, double dt, int64_t n,
                                   const __grid_constant__ NormEnd E) {
-  float acc = 0.f;
+  FloatSum acc;
   for (int64_t i = gtid(); i < n; i += gstride()) {
     const double v = fsrc ? fma(dt, fsrc[i], u[i]) : u[i];
     b[i] = v;
     const float vf = f64_to_f32_rn_bits(v);
-    acc = fmaf(vf, vf, acc);
+    acc.add(vf * vf);
   }
-  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
+  norm_end<ONE>(E, block_sum((double)acc.value()), blockIdx.x, gridDim.x);
 }
 
 // ---- mixed precision (iterative refinement): u += e, and r32 = (float)(b - A u) with its norm
@@ -585,7 +586,7 @@ __global__ void k_ir_residual(float* r32, const double* u, const double* b, Leve
                               const __grid_constant__ NormEnd E) {
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
   const float nscale = E.nsp ? *E.nsp : 1.f;
-  float acc = 0.f;
+  FloatSum acc;
   for (int64_t idx = gtid(); idx < n; idx += gstride()) {
     const int i = (int)(idx & (L.nx - 1));
     const int j = (int)((idx >> L.lx) & (L.ny - 1));
@@ -611,9 +612,9 @@ __global__ void k_ir_residual(float* r32, const double* u, const double* b, Leve
     }
     r32[idx] = rv;
     const float rs = rv * nscale;
-    acc = fmaf(rs, rs, acc);
+    acc.add(rs * rs);
   }
-  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
+  norm_end(E, block_sum((double)acc.value()), blockIdx.x, gridDim.x);
 }
 
 // The four cells of a group (x0 .. x0 + 3) and their neighbours, 0 where there is none.
@@ -673,7 +674,7 @@ struct Group4 {
 // Where a cell's own stencil lies more than 2^kGroupSpread below the group's largest value, the group takes float64.
 // About 90 (2D) and 110 (3D) instructions per cell; a thread per cell with its own conversions took 250, the 3D
 // plane-streaming kernel (ir_strip.cu) 247.
-template <int DIM, bool IR>
+template <int DIM, bool IR, bool ONE = false>
 __global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<IR, float, double>::type* r, const double* u,
                                                    const double* f, const __grid_constant__ LevelDesc<double> L,
                                                    const __grid_constant__ NormEnd E) {
@@ -682,7 +683,7 @@ __global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<
   const int lg = L.lx - 2;
   const int64_t ngroups = (int64_t)1 << (lg + L.ly + L.lz);
   const float nscale = E.nsp ? *E.nsp : 1.f;
-  float acc = 0.f;
+  FloatSum acc;
   for (int64_t g = gtid(); g < ngroups; g += gstride()) {
     const int x0 = (int)(g & ((1 << lg) - 1)) << 2;
     const int64_t rest = g >> lg;
@@ -740,26 +741,28 @@ __global__ void __launch_bounds__(256, 3) k_residual4(typename std::conditional<
       for (int k = 0; k < 4; ++k) oq.v[k] = rv[k];
       oq.st(r + idx);
     }
+    float sq = 0.f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const float v = o[k] * nscale;
-      acc = fmaf(v, v, acc);
+      sq = fmaf(v, v, sq);
     }
+    acc.add(sq);
   }
-  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
+  norm_end<ONE>(E, block_sum((double)acc.value()), blockIdx.x, gridDim.x);
 }
 
 // ||x||, squares of the float-rounded values (norms for stopping
 // tests need a few digits only, and the conversion keeps the work off the FP64 pipe)
-template <typename T>
+template <typename T, bool ONE = false>
 __global__ void k_norm2(const T* x, int64_t n, const __grid_constant__ NormEnd E) {
   const float nscale = E.nsp ? *E.nsp : 1.f;
-  float acc = 0.f;
+  FloatSum acc;
   for (int64_t i = gtid(); i < n; i += gstride()) {
     const float v = (float)x[i] * nscale;
-    acc = fmaf(v, v, acc);
+    acc.add(v * v);
   }
-  norm_end(E, block_sum((double)acc), blockIdx.x, gridDim.x);
+  norm_end<ONE>(E, block_sum((double)acc.value()), blockIdx.x, gridDim.x);
 }
 
 template <typename T>

@@ -175,6 +175,19 @@ __device__ __forceinline__ T residual_point(const T* __restrict__ u, const T* __
   return fma(L.c, nb, fma(-L.d[cls], u[idx], f[idx]));
 }
 
+// A thread's sum of many float values, with the rounding errors of the additions kept (Knuth's TwoSum): a thread of a norm
+// kernel adds up to a few hundred squares, and the FP64 pipe stays out of it.
+struct FloatSum {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = hi + x, y = t - hi;
+    lo += (hi - (t - y)) + (x - y);
+    hi = t;
+  }
+  // rounded once; an infinite sum leaves no error term
+  __device__ __forceinline__ float value() const { return lo == lo ? hi + lo : hi; }
+};
+
 // Block-wide sum of one double per thread; result valid in thread 0. blockDim.x <= 1024.
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double warp_part[32];

@@ -80,6 +80,13 @@ constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smo
 // instructions per cell (512^3: 1.64 ms against 1.22) and keeps the small grids, where both are bound by latency.
 constexpr int64_t kIr4MaxCells2D = (int64_t)1 << 22;
 constexpr int64_t kIr4MinCells3D = (int64_t)1 << 21;
+// Blocks per SM of the kernels that form a norm. As many as their registers let run (k_residual4: 80 registers), so that the
+// last block adds 456 to 1216 partial sums instead of 2432 one after the other (6 us; batched loads there cost the small grids
+// more than they saved): fas_residual with a per-cell diffusivity on 1024^2 62 -> 50 us (57 with a launch of its own for the
+// sum), the refinement residual on 2048^2 67 -> 62, a 1024^2 mixed heat run 5.24 -> 4.88 ms. In 3D twice as many up to 2^24
+// cells (128^3: 62 -> 54 us), and from there all, whose order suits the cache (512^3 mixed heat run: 25.1 ms, 25.8 with six).
+constexpr int kStreamBlocks = 8, kPointBlocks = 4;
+constexpr int group_blocks(int dim, int64_t cells) { return dim == 2 ? 3 : cells < ((int64_t)1 << 24) ? 6 : 16; }
 // Largest 3D float64 level whose residual-restriction is spread over lanes (64 x 32 x 32: the same as one thread per coarse
 // cell; below 12 us -> 7, 256 x 128 x 64: 28 us -> 49, its reads being of 2 cells at a time).
 constexpr int64_t kLanesMaxCells3D = (int64_t)1 << 16;
@@ -103,6 +110,12 @@ constexpr int64_t kFusedMinCells2DUntiled = (int64_t)1 << 20;
 int grid_for(const fas_ctx* c, int64_t work) {
   int64_t g = (work + kBlock - 1) / kBlock;
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, c->max_blocks));
+}
+
+// Blocks of a kernel that forms a norm, at most per_sm on an SM (and so at most the max_blocks that `partials` holds).
+int norm_grid(const fas_ctx* c, int64_t work, int per_sm) {
+  const int64_t g = (work + kBlock - 1) / kBlock;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(g, (int64_t)c->sm_count * per_sm));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -738,11 +751,19 @@ void launch_residual(fas_ctx* c, const LevelDesc<T>& L, int level, T* r, const T
   Prof pr(c, FAS_K_RESIDUAL, level, (double)n);
   if constexpr (std::is_same<T, double>::value) {
     if ((c->p.path != 1 || L.fax >= 0) && !L.varkappa && L.nx % 4 == 0) {
-      k_residual4<DIM, false><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r, u, f, L, E);
+      const int g = norm_grid(c, n / 4, group_blocks(DIM, n));
+      if (g == 1)
+        k_residual4<DIM, false, true><<<1, kBlock, 0, c->stream>>>(r, u, f, L, E);
+      else
+        k_residual4<DIM, false><<<g, kBlock, 0, c->stream>>>(r, u, f, L, E);
       return;
     }
   }
-  k_residual<T, DIM><<<grid_for(c, n), kBlock, 0, c->stream>>>(r, u, f, L, E);
+  const int g = norm_grid(c, n, kPointBlocks);
+  if (g == 1)
+    k_residual<T, DIM, true><<<1, kBlock, 0, c->stream>>>(r, u, f, L, E);
+  else
+    k_residual<T, DIM><<<g, kBlock, 0, c->stream>>>(r, u, f, L, E);
 }
 
 template <typename T, int DIM>
@@ -989,7 +1010,11 @@ fas_status sync_read(fas_ctx* c, double* out) {
 void enqueue_norm(fas_ctx* c, const double* x, const NormEnd& E) {
   const int64_t n = c->shape[0].cells();
   Prof pr(c, FAS_K_NORM, 0, (double)n);
-  k_norm2<double><<<grid_for(c, n), kBlock, 0, c->stream>>>(x, n, E);
+  const int g = norm_grid(c, n, kStreamBlocks);
+  if (g == 1)
+    k_norm2<double, true><<<1, kBlock, 0, c->stream>>>(x, n, E);
+  else
+    k_norm2<double><<<g, kBlock, 0, c->stream>>>(x, n, E);
 }
 
 // r32 = (float)(b - A u) on level 0 and its norm
@@ -998,22 +1023,25 @@ void launch_ir_residual(fas_ctx* c, float* r32, const double* u, const double* b
   const int64_t n = c->shape[0].cells();
   Prof pr(c, FAS_K_IR, 0, (double)n);
   const bool group = !L.varkappa && L.nx % 4 == 0;  // on every path: r32 does not depend on it
-  if (group && c->p.dim == 2 && n <= kIr4MaxCells2D)
-    k_residual4<2, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
-  else if (group && c->p.dim == 3 && n >= kIr4MinCells3D)
-    k_residual4<3, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
-  else if (ir_strip_supported(L) &&
+  const bool first = group && (c->p.dim == 2 ? n <= kIr4MaxCells2D : n >= kIr4MinCells3D);
+  if (!first && ir_strip_supported(L) &&
       launch_ir_strip(r32, u, b, L, E, c->ir_ticket, c->sm_count, c->max_blocks, c->stream,
                       Ir3Wait{g_wait_limit_ns.load(), take_withhold(1)}) == cudaSuccess)
-    ;  // the strip kernels took the level
-  else if (group && c->p.dim == 2)
-    k_residual4<2, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
-  else if (group)
-    k_residual4<3, true><<<grid_for(c, n / 4), kBlock, 0, c->stream>>>(r32, u, b, L, E);
-  else if (c->p.dim == 2)
-    k_ir_residual<2><<<grid_for(c, n), kBlock, 0, c->stream>>>(r32, u, b, L, E);
+    return;  // the strip kernels took the level
+  auto launch = [&](auto dim) {
+    constexpr int DIM = decltype(dim)::value;
+    const int g = norm_grid(c, group ? n / 4 : n, group ? group_blocks(DIM, n) : kPointBlocks);
+    if (!group)
+      k_ir_residual<DIM><<<g, kBlock, 0, c->stream>>>(r32, u, b, L, E);
+    else if (g == 1)
+      k_residual4<DIM, true, true><<<1, kBlock, 0, c->stream>>>(r32, u, b, L, E);
+    else
+      k_residual4<DIM, true><<<g, kBlock, 0, c->stream>>>(r32, u, b, L, E);
+  };
+  if (c->p.dim == 2)
+    launch(std::integral_constant<int, 2>());
   else
-    k_ir_residual<3><<<grid_for(c, n), kBlock, 0, c->stream>>>(r32, u, b, L, E);
+    launch(std::integral_constant<int, 3>());
 }
 
 // The norm of b - A u; mixed precision also leaves r32 = (float)(b - A u) in h32.f[0]
@@ -1102,7 +1130,11 @@ fas_status enqueue_body(fas_ctx* c, double* u, const double* f_in, cudaGraphCond
 void enqueue_heat_rhs(fas_ctx* c, const double* u, const double* fsrc, double dt, int max_cycles) {
   const int64_t n = c->shape[0].cells();
   Prof pr(c, FAS_K_OTHER, 0, (double)n);
-  k_heat_rhs<<<grid_for(c, n), kBlock, 0, c->stream>>>(c->b, u, fsrc, dt, n, norm_rhs(c, max_cycles));
+  const int g = norm_grid(c, n, kStreamBlocks);
+  if (g == 1)
+    k_heat_rhs<true><<<1, kBlock, 0, c->stream>>>(c->b, u, fsrc, dt, n, norm_rhs(c, max_cycles));
+  else
+    k_heat_rhs<><<<g, kBlock, 0, c->stream>>>(c->b, u, fsrc, dt, n, norm_rhs(c, max_cycles));
 }
 
 // Enqueue the read-back of the refinement residual's timeout word (the host copy is valid after the

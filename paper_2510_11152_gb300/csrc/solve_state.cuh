@@ -94,38 +94,27 @@ __device__ __forceinline__ void norm_decide(const NormEnd& E, double norm) {
 
 // The end of a kernel of nblocks blocks whose thread 0 holds its block's sum of squares: every thread of
 // the block calls it, and nothing after it may depend on the block's other work. Returns true in thread
-// 0 of the last block.
+// 0 of the last block. ONE: the kernel is one block, whose sum is the whole one (a partial written, counted and read back
+// takes 2 us of the small grids' cycles; as a run-time case it cost the other grids 1 to 2 %).
+template <bool ONE = false>
 __device__ __forceinline__ bool norm_end(const NormEnd& E, double part, int block, int nblocks) {
-  __shared__ int last;
-  if (nblocks == 1) {  // small grids: the block's sum is the whole one
-    if (threadIdx.x != 0) return false;
-    norm_decide(E, sqrt(part) / (E.nsp ? (double)*E.nsp : 1.0));
-    return true;
-  }
-  if (threadIdx.x == 0) {
-    E.partials[block] = part;
-    __threadfence();
-    last = atomicAdd(E.ticket, 1u) == (unsigned)nblocks - 1u;
-  }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  // loads in batches: one after the other, the ten per thread that a full grid's 2432 partials take cost 6 us
-  constexpr int kBatch = 8;
-  double v = 0.0;
-  for (int b0 = threadIdx.x; b0 < nblocks; b0 += kBatch * blockDim.x) {
-    double x[kBatch];
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) {
-      const int b = b0 + k * (int)blockDim.x;
-      x[k] = b < nblocks ? __ldcg(E.partials + b) : 0.0;
+  double v = part;
+  if constexpr (!ONE) {
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+      E.partials[block] = part;
+      __threadfence();
+      last = atomicAdd(E.ticket, 1u) == (unsigned)nblocks - 1u;
     }
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) v += x[k];
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    v = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += __ldcg(E.partials + b);
+    v = block_sum(v);
   }
-  v = block_sum(v);
   if (threadIdx.x != 0) return false;
-  *E.ticket = 0u;
+  if constexpr (!ONE) *E.ticket = 0u;
   norm_decide(E, sqrt(v) / (E.nsp ? (double)*E.nsp : 1.0));
   return true;
 }
