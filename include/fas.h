@@ -55,9 +55,14 @@ typedef enum {
  * relation for it; here the ghost of the first cell is the last cell and vice versa, and the face
  * between them is an interior face). Both faces of an axis must be PERIODIC or neither; periodic axes
  * need cell-centred unknowns and a constant kappa (FAS_EUNSUPPORTED otherwise) and run the
- * register-tile kernels in 2D, the per-operation or (large float32 levels) column kernels in 3D. With alpha = 0 and no Dirichlet face the operator is singular and is handled
- * like the all-Neumann pressure solve (mean-free right-hand side, mean removed after every cycle). */
+ * register-tile kernels in 2D, the per-operation or (large float32 levels) column kernels in 3D. With
+ * alpha = 0 and no Dirichlet face the operator is singular and is handled like the all-Neumann pressure
+ * solve (mean-free right-hand side, mean removed after every cycle). */
 typedef enum { FAS_BC_NEUMANN = 0, FAS_BC_DIRICHLET = 1, FAS_BC_PERIODIC = 2 } fas_bc;
+/* FP64 cycles on 2D cell levels compute in 64-bit block fixed point, in units of at most 2^-54 of the largest
+ * value of a region of 64 columns x 32 or 64 rows, wherever the largest values of its patches of 2 x 1..4 cells
+ * lie within 2^10 of one another, and in float64 elsewhere; fields are stored, and residual norms formed, in
+ * float64. */
 typedef enum { FAS_FP64 = 0, FAS_MIXED = 1 } fas_precision;
 
 /* Where the unknowns sit (Sec. 4.1, the MAC staggered grid). FAS_CELL: cell centres (Sec. 2.1).

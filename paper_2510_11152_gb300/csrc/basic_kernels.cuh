@@ -390,13 +390,14 @@ __device__ __forceinline__ void smooth_colour4_body(T* u, const T* f, const Leve
   }
 }
 
-// Blocks per SM: at least three in float64 3D, whose phase waits for its rows from L2 with too few in flight at two blocks (94
-// registers; 256 x 128 x 64 heat run: 8.03 -> 7.44 ms; four blocks spill: 7.95), four or five for the others, as many as their
-// single-cell form had.
+// Blocks per SM: at least three in float64 3D, whose phase waits for its rows from L2 with too few in flight at two
+// blocks (94 registers; 256 x 128 x 64 heat run: 8.03 -> 7.44 ms; four blocks spill: 7.95), four or five for the others, as
+// many as their single-cell form had (three cost mixed solves on the per-operation path up to 7 %).
 template <typename T, int DIM>
 constexpr int kColour4Blocks = DIM == 3 ? (sizeof(T) == 8 ? 3 : 4) : (sizeof(T) == 8 ? 4 : 5);
 template <typename T, int DIM>
-__global__ void __launch_bounds__(256, kColour4Blocks<T, DIM>) k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
+__global__ void __launch_bounds__(256, kColour4Blocks<T, DIM>)
+    k_smooth_colour4(T* u, const T* f, LevelDesc<T> L, int colour) {
   if (L.per)
     smooth_colour4_body<T, DIM, true>(u, f, L, colour);
   else
@@ -869,8 +870,8 @@ __device__ void coarse_smooth(T* u, const T* f, const LevelDesc<T>& L, int sweep
 // Single-CTA V-cycle with every level held in shared memory: levels l0..nlev-1 of u and f, and the
 // restricted start u0 of the coarser ones. Same steps and same per-point arithmetic as the grid-wide
 // kernels (the residual is evaluated per child inside the restriction instead of being stored
-// first), so the results are identical but for the rounding of 3D float64 neighbour sums (sum6); the latency of each dependent step is a shared-memory round
-// trip instead of an L2 one.
+// first), so the results are identical but for the rounding of 3D float64 neighbour sums (sum6); the
+// latency of each dependent step is a shared-memory round trip instead of an L2 one.
 // ------------------------------------------------------------------------------------------------
 struct SmemLayout {
   int64_t off_u[kMaxLevels], off_f[kMaxLevels], off_u0[kMaxLevels];  // element offsets

@@ -65,8 +65,11 @@ bool is_pow2(int n) { return n >= 1 && (n & (n - 1)) == 0; }
 
 constexpr int kBlock = 256;
 constexpr int kCoarseThreads = 1024;
-constexpr int64_t kSwitchCells2D = 16384;  // levels at or below this size run in one CTA
-constexpr int64_t kSwitchCells2DLarge = 4096;  // the same on 2D grids of at least kLargeGrid2D cells
+// Largest level that the single-CTA kernel (k_coarse_smem) starts from, in hierarchies that the register-tile kernels
+// do not take: face grids, 3D, narrow grids, the reference path, more than four sweeps, large float64 grids with a
+// per-cell diffusivity.
+constexpr int64_t kSwitchCells2D = 16384;      // float32, 2D
+constexpr int64_t kSwitchCells2DLarge = 4096;  // the same on grids of at least kLargeGrid2D cells
 constexpr int64_t kLargeGrid2D = (int64_t)1 << 24;
 constexpr int64_t kSwitchCells3D = 4096;
 constexpr int64_t kSwitchCells2DF64 = 1024;
@@ -75,16 +78,18 @@ constexpr size_t kCoarseSmemMax = 200 * 1024;    // field arrays of the single-C
 constexpr size_t kCoarseSmemLimit = 227 * 1024;  // with its level descriptors (per-CTA maximum)
 constexpr int64_t kSweep3dMinCells = (int64_t)1 << 26;  // smallest 3D level smoothed by the fused sweep
 // Refinement residual by groups of four cells (k_residual4) or by the strip kernels (ir_strip.cu). 2D: a strip
-// kernel's warp walks rows one after the other, and small grids leave it few warps (1024^2: 31 us against 18;
-// 2048^2: 45 against 42; 4096^2: 106 against 123; 8192^2: 351 against 428). 3D: the plane-streaming kernel takes 247
-// instructions per cell (512^3: 1.64 ms against 1.22) and keeps the small grids, where both are bound by latency.
+// kernel's warp walks rows one after the other, and small grids leave it few warps (1024^2: 36 us against 18;
+// 2048^2: 48 against 39; 4096^2: 109 against 127; 8192^2: 350 against 466, all with the events' 4 us). 3D: the
+// plane-streaming kernel takes 247 instructions per cell and is the slower one throughout (128^3: 84 us against 34,
+// 256^3: 368 against 171); the small grids keep it because they are what its bounded waits are tested on.
 constexpr int64_t kIr4MaxCells2D = (int64_t)1 << 22;
 constexpr int64_t kIr4MinCells3D = (int64_t)1 << 21;
-// Blocks per SM of the kernels that form a norm. As many as their registers let run (k_residual4: 80 registers), so that the
-// last block adds 456 to 1216 partial sums instead of 2432 one after the other (6 us; batched loads there cost the small grids
-// more than they saved): fas_residual with a per-cell diffusivity on 1024^2 62 -> 50 us (57 with a launch of its own for the
-// sum), the refinement residual on 2048^2 67 -> 62, a 1024^2 mixed heat run 5.24 -> 4.88 ms. In 3D twice as many up to 2^24
-// cells (128^3: 62 -> 54 us), and from there all, whose order suits the cache (512^3 mixed heat run: 25.1 ms, 25.8 with six).
+// Blocks per SM of the kernels that form a norm. As many as their registers let run (k_residual4: 80 registers), so that
+// the last block adds 456 to 1216 partial sums instead of 2432 one after the other (6 us; batched loads there cost the
+// small grids more than they saved): fas_residual with a per-cell diffusivity on 1024^2 62 -> 50 us (57 with a launch of
+// its own for the sum), the refinement residual on 2048^2 67 -> 62, a 1024^2 mixed heat run 5.24 -> 4.88 ms. In 3D twice
+// as many up to 2^24 cells (128^3: 62 -> 54 us), and from there all, whose order suits the cache (512^3 mixed heat run:
+// 25.1 ms, 25.8 with six).
 constexpr int kStreamBlocks = 8, kPointBlocks = 4;
 constexpr int group_blocks(int dim, int64_t cells) { return dim == 2 ? 3 : cells < ((int64_t)1 << 24) ? 6 : 16; }
 // Largest 3D float64 level whose residual-restriction is spread over lanes (64 x 32 x 32: the same as one thread per coarse
@@ -96,11 +101,11 @@ constexpr int64_t kLanesMaxCells3D = (int64_t)1 << 16;
 // they win for every shape measured (256^3: 755 us without, 585 with; 1024 x 128 x 128: 754, 668).
 constexpr int64_t kCol3dMinCells = (int64_t)1 << 24;
 // Largest grid with a per-cell diffusivity whose hierarchy runs the register-tile kernels in float64: they read eight
-// more words per cell (the fractions), and on larger grids the per-operation kernels are faster (a cycle of a solve on 1024^2:
-// 285 us against 288 per operation, 512^2: 123 against 179; but 2048 x 1024: 480 against 453, 2048^2: 843 against 667). In
-// float32 (cells by 32-bit index) they win throughout.
-constexpr size_t kTileBytesUnasked = (size_t)256 << 20;  // up to this size the free memory is not looked at
+// more words per cell (the fractions), and on larger grids the per-operation kernels are faster (a cycle of a solve on
+// 1024^2: 285 us against 288 per operation, 512^2: 123 against 179; but 2048 x 1024: 480 against 453, 2048^2: 843 against
+// 667). In float32 (cells by 32-bit index) they win throughout.
 constexpr int64_t kTileMaxCellsKappa = (int64_t)1 << 20;
+constexpr size_t kTileBytesUnasked = (size_t)256 << 20;  // up to this size the free memory is not looked at
 // Smallest 2D level of the sweep-fused kernels: above the register-tile kernels (whose blocks recompute half again as
 // many cells; 4096^2 level of an 8192^2 run, pre-smoothing: 68 us against 89, 2048^2: 29 against 28, 1024^2: 18
 // against 8), and in hierarchies that those do not take.
@@ -392,12 +397,11 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
   // single-CTA switch level: the first level small enough that the GPU cannot be filled and whose
   // whole sub-hierarchy (u, f on every level, u0 below it) fits in the CTA's shared memory. On a
   // large 2D grid nothing else runs beside the small levels, and one CTA smoothing 128^2 is slower than
-  // per-operation launches across the GPU (8192^2: 118.1 -> 116.1 ms per 20-step run with the switch
-  // at 64^2); smaller grids, often solved side by side in a batch, keep the switch at 128^2 (the
-  // 96-problem batch was 2 % slower with 64^2).
-  // In float64 one SM's FP64 pipe bounds the kernel and the switch is lower (levels that the register-tile
-  // kernels do not take): 512^2 adjoint 42.4 ms with 64^2, 38.5 with 32^2, 40.8 with 16^2; 128^3 cavity step
-  // 10.46 ms with 16^3, 10.15 with 8^3, 10.40 with 4^3.
+  // per-operation launches across the GPU: the switch is at 64^2 there. (The 2D lines were drawn on 8192^2 runs, batches
+  // and a 512^2 adjoint whose small levels the register-tile kernels have taken over since; the hierarchies that are
+  // left kept them.)
+  // In float64 one SM's FP64 pipe bounds the kernel and the switch is lower: 128^3 cavity step 9.74 ms with 16^3, 9.07
+  // with 8^3; 256 x 128 x 64 heat run 7.54 and 7.05.
   const int64_t sw_cells = sizeof(T) == 8   ? (p.dim == 2 ? kSwitchCells2DF64 : kSwitchCells3DF64)
                            : p.dim != 2     ? kSwitchCells3D
                            : c->shape[0].cells() >= kLargeGrid2D ? kSwitchCells2DLarge

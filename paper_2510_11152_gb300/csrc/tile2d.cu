@@ -20,14 +20,15 @@
 //     X_c = a N + B,   N = sum of the neighbours (exact), a as a 64-bit fraction,
 // three wide integer multiply-adds. s leaves just enough high bits for the largest value that the
 // smoothing can reach (a N is an average: each phase adds at most max |B|), so the unit in the last
-// place is 2^-56 of the region's largest value or below, finer than the float64 rounding of that value.
+// place is at most 2^-55 (one or two sweeps) or 2^-54 (three or four) of the region's largest value, finer than the
+// float64 rounding of that value.
 // The scaled residual rho = B - u + a N = (f - A u) / d needs no cancellation-prone products. Regions whose
 // threads' patches of cells (2 columns x 2 or 4 rows) differ by more than 2^10 in magnitude, or that hold a non-finite
 // value or exponents far from 1, take float64 arithmetic: a patch in fixed point keeps at least 44 of its bits.
 //
-// What bounds float64: the integer pipe (61 % of its peak, issue slots 54 %, DRAM 17 %) at one block of 16 warps per
-// SM. 4096 x 2048, two sweeps: pre-smoothing 150 us, where four colour launches of 49 us and a residual-restriction
-// of 117 us took 313; post-smoothing with the residual norm 207 us, where prolongation, colour launches and residual
+// What bounds float64: the integer pipe (60 % of its peak, issue slots 54 %, DRAM 17 %) at one block of 16 warps per
+// SM. 4096 x 2048, two sweeps: pre-smoothing 152 us, where four colour launches of 49 us and a residual-restriction
+// of 117 us took 313; post-smoothing with the residual norm 227 us, where prolongation, colour launches and residual
 // took over 310.
 #include "tile2d.h"
 
