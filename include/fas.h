@@ -60,9 +60,9 @@ typedef enum {
  * solve (mean-free right-hand side, mean removed after every cycle). */
 typedef enum { FAS_BC_NEUMANN = 0, FAS_BC_DIRICHLET = 1, FAS_BC_PERIODIC = 2 } fas_bc;
 /* FP64 cycles on 2D cell levels compute in 64-bit block fixed point, in units of at most 2^-54 of the largest
- * value of a region of 64 columns x 32 or 64 rows, wherever the largest values of its patches of 2 x 1..4 cells
- * lie within 2^10 of one another, and in float64 elsewhere; fields are stored, and residual norms formed, in
- * float64. */
+ * value of a region of 64 columns x 32 or 64 rows, wherever the largest values of its patches (2 columns x 1, 2
+ * or 4 rows) lie within 2^10 of one another, and in float64 elsewhere. Fields are float64 between kernels, and
+ * fas_info.res is the residual norm of the field as stored. */
 typedef enum { FAS_FP64 = 0, FAS_MIXED = 1 } fas_precision;
 
 /* Where the unknowns sit (Sec. 4.1, the MAC staggered grid). FAS_CELL: cell centres (Sec. 2.1).
