@@ -97,9 +97,11 @@ constexpr int group_blocks(int dim, int64_t cells) { return dim == 2 ? 3 : cells
 constexpr int64_t kLanesMaxCells3D = (int64_t)1 << 16;
 // Smallest 3D level of the column-streaming kernels. A block walks its planes one after the other, and smaller levels
 // have too few blocks and planes: a cycle on a 128^3 grid takes 166 us without them on level 0 and 184 with, 512 x 64 x 64
-// (planes x rows x columns) 167 against 202, 256 x 32 x 512 225 against 240, 512 x 64 x 256 359 against 399; from 2^24 on
-// they win for every shape measured (256^3: 755 us without, 585 with; 1024 x 128 x 128: 754, 668).
+// (planes x rows x columns) 167 against 202, 256 x 32 x 512 225 against 240, 512 x 64 x 256 359 against 399. From 2^24 on
+// they win (256^3: 711 us without, 590 with; 2048 x 256 x 32: 712, 664; 32 x 2048 x 256: 686, 595) but for long columns of
+// at most 64 x 64, whose few regions are mostly halo (4096 x 64 x 64: 723, 840).
 constexpr int64_t kCol3dMinCells = (int64_t)1 << 24;
+constexpr int kCol3dMinWidth = 128;  // of the larger of a plane's axes
 // Largest grid with a per-cell diffusivity whose hierarchy runs the register-tile kernels in float64: they read eight
 // more words per cell (the fractions), and on larger grids the per-operation kernels are faster (a cycle of a solve on
 // 1024^2: 285 us against 288 per operation, 512^2: 123 against 179; but 2048 x 1024: 480 against 453, 2048^2: 843 against
@@ -599,7 +601,8 @@ fas_status build_hier(fas_ctx* c, Hier<T>& H, bool buffers, bool level0_buffers)
       // buffers
       if (p.dim == 3 && p.path == 0 && p.ordering == FAS_ORDER_FORWARD) {
         while (H.ncol < H.switch_level && col3d_supported(H.desc[H.ncol], p.nu1) &&
-               col3d_supported(H.desc[H.ncol], p.nu2) && c->shape[H.ncol].cells() >= kCol3dMinCells)
+               col3d_supported(H.desc[H.ncol], p.nu2) && c->shape[H.ncol].cells() >= kCol3dMinCells &&
+               std::max(c->shape[H.ncol].nx, c->shape[H.ncol].ny) >= kCol3dMinWidth)
           H.ncol++;
         const size_t first = H.owned.size();
         for (int l = 0; l < H.ncol; ++l)
